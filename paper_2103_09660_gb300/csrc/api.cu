@@ -32,6 +32,7 @@ void destroy_graph(hnv_graph* g) {
   cudaStream_t s = g->stream;
   for (auto& lv : g->levels) free_level(&lv, s);
   g->levels.clear();
+  dev_free(g->team_levels, s);
   dev_free(g->partials, s);
   dev_free(g->jacobi_tmp, s);
   dev_free(g->d_err, s);
@@ -127,8 +128,25 @@ int vcycle_impl(hnv_graph* g, const void* z_coarsest, void* z_v_out, void* z_e_o
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   const Level& top = g->levels[L];
   const uint8_t* zc = static_cast<const uint8_t*>(z_coarsest);
-  if (top.n > 0) HNV_CUDA(cudaMemcpyAsync(zv(L), zc, row_bytes * top.n, kind, s));
-  if (top.m > 0)
+  // the levels from the coarsest down that are small enough take one launch
+  int first_big = L;
+  if (on_device && team_enabled(d) && sweeps <= kTeamMaxSweeps && team_fits(top, dtype, d) &&
+      team_ready(g, s))
+    while (first_big >= 0 && team_fits(g->levels[first_big], dtype, d)) --first_big;
+  if (first_big < L) {
+    const int b = first_big + 1;
+    TeamGraph t;
+    t.top = L;
+    t.bottom = b;
+    t.zc = reinterpret_cast<const uint4*>(zc);
+    t.zv0 = reinterpret_cast<uint4*>(zv(b));
+    t.ze0 = reinterpret_cast<uint4*>(ze(b));
+    t.buf[0] = reinterpret_cast<uint4*>(buf[0]);
+    t.buf[1] = reinterpret_cast<uint4*>(buf[1]);
+    t.ckpt = reinterpret_cast<uint4*>(ckpt);
+    HNV_CHECK(team_run(g, t, dtype, d, omega, sweeps, mode, s));
+  } else if (top.n > 0) HNV_CUDA(cudaMemcpyAsync(zv(L), zc, row_bytes * top.n, kind, s));
+  if (first_big == L && top.m > 0)
     HNV_CUDA(cudaMemcpyAsync(ze(L), zc + (size_t)top.n * row_bytes, row_bytes * top.m, kind, s));
   std::vector<size_t> off(L + 2, 0);
   for (int l = 0; l <= L; ++l)
@@ -144,9 +162,11 @@ int vcycle_impl(hnv_graph* g, const void* z_coarsest, void* z_v_out, void* z_e_o
                                cudaMemcpyDeviceToDevice, s));
     return HNV_OK;
   };
-  HNV_CHECK(save(L));
-  HNV_CHECK(refine_level(g, L, zv(L), ze(L), dtype, d, omega, sweeps, mode, s));
-  for (int l = L - 1; l >= 0; --l) {
+  if (first_big == L) {
+    HNV_CHECK(save(L));
+    HNV_CHECK(refine_level(g, L, zv(L), ze(L), dtype, d, omega, sweeps, mode, s));
+  }
+  for (int l = std::min(first_big, L - 1); l >= 0; --l) {
     HNV_CHECK(project_level(g, l, zv(l + 1), ze(l + 1), zv(l), ze(l), dtype, d, s));
     HNV_CHECK(save(l));
     HNV_CHECK(refine_level(g, l, zv(l), ze(l), dtype, d, omega, sweeps, mode, s));
@@ -202,7 +222,7 @@ int hnv_build_incidence(int32_t n_nodes, int32_t n_edges, const int64_t* edge_pt
       break;
     }
     if ((rc = dev_alloc((void**)&g->d_err, sizeof(int32_t), s)) != HNV_OK) break;
-    if ((rc = dev_alloc((void**)&g->d_buf, 64 * sizeof(int32_t), s)) != HNV_OK) break;
+    if ((rc = dev_alloc((void**)&g->d_buf, (kBufWords + kTeamWords) * sizeof(int32_t), s)) != HNV_OK) break;
     {
       cudaError_t e = cudaEventCreateWithFlags(&g->fork_ev, cudaEventDisableTiming);
       for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
@@ -284,6 +304,8 @@ int hnv_coarsen(hnv_graph* g, const hnv_coarsen_params* p, int32_t* n_levels) {
     g->levels.pop_back();
   }
   drop_maps(&g->levels[0], s);
+  dev_free(g->team_levels, s);   // describes the old hierarchy
+  g->team_levels = nullptr;
   const int32_t m0 = g->levels[0].m;
   {
     PhaseScope ps(HNV_PHASE_COARSEN, s, 0.0);

@@ -18,6 +18,11 @@
 // every item of the half-sweep (warps take tasks from a counter; see
 // batched_persistent_kernel). Both are followed by the split-row reduction.
 //
+// Graphs whose levels are all small (team_fits) take neither: with the
+// per-class setting they are dealt over teams of blocks that run a graph's
+// whole V-cycle each, in one launch (team.cu), and only the other graphs are
+// lined up by level.
+//
 // Autotuner: the row-class boundaries (PlanShape) and the lanes per row of
 // the short classes of the per-class kernel, and the persistent kernel, are
 // timed on a whole V-cycle of the batch with one sweep per level (the coarse
@@ -248,7 +253,7 @@ batched_finalize_kernel(const int4* __restrict__ long_desc, const int32_t* __res
     return;
   }
   dev::finalize_huge<T>(ds, reinterpret_cast<float*>(sm4), sd.partials, sd.inv_norm, sd.self_in,
-                        sd.out, dv, keep, scale);
+                        sd.out, dv, keep, scale, kFinThreads / dv);
 }
 
 // index of the segment of `prefix` (n+1 ascending offsets) holding i
@@ -342,9 +347,12 @@ struct hnv_batch {
   // side streams: a half-sweep's row classes run concurrently (see enqueue_half)
   cudaStream_t aux[2] = {nullptr, nullptr};
   cudaEvent_t fork_ev = nullptr;
+  cudaEvent_t used_ev = nullptr;   // after the last V-cycle (what it used is freed after it)
+  bool used = false;
   cudaEvent_t join_ev[2] = {nullptr, nullptr};
   std::vector<int> top;            // coarsest level of each graph
-  int Lmax = 0;
+  std::vector<int> step_top;       // the same, -1 for a graph the teams run
+  int Lmax = 0, step_lmax = -1;    // deepest level of all graphs, of the step lists
   PlanShape shape;
   int lanes[3] = {0, 0, 0};        // lanes per row of classes A, B, rest (0: default)
   // per-graph plans for `shape`: plans[side][graph][level]
@@ -361,6 +369,10 @@ struct hnv_batch {
   const void* built_zc = nullptr;
   const void* built_zv = nullptr;
   const void* built_ze = nullptr;
+  int built_kernel = -1;
+  // the teams' graphs (device, in team order) and barrier words
+  TeamArgs team;
+  int teams = 0;
   // captured V-cycle
   cudaGraphExec_t exec = nullptr;
   float exec_omega = -1.f;
@@ -398,11 +410,12 @@ int alloc_into(std::vector<void*>& owned, void** p, size_t bytes, cudaStream_t s
 // both sum every row in the same order; elsewhere it uses its tuned shape.
 int build_plans(hnv_batch* b, size_t row_bytes, cudaStream_t s, int only_level = -1) {
   BTRACE("build_plans row_bytes=%zu only_level=%d", row_bytes, only_level);
+  if (b->used) cudaStreamWaitEvent(s, b->used_ev, 0);
   free_list(b->plan_owned, s);
   for (int side = 0; side < 2; ++side) b->plans[side].assign(b->graphs.size(), {});
   for (size_t i = 0; i < b->graphs.size(); ++i) {
     hnv_graph* g = b->graphs[i];
-    const int L = (int)g->levels.size();
+    const int L = b->step_top[i] + 1;   // none for a team's graph
     for (int side = 0; side < 2; ++side) b->plans[side][i].assign(L, SplitPlan());
     for (int l = 0; l < L; ++l) {
       if (only_level >= 0 && l != only_level) continue;
@@ -428,12 +441,117 @@ int build_plans(hnv_batch* b, size_t row_bytes, cudaStream_t s, int only_level =
   return HNV_OK;
 }
 
+// Which graphs the teams run: every level small, and the per-class setting.
+// Returns whether that changed (plans and steps are then stale).
+bool choose_teams(hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
+  std::vector<int> top = b->top;
+  if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && team_enabled(d) && sweeps <= kTeamMaxSweeps)
+    for (size_t i = 0; i < b->graphs.size(); ++i) {
+      bool fits = true;
+      for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
+      if (fits && team_ready(b->graphs[i], s)) top[i] = -1;
+    }
+  if (top == b->step_top) return false;
+  b->step_top = top;
+  b->step_lmax = -1;
+  for (int t : top) b->step_lmax = std::max(b->step_lmax, t);
+  return true;
+}
+
+// Deals the teams' graphs (longest first, each to the team with the least
+// work so far) over the number of teams with the shortest longest team, and
+// uploads their descriptors. Row buffers and partials belong to a team, so
+// that its next graph finds them in L2.
+int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, uint8_t* ze0,
+                cudaStream_t s) {
+  const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
+  std::vector<int> own;
+  for (size_t i = 0; i < b->graphs.size(); ++i)
+    if (b->step_top[i] < 0) own.push_back((int)i);
+  b->teams = 0;
+  if (own.empty()) return HNV_OK;
+  const int sms = num_sms();
+  std::vector<std::vector<int>> best;
+  double best_us = -1.0;
+  int best_blocks = 1;
+  for (int blocks = sms; blocks >= 1; blocks /= 2) {
+    const int teams = std::min<int>(sms / blocks, (int)own.size());
+    std::vector<std::pair<double, int>> cost;
+    for (int i : own) {
+      double us = 0.0;
+      for (const Level& lv : b->graphs[i]->levels) us += team_sweep_us(lv, dt, d, blocks);
+      cost.push_back({us, i});
+    }
+    std::sort(cost.begin(), cost.end(), [](const std::pair<double, int>& x, const std::pair<double, int>& y) {
+      return x.first != y.first ? x.first > y.first : x.second < y.second;
+    });
+    std::vector<std::vector<int>> deal(teams);
+    std::vector<double> load(teams, 0.0);
+    for (const auto& c : cost) {
+      const int t = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      deal[t].push_back(c.second);
+      load[t] += c.first;
+    }
+    const double us = *std::max_element(load.begin(), load.end());
+    if (best_us < 0.0 || us < best_us) {
+      best_us = us;
+      best = deal;
+      best_blocks = blocks;
+    }
+    if (teams == (int)own.size()) break;
+  }
+  const int teams = (int)best.size();
+  std::vector<TeamGraph> hg;
+  std::vector<int32_t> first{0};
+  for (const std::vector<int>& list : best) {
+    size_t rows = 0;
+    int64_t chunks = 1;
+    for (int i : list)
+      for (size_t l = 0; l < b->graphs[i]->levels.size(); ++l) {
+        const Level& lv = b->graphs[i]->levels[l];
+        if (l > 0) rows = std::max(rows, (size_t)lv.n + lv.m);
+        chunks = std::max<int64_t>(chunks, std::max(lv.planE.n_chunks, lv.planV.n_chunks));
+      }
+    TeamGraph t;
+    for (int k = 0; k < 2 && rows > 0; ++k)
+      HNV_CHECK(alloc_into(b->step_owned, (void**)&t.buf[k], rows * rb, s));
+    HNV_CHECK(alloc_into(b->step_owned, (void**)&t.partials, sizeof(float) * (size_t)chunks * d, s));
+    for (int i : list) {
+      const hnv_graph* g = b->graphs[i];
+      t.levels = g->team_levels;
+      t.top = b->top[i];
+      t.zc = (const uint4*)(zc + (size_t)b->coarse_off[i] * rb);
+      t.zv0 = (uint4*)(zv0 + (size_t)b->v_off[i] * rb);
+      t.ze0 = (uint4*)(ze0 + (size_t)b->e_off[i] * rb);
+      t.err = g->d_err;
+      hg.push_back(t);
+    }
+    first.push_back((int32_t)hg.size());
+  }
+  TeamGraph* dg = nullptr;
+  int32_t* df = nullptr;
+  b->team = TeamArgs();
+  HNV_CHECK(alloc_into(b->step_owned, (void**)&dg, sizeof(TeamGraph) * hg.size(), s));
+  HNV_CHECK(alloc_into(b->step_owned, (void**)&df, sizeof(int32_t) * first.size(), s));
+  HNV_CHECK(alloc_into(b->step_owned, (void**)&b->team.barriers, sizeof(uint32_t) * 32 * teams, s));
+  HNV_CUDA(cudaMemcpyAsync(dg, hg.data(), sizeof(TeamGraph) * hg.size(), cudaMemcpyHostToDevice, s));
+  HNV_CUDA(cudaMemcpyAsync(df, first.data(), sizeof(int32_t) * first.size(), cudaMemcpyHostToDevice, s));
+  HNV_CUDA(cudaStreamSynchronize(s));   // the host vectors die here
+  b->team.graphs = dg;
+  b->team.team_first = df;
+  b->team.blocks = best_blocks;
+  b->teams = teams;
+  return HNV_OK;
+}
+
 void free_steps(hnv_batch* b, cudaStream_t s) {
+  if (b->used) cudaStreamWaitEvent(s, b->used_ev, 0);
   free_list(b->step_owned, s);
   b->steps.clear();
   b->partials = nullptr;
   b->arena[0] = b->arena[1] = nullptr;
   b->built_dt = b->built_d = -1;
+  b->teams = 0;
   if (b->exec) {
     cudaGraphExecDestroy(b->exec);
     b->exec = nullptr;
@@ -445,18 +563,18 @@ void free_steps(hnv_batch* b, cudaStream_t s) {
 // times step 0).
 int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, uint8_t* ze0,
                 cudaStream_t s, int only_step = -1) {
-  BTRACE("build_steps dt=%d d=%d only_step=%d Lmax=%d", dt, d, only_step, b->Lmax);
+  BTRACE("build_steps dt=%d d=%d only_step=%d Lmax=%d", dt, d, only_step, b->step_lmax);
   free_steps(b, s);
   const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
   const int32_t dv = (int32_t)(rb / 16);
   const size_t G = b->graphs.size();
-  b->steps.assign(b->Lmax + 1, BStep());
+  b->steps.assign(b->step_lmax + 1, BStep());
   // arenas for levels >= 1 (parity of the level)
   size_t arena_rows = 0;
-  for (int st = 1; st <= b->Lmax; ++st) {
+  for (int st = 1; st <= b->step_lmax; ++st) {
     size_t rows = 0;
     for (size_t i = 0; i < G; ++i)
-      if (b->top[i] >= st) rows += (size_t)b->graphs[i]->levels[st].n + b->graphs[i]->levels[st].m;
+      if (b->step_top[i] >= st) rows += (size_t)b->graphs[i]->levels[st].n + b->graphs[i]->levels[st].m;
     arena_rows = std::max(arena_rows, rows);
   }
   if (arena_rows > 0 && only_step != 0) {
@@ -464,12 +582,12 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
     HNV_CHECK(alloc_into(b->step_owned, (void**)&b->arena[1], arena_rows * rb, s));
   }
   // row pointers of graph i at level st
-  std::vector<std::vector<uint8_t*>> zvp(b->Lmax + 1, std::vector<uint8_t*>(G, nullptr));
+  std::vector<std::vector<uint8_t*>> zvp(b->step_lmax + 1, std::vector<uint8_t*>(G, nullptr));
   std::vector<std::vector<uint8_t*>> zep = zvp;
-  for (int st = 0; st <= b->Lmax; ++st) {
+  for (int st = 0; st <= b->step_lmax; ++st) {
     size_t off = 0;
     for (size_t i = 0; i < G; ++i) {
-      if (b->top[i] < st) continue;
+      if (b->step_top[i] < st) continue;
       const Level& lv = b->graphs[i]->levels[st];
       if (st == 0) {
         zvp[st][i] = zv0 + (size_t)b->v_off[i] * rb;
@@ -483,16 +601,16 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
   }
   // partials: the largest step-side total
   size_t max_chunks = 1;
-  for (int st = 0; st <= b->Lmax; ++st)
+  for (int st = 0; st <= b->step_lmax; ++st)
     for (int side = 0; side < 2; ++side) {
       size_t c = 0;
       for (size_t i = 0; i < G; ++i)
-        if (b->top[i] >= st) c += b->plans[side][i][st].n_chunks;
+        if (b->step_top[i] >= st) c += b->plans[side][i][st].n_chunks;
       max_chunks = std::max(max_chunks, c);
     }
   HNV_CHECK(alloc_into(b->step_owned, (void**)&b->partials, max_chunks * sizeof(float) * d, s));
 
-  for (int st = 0; st <= b->Lmax; ++st) {
+  for (int st = 0; st <= b->step_lmax; ++st) {
     if (only_step >= 0 && st != only_step) continue;
     BStep& S = b->steps[st];
     for (int side = 0; side < 2; ++side) {
@@ -502,7 +620,7 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       B.n_graphs = (int32_t)G;
       int64_t n_items = 0, n_long = 0, chunk_base = 0;
       for (size_t i = 0; i < G; ++i) {
-        if (b->top[i] < st) continue;
+        if (b->step_top[i] < st) continue;
         const Level& lv = b->graphs[i]->levels[st];
         const SplitPlan& p = b->plans[side][i][st];
         GraphSide& gs = hs[i];
@@ -544,7 +662,7 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       for (int cls = 0; cls < 3; ++cls) {
         int64_t cls_count = 0;
         for (size_t i = 0; i < G; ++i) {
-          if (b->top[i] < st) continue;
+          if (b->step_top[i] < st) continue;
           const SplitPlan& p = b->plans[side][i][st];
           int64_t first = 0, count = 0;
           if (cls == 0) { first = 0; count = p.n_a; }
@@ -563,7 +681,7 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       for (int part = 0; part < 2; ++part) {   // rows with few chunks first, then the rest
         int64_t cnt_part = 0;
         for (size_t i = 0; i < G; ++i) {
-          if (b->top[i] < st) continue;
+          if (b->step_top[i] < st) continue;
           const SplitPlan& p = b->plans[side][i][st];
           const int64_t first = part == 0 ? 0 : p.n_mid;
           const int64_t count = part == 0 ? p.n_mid : p.n_huge;
@@ -594,9 +712,9 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
     std::vector<CopyDesc> cd;
     std::vector<int64_t> cpre{0};
     for (size_t i = 0; i < G; ++i) {
-      if (b->top[i] < st) continue;
+      if (b->step_top[i] < st) continue;
       const Level& lv = b->graphs[i]->levels[st];
-      if (b->top[i] > st) {
+      if (b->step_top[i] > st) {
         pd.push_back(ProjDesc{lv.rep_v, lv.rep_e, lv.n, lv.m, (const uint4*)zvp[st + 1][i],
                               (const uint4*)zep[st + 1][i], (uint4*)zvp[st][i],
                               (uint4*)zep[st][i]});
@@ -633,8 +751,10 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
     }
     HNV_CUDA(cudaStreamSynchronize(s));
   }
+  if (only_step < 0) HNV_CHECK(build_teams(b, dt, d, zc, zv0, ze0, s));
   b->built_dt = dt;
   b->built_d = d;
+  b->built_kernel = b->kernel;
   return HNV_OK;
 }
 
@@ -808,7 +928,15 @@ int enqueue_vcycle(const hnv_batch* b, int d, float omega, int sweeps, cudaStrea
     if (need > b->counters_n) HNV_FAIL(HNV_ERR_STATE, "persistent counters not allocated");
     if (need > 0) HNV_CUDA(cudaMemsetAsync(counter, 0, sizeof(int32_t) * (size_t)need, s));
   }
-  for (int st = b->Lmax; st >= 0; --st) {
+  if (b->teams > 0) {
+    HNV_CUDA(cudaMemsetAsync(b->team.barriers, 0, sizeof(uint32_t) * 32 * b->teams, s));
+    TeamArgs a = b->team;
+    a.sweeps = sweeps;
+    a.keep = 1.0f - omega;
+    a.omega = omega;
+    HNV_CHECK(team_launch(a, b->teams, sizeof(T) == 2 ? HNV_BF16 : HNV_F32, d, s));
+  }
+  for (int st = b->step_lmax; st >= 0; --st) {
     const BStep& S = b->steps[st];
     BTRACE("enqueue step %d copies %d proj %d", st, S.n_copies, S.n_proj);
     if (S.n_copies) {
@@ -915,6 +1043,7 @@ int hnv_batch_create(hnv_graph* const* graphs, int32_t count, hnv_batch** out) {
   b->graphs.assign(graphs, graphs + count);
   for (int32_t i = 0; i < count; ++i) b->generation.push_back(graphs[i]->generation);
   b->device = dev0;
+  b->step_top.assign(count, -2);   // not dealt yet
   b->coarse_off.assign(count + 1, 0);
   b->v_off.assign(count + 1, 0);
   b->e_off.assign(count + 1, 0);
@@ -932,6 +1061,7 @@ int hnv_batch_create(hnv_graph* const* graphs, int32_t count, hnv_batch** out) {
   cudaSetDevice(dev0);
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->used_ev, cudaEventDisableTiming);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
     e = cudaStreamCreateWithFlags(&b->aux[i], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join_ev[i], cudaEventDisableTiming);
@@ -1001,10 +1131,11 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       // per row and the kernel only change the launches
       b->shape = shapes[si];
       std::fill(b->lanes, b->lanes + 3, 0);
+      b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
+      choose_teams(b, dt, d, 1, s);
       rc = build_plans(b, rb, s);
       if (rc == HNV_OK)
         rc = build_steps(b, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
-      b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
       const int cand_a[3] = {2, 4, 8}, cand_b[3] = {4, 8, 16};
       for (int ia = 0; ia < 3 && rc == HNV_OK; ++ia)
         for (int ib = 0; ib < 3 && rc == HNV_OK; ++ib) {
@@ -1024,7 +1155,12 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       if (si == 0 && rc == HNV_OK) {
         std::fill(b->lanes, b->lanes + 3, 0);
         b->kernel = HNV_BATCH_KERNEL_PERSISTENT;
-        rc = time_vcycle1(b, dt, d, omega, s, &persistent_ms);
+        if (choose_teams(b, dt, d, 1, s)) {
+          rc = build_plans(b, rb, s);
+          if (rc == HNV_OK)
+            rc = build_steps(b, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
+        }
+        if (rc == HNV_OK) rc = time_vcycle1(b, dt, d, omega, s, &persistent_ms);
         if (rc == HNV_OK && (best_ms < 0.f || persistent_ms < best_ms)) {
           best_ms = persistent_ms;
           best_shape = shapes[si];
@@ -1088,12 +1224,13 @@ int hnv_batch_vcycle(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* 
   int rc = HNV_OK;
   do {
     const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
-    if (!b->plans_ready || b->plans_row_bytes != rb) {
+    const bool dealt = choose_teams(b, (int)dt, d, sweeps_per_level, cs);
+    if (dealt || !b->plans_ready || b->plans_row_bytes != rb) {
       if ((rc = build_plans(b, rb, cs)) != HNV_OK) break;
       free_steps(b, cs);
     }
     if (b->built_dt != (int)dt || b->built_d != d || b->built_zc != z_coarsest ||
-        b->built_zv != z_v_out || b->built_ze != z_e_out || b->steps.empty()) {
+        b->built_zv != z_v_out || b->built_ze != z_e_out || b->built_kernel != b->kernel) {
       if ((rc = build_steps(b, dt, d, (const uint8_t*)z_coarsest, (uint8_t*)z_v_out,
                             (uint8_t*)z_e_out, cs)) != HNV_OK)
         break;
@@ -1147,6 +1284,12 @@ int hnv_batch_vcycle(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* 
     if (e != cudaSuccess) rc = cuda_status(e, "cudaGraphLaunch");
     else note_launches(b->exec_kernels);
   } while (0);
+  if (rc == HNV_OK) {
+    // (an event recorded under capture cannot order later work)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+      b->used = cudaEventRecord(b->used_ev, s) == cudaSuccess;
+  }
   if (prev >= 0) cudaSetDevice(prev);
   return rc;
 }
@@ -1182,6 +1325,7 @@ void hnv_batch_free(hnv_batch* b) {
     if (b->join_ev[i]) cudaEventDestroy(b->join_ev[i]);
   }
   if (b->fork_ev) cudaEventDestroy(b->fork_ev);
+  if (b->used_ev) cudaEventDestroy(b->used_ev);
   if (prev >= 0) cudaSetDevice(prev);
   delete b;
 }

@@ -39,6 +39,26 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
                        float omega, int max_sweeps, float eps, int mode, int32_t* sweeps_done,
                        float* last_delta, cudaStream_t s) {
   const Level& lv = g->levels[level];
+  if (max_sweeps > 0 && team_enabled(d) && team_fits(lv, dtype, d) && team_ready(g, s)) {
+    // sweeps, changes and the test in one launch (at most kTeamMaxSweeps each)
+    int32_t done = 0, res[2] = {0, 0};
+    float delta = 0.f;
+    do {
+      TeamGraph t;
+      t.top = t.bottom = level;
+      t.zv0 = static_cast<uint4*>(z_v);
+      t.ze0 = static_cast<uint4*>(z_e);
+      const int k = max_sweeps - done < kTeamMaxSweeps ? max_sweeps - done : kTeamMaxSweeps;
+      HNV_CHECK(team_run(g, t, dtype, d, omega, k, mode, s, &eps));
+      HNV_CHECK(read_ints(g, g->d_buf + kTeamResult, 2, res, s));
+      if (res[0] <= 0) HNV_FAIL(HNV_ERR_TIMEOUT, "a bounded wait of a refinement kernel gave up");
+      done += res[0];
+      std::memcpy(&delta, &res[1], sizeof(float));
+    } while (done < max_sweeps && !(delta <= eps));
+    *sweeps_done = done;
+    *last_delta = delta;
+    return HNV_OK;
+  }
   const size_t rb = (dtype == HNV_BF16 ? 2 : 4) * (size_t)d;
   const int64_t vec_v = (int64_t)lv.n * (int64_t)(rb / 16), vec_e = (int64_t)lv.m * (int64_t)(rb / 16);
   TempPool pool(s);

@@ -239,6 +239,7 @@ struct SplitPlan {
   int32_t n_a = 0, n_b = 0, n_c = 0, n_d = 0;  // rows per class
   int32_t n_chunks = 0;                        // chunk items (after the D rows)
   int32_t n_mid = 0, n_huge = 0;               // split rows by chunk count
+  int32_t n_mid_chunks = 0;                    // chunk items of the n_mid rows (they come first)
   int32_t n_zero = 0;
   int4* items = nullptr;              // [n_a + n_b + n_c + n_d + n_chunks]
   int4* long_desc = nullptr;          // [n_mid + n_huge]
@@ -285,6 +286,12 @@ struct Level {
   std::vector<void*> panel_owned[2];
 };
 
+struct TeamLevel;
+// 32-bit words of hnv_graph::d_buf: 64 of scratch, then the team kernel's
+// barrier line, the stopping rule's 3 running maxima and its 2 results.
+constexpr int kBufWords = 64, kTeamBarrier = 64, kTeamDelta = 96, kTeamResult = 100,
+              kTeamWords = 64;
+
 }  // namespace hnv
 
 struct hnv_graph {
@@ -293,7 +300,8 @@ struct hnv_graph {
   std::vector<hnv::Level> levels;
   int32_t* d_err = nullptr;      // device error word
   int32_t* h_buf = nullptr;      // pinned host scratch (64 ints)
-  int32_t* d_buf = nullptr;      // device scratch (64 ints)
+  int32_t* d_buf = nullptr;      // device scratch (64 ints), then the team kernel's (kTeamWords)
+  hnv::TeamLevel* team_levels = nullptr;   // device, one per level (team.cu)
   float* partials = nullptr;     // split-row partial sums
   size_t partials_bytes = 0;
   float* jacobi_tmp = nullptr;   // Jacobi: next hyperedge rows
@@ -385,6 +393,86 @@ int gather_rows_f32(const SplitPlan& plan, const int32_t* idx, const float* wgt,
                     const float* norm, const float* src, const float* self_in, float* out, int d,
                     float keep, float scale, float* partials, cudaStream_t s,
                     const hnv_graph* conc = nullptr);
+
+// team.cu: whole V-cycles or sweeps of small graphs in one cooperative launch.
+// One side of a level for the team kernel: its regular plan (rows of 1-16
+// incidences first) and arrays.
+struct TeamSide {
+  const int4* items = nullptr;
+  const int4* long_desc = nullptr;
+  const int32_t* idx = nullptr;
+  const float* inc_w = nullptr;
+  const float* inv_norm = nullptr;
+  // items [0, n_a): rows of 1-4 incidences; [n_a, n_short): of 5-16; [n_short, n_rows): longer
+  // whole rows; [n_rows, n_items): chunks, the n_mid rows' n_mid_chunks first
+  int32_t n_a = 0, n_short = 0, n_rows = 0, n_items = 0, n_mid = 0, n_huge = 0, n_mid_chunks = 0;
+};
+
+struct TeamLevel {
+  TeamSide side[2];               // 0 hyperedge rows, 1 node rows
+  const int32_t* rep_v = nullptr;
+  const int32_t* rep_e = nullptr;
+  int32_t n = 0, m = 0;
+  int64_t row0 = 0;               // rows of the finer levels (checkpoint offset)
+};
+
+// Levels top .. bottom of one graph: the rows start from zc (null: they are
+// in place), level `bottom` is refined in zv0 / ze0, a level l above it in
+// buf[l & 1] (node rows, then hyperedge rows).
+struct TeamGraph {
+  const TeamLevel* levels = nullptr;   // device
+  int32_t top = 0, bottom = 0;
+  const uint4* zc = nullptr;
+  uint4* zv0 = nullptr;
+  uint4* ze0 = nullptr;
+  uint4* buf[2] = {nullptr, nullptr};
+  float* partials = nullptr;
+  uint4* jtmp = nullptr;               // Jacobi: m rows of the largest level
+  uint4* ckpt = nullptr;               // every level's starting rows, or null
+  int32_t* err = nullptr;              // the graph's error word
+};
+
+struct TeamArgs {
+  TeamGraph one;                       // with graphs == null: one graph, one team
+  const TeamGraph* graphs = nullptr;   // device: graphs of team t are
+  const int32_t* team_first = nullptr; //   [team_first[t], team_first[t + 1])
+  int32_t blocks = 1;                  // blocks per team
+  int32_t dv = 0, sweeps = 0, jacobi = 0;
+  float keep = 0.f, omega = 0.f;
+  uint32_t* barriers = nullptr;        // 32 words per team, zeroed before the launch
+  // stopping rule (result != null): delta holds 3 words, zeroed before the
+  // launch; result receives {sweeps done, bits of the last largest change}
+  unsigned* delta = nullptr;
+  int32_t* result = nullptr;
+  float eps = 0.f;
+};
+
+// Levels the team kernel takes: rows of at most 64 vectors, and so little
+// work per half-sweep that launches, not bandwidth, would set its time.
+constexpr int64_t kTeamMaxRowBytes = 1024;
+constexpr int64_t kTeamMaxGather = 192000000;   // bytes gathered per half-sweep
+constexpr int64_t kTeamMaxRows = 96000000;      // bytes of both row tables
+constexpr int kTeamMaxSweeps = 512;             // of one launch
+bool team_fits(const Level& lv, int dtype, int d);
+void team_level(const Level& lv, int64_t row0, TeamLevel* out);
+// Blocks that the items of one level's larger side fill.
+int team_blocks_for(const Level& lv, int dtype, int d);
+// Estimated microseconds of one sweep of a level by a team of `blocks`.
+double team_sweep_us(const Level& lv, int dtype, int d, int blocks);
+int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s);
+// The team path applies at all (it is off while phases are timed, and where
+// an environment switch asks for another gather).
+bool team_enabled(int d);
+// Levels top .. bottom of g (all of which fit) in one launch on s.
+// With eps, the stopping rule: the sweeps done and the last change are left
+// in d_buf + kTeamResult.
+int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
+             cudaStream_t s, const float* eps = nullptr);
+// Uploads the hierarchy's TeamLevels on first use (dropped with the
+// hierarchy). False where it cannot: under capture, or out of memory; the
+// caller then takes the per-launch path.
+bool team_ready(hnv_graph* g, cudaStream_t s);
+int forced_panels();   // HNV_PANELS, or -1
 
 // Two-phase sweeps whose split-row partial sums go to caller-provided
 // scratch (at least max(planE.n_chunks, planV.n_chunks) * d floats); no

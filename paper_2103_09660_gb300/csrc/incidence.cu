@@ -343,7 +343,14 @@ int build_split_plan(hnv_graph* g, std::vector<void*>* owned, const int32_t* ptr
     HNV_CHECK(launch("long_chunk_counts", long_chunk_counts, grid_for(n_long, 256), 256, 0, s,
                      (const uint64_t*)sorted, off[5], n_long, ptr, T, chunk_off));
     HNV_CHECK(exclusive_scan_i32(chunk_off, chunk_off, n_long, cnt + 8, s));
-    HNV_CHECK(read_ints(g, cnt + 8, 1, &plan->n_chunks, s));
+    // the offset of the first row with many chunks = chunks of those before it
+    if (c[5] > 0 && c[6] > 0)
+      HNV_CUDA(cudaMemcpyAsync(cnt + 9, chunk_off + c[5], sizeof(int32_t),
+                               cudaMemcpyDeviceToDevice, s));
+    int32_t ch[2];
+    HNV_CHECK(read_ints(g, cnt + 8, 2, ch, s));
+    plan->n_chunks = ch[0];
+    plan->n_mid_chunks = c[6] == 0 ? ch[0] : (c[5] > 0 ? ch[1] : 0);
   }
   const int64_t n_items = (int64_t)n_rows_items + plan->n_chunks;
   if (n_items > 0)
@@ -492,12 +499,8 @@ __global__ void panel_fill(int32_t R, const int32_t* __restrict__ list,
   }
 }
 
-// Panels worth cutting the long rows of `base` into, for a neighbour table
-// of table_bytes: panels of about 64 MB (half of L2) so that a panel's rows
-// stay in L2 while every row piece gathering from it runs, but no more than
-// keep pieces at 32 incidences on average (each piece writes and reads one
-// partial row), and none at all if the table mostly fits L2 or the panels
-// would be larger than L2.
+}  // namespace
+
 int forced_panels() {
   static int forced = -2;
   if (forced == -2) {
@@ -507,6 +510,14 @@ int forced_panels() {
   return forced;
 }
 
+namespace {
+
+// Panels worth cutting the long rows of `base` into, for a neighbour table
+// of table_bytes: panels of about 64 MB (half of L2) so that a panel's rows
+// stay in L2 while every row piece gathering from it runs, but no more than
+// keep pieces at 32 incidences on average (each piece writes and reads one
+// partial row), and none at all if the table mostly fits L2 or the panels
+// would be larger than L2.
 constexpr int64_t kPanelMinTable = 96000000;   // below: the table mostly stays in L2
 
 int choose_panels(int64_t table_bytes, int64_t long_rows, int64_t long_nnz) {

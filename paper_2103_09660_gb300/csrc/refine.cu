@@ -22,6 +22,7 @@
 // the relaxation.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdlib>
 
 #include "refine_device.cuh"
@@ -174,7 +175,7 @@ finalize_kernel(const int4* __restrict__ long_desc, int32_t n_mid, int32_t n_hug
   const int32_t k = n_mid + (int32_t)blockIdx.x - mid_blocks;
   if (k >= n_mid + n_huge) return;
   dev::finalize_huge<T>(long_desc[k], reinterpret_cast<float*>(sm4), partials, inv_norm, self_in,
-                        out, dv, keep, scale);
+                        out, dv, keep, scale, kFinThreads / dv);
 }
 
 // Out-of-place sweeps (Jacobi): rows without neighbours carry over.
@@ -471,10 +472,81 @@ int ensure_scratch(float** p, size_t* have, size_t need, cudaStream_t s) {
 
 }  // namespace
 
+bool team_enabled(int d) { return !timing_on() && !use_tma(d) && forced_panels() < 1; }
+
+bool team_ready(hnv_graph* g, cudaStream_t s) {
+  if (g->team_levels) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    return false;
+  std::vector<TeamLevel> h(g->levels.size());
+  int64_t row0 = 0;
+  for (size_t l = 0; l < h.size(); ++l) {
+    team_level(g->levels[l], row0, &h[l]);
+    row0 += (int64_t)g->levels[l].n + g->levels[l].m;
+  }
+  TeamLevel* t = nullptr;
+  if (dev_alloc((void**)&t, sizeof(TeamLevel) * h.size(), s) != HNV_OK) {
+    clear_error_detail();
+    return false;
+  }
+  // done before any stream reads it (later calls may come on other streams)
+  if (cudaMemcpyAsync(t, h.data(), sizeof(TeamLevel) * h.size(), cudaMemcpyHostToDevice, s) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess) {
+    dev_free(t, s);
+    return false;
+  }
+  g->team_levels = t;
+  return true;
+}
+
+int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
+             cudaStream_t s, const float* eps) {
+  int64_t chunks = 1, m = 1;
+  int blocks = 1;
+  for (int l = t.bottom; l <= t.top; ++l) {
+    const Level& lv = g->levels[l];
+    chunks = std::max<int64_t>(chunks, std::max(lv.planE.n_chunks, lv.planV.n_chunks));
+    m = std::max<int64_t>(m, lv.m);
+    blocks = std::max(blocks, team_blocks_for(lv, dtype, d));
+  }
+  HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes, sizeof(float) * (size_t)chunks * d, s));
+  if (mode == HNV_SWEEP_JACOBI)
+    HNV_CHECK(ensure_scratch(&g->jacobi_tmp, &g->jacobi_bytes, elem_size(dtype) * (size_t)m * d, s));
+  HNV_CUDA(cudaMemsetAsync(g->d_buf + kBufWords, 0, sizeof(int32_t) * kTeamWords, s));
+  t.levels = g->team_levels;
+  t.err = g->d_err;
+  t.partials = g->partials;
+  t.jtmp = reinterpret_cast<uint4*>(g->jacobi_tmp);
+  TeamArgs a;
+  a.one = t;
+  a.blocks = blocks;
+  a.sweeps = sweeps;
+  a.jacobi = mode == HNV_SWEEP_JACOBI;
+  a.keep = 1.0f - omega;
+  a.omega = omega;
+  a.barriers = reinterpret_cast<uint32_t*>(g->d_buf + kTeamBarrier);
+  if (eps) {
+    a.delta = reinterpret_cast<unsigned*>(g->d_buf + kTeamDelta);
+    a.result = g->d_buf + kTeamResult;
+    a.eps = *eps;
+  }
+  return team_launch(a, 1, dtype, d, s);
+}
+
 int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d, float omega,
                  int sweeps, int mode, cudaStream_t s) {
   NvtxRange nvtx("hnv refine level %d (%d sweeps)", level, sweeps);
   Level& lv = g->levels[level];
+  if (sweeps > 0 && sweeps <= kTeamMaxSweeps && team_enabled(d) && team_fits(lv, dtype, d) &&
+      team_ready(g, s)) {
+    TeamGraph t;
+    t.top = t.bottom = level;
+    t.zv0 = static_cast<uint4*>(z_v);
+    t.ze0 = static_cast<uint4*>(z_e);
+    return team_run(g, t, dtype, d, omega, sweeps, mode, s);
+  }
   const size_t es = elem_size(dtype);
   const SplitPlan* planE = &lv.planE;
   const SplitPlan* planV = &lv.planV;

@@ -1,0 +1,165 @@
+"""Small graphs run whole V-cycles in one cooperative launch (team.cu). Every
+row is summed in the order of the per-launch kernels, so both paths give the
+same bits. Phase timing needs a launch per half-sweep and so selects the
+per-launch path; a graph that is too large for the one-launch path, or a
+capture before its first use, takes it as well."""
+
+import numpy as np
+import pytest
+
+import hypergen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def H():
+    from paper_2103_09660_gb300 import build
+    build.build()
+    import paper_2103_09660_gb300 as mod
+    import torch
+    assert torch.cuda.is_available()
+    return mod
+
+
+def _hub_graph(hub, mids, seed=0):
+    """Node 0 in `hub` hyperedges, nodes 1.. in `mids` each, and hyperedges of
+    4, 5, 16, 17, 64, 65, 128, 129 and 300 members."""
+    rng = np.random.default_rng(seed)
+    n = 700
+    edges = [[0, 20 + i % 600, 21 + i % 600] for i in range(hub)]
+    for v, k in enumerate(mids):
+        edges += [[v + 1, 20 + (7 * i) % 600, 640 + i % 50] for i in range(k)]
+    edges += [rng.choice(n, k, replace=False).tolist() for k in (4, 5, 16, 17, 64, 65, 128, 129, 300)]
+    ptr = np.concatenate([[0], np.cumsum([len(e) for e in edges])]).astype(np.int64)
+    return hypergen.Hypergraph(n=n, m=len(edges), edge_ptr=ptr,
+                               edge_nodes=np.concatenate(edges).astype(np.int32),
+                               weights=rng.uniform(0.5, 2.0, len(edges)).astype(np.float32))
+
+
+def _both(H, f):
+    """f() on the one-launch path and on the per-launch path."""
+    import torch
+    before = H.kernel_launch_count()
+    a = f()
+    torch.cuda.synchronize()
+    one = H.kernel_launch_count() - before
+    H.timing_enable(True)
+    try:
+        before = H.kernel_launch_count()
+        b = f()
+        torch.cuda.synchronize()
+        many = H.kernel_launch_count() - before
+    finally:
+        H.timing_enable(False)
+        H.timing_reset()
+    return a, b, one, many
+
+
+# split rows: none; a few of 2-3 chunks (summed inside a block); many chunks
+# (more than 32, a reduction step); and rows of both kinds
+GRAPHS = [(40, []), (40, [129, 300]), (4200, []), (5000, [129, 300, 4096, 1000])]
+
+
+@pytest.mark.parametrize("hub,mids", GRAPHS)
+@pytest.mark.parametrize("dtname,d", [("f32", 4), ("f32", 36), ("f32", 100), ("f32", 256),
+                                      ("bf16", 8), ("bf16", 72), ("bf16", 512)])
+def test_one_launch_gives_the_same_bits(H, hub, mids, dtname, d):
+    import torch
+    dt = torch.float32 if dtname == "f32" else torch.bfloat16
+    hg = _hub_graph(hub, mids)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    with H.Graph.from_hypergraph(hg) as G:
+        L = G.coarsen(min_nodes=30, max_levels=3)
+        top = G.level_info(L - 1)
+        zc = torch.randn((top[0] + top[1], d), generator=g, device="cuda").to(dt)
+        zv = torch.empty((hg.n, d), dtype=dt, device="cuda")
+        ze = torch.empty((hg.m, d), dtype=dt, device="cuda")
+        z0v = torch.randn((hg.n, d), generator=g, device="cuda").to(dt)
+        z0e = torch.randn((hg.m, d), generator=g, device="cuda").to(dt)
+        for omega in (0.3, 1.0):
+            def vcycle():
+                zv.fill_(float("nan"))
+                ze.fill_(float("nan"))
+                G.vcycle(zc, zv, ze, omega, 3)
+                return zv.clone(), ze.clone()
+            a, b, one, many = _both(H, vcycle)
+            assert one == 1 and many > one
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+            for mode in (H.SWEEP_TWO_PHASE, H.SWEEP_JACOBI):
+                def refine():
+                    v, e = z0v.clone(), z0e.clone()
+                    G.refine(0, v, e, omega, 3, mode)
+                    return v, e
+                a, b, one, many = _both(H, refine)
+                assert one == 1 and many > one
+                assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+                def until():
+                    v, e = z0v.clone(), z0e.clone()
+                    return v, e, G.refine_until(0, v, e, omega, 12, 0.2, mode)
+                a, b, one, many = _both(H, until)
+                assert one == 1 and many > one
+                assert a[2] == b[2]
+                assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+        G.sync_status()
+
+
+def test_more_sweeps_than_one_launch_takes(H):
+    """The stopping rule over several launches; a fixed number of sweeps above
+    the limit takes the per-launch path."""
+    import torch
+    hg = _hub_graph(40, [129])
+    with H.Graph.from_hypergraph(hg) as G:
+        z = torch.randn((hg.n + hg.m, 8), device="cuda")
+
+        def until():
+            v, e = z[:hg.n].clone(), z[hg.n:].clone()
+            return v, e, G.refine_until(0, v, e, 0.001, 1100, -1.0)
+        a, b, one, many = _both(H, until)
+        assert one == 3 and a[2] == b[2] and a[2][0] == 1100
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+        def refine():
+            v, e = z[:hg.n].clone(), z[hg.n:].clone()
+            G.refine(0, v, e, 0.001, 513)
+            return v, e
+        a, b, one, many = _both(H, refine)
+        assert one == many
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+def test_saved_rows_gradients_and_capture(H):
+    """The differentiable V-cycle saves every level's starting rows in the same
+    launch; a captured V-cycle replays it."""
+    import torch
+    hg = _hub_graph(300, [129, 300])
+    d = 32
+    with H.Graph.from_hypergraph(hg) as G:
+        L = G.coarsen(min_nodes=30, max_levels=3)
+        top = G.level_info(L - 1)
+        zc = torch.randn((top[0] + top[1], d), device="cuda")
+        w = torch.rand(hg.m, device="cuda") + 0.5
+
+        def grads():
+            ww, zz = w.clone().requires_grad_(True), zc.clone().requires_grad_(True)
+            v, e = H.vcycle_autograd(G, ww, zz, 0.5, 3)
+            return (v.detach(), e.detach()) + torch.autograd.grad(v.square().sum() + e.sum(), [ww, zz])
+        a, b, one, many = _both(H, grads)
+        assert one < many
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+        zv, ze = torch.empty((hg.n, d), device="cuda"), torch.empty((hg.m, d), device="cuda")
+        G.vcycle(zc, zv, ze, 0.5, 3)
+        want = zv.clone(), ze.clone()
+        graph = torch.cuda.CUDAGraph()
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.graph(graph, stream=s):
+            H.hnv_vcycle(G.handle, zc, zv, ze, 0.5, 3, H.SWEEP_TWO_PHASE, s)
+        zv.zero_()
+        ze.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(zv, want[0]) and torch.equal(ze, want[1])
