@@ -157,33 +157,138 @@ int radix_shifts(int low_bits, int high_bits, int* shifts);
 // Number of bits needed to hold values in [0, count).
 int bits_for_count(int64_t count);
 
-// Visits every entry k of the rows [0, rows) of a CSR with offsets ptr as
-// f(row, k). A warp takes 32 consecutive rows, whose entries are contiguous,
-// and walks them 32 at a time (coalesced, every lane busy whatever the row
-// lengths), finding each entry's row by a binary search over the 32 row
-// starts held one per lane. Launch with one thread per row (any grid).
-template <typename P, typename F>
-__device__ __forceinline__ void csr_rows_warp_visit(int64_t rows, const P* __restrict__ ptr,
-                                                    F f) {
+// Last index i in [0, n) with ptr[i] <= key (ptr ascending, ptr[0] <= key),
+// found by one warp 32 probes at a time.
+template <typename P>
+__device__ __forceinline__ int64_t warp_last_le(const P* __restrict__ ptr, int64_t n, int64_t key) {
   const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t r0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
-       r0 < rows; r0 += warps * 32) {
-    const int64_t last = r0 + 32 < rows ? r0 + 32 : rows;
-    const int64_t mine = r0 + lane < last ? r0 + lane : last;
-    const int64_t start = (int64_t)ptr[mine];  // lanes past the last row hold the end
-    const int64_t first = __shfl_sync(0xffffffffu, start, 0);
-    const int64_t end = (int64_t)ptr[last];
-    for (int64_t base = first; base < end; base += 32) {
-      const int64_t k = base + lane;
-      int j = 0;
+  int64_t lo = 0, hi = n;   // the answer is in [lo, hi)
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 31) / 32;
+    const int64_t at = lo + lane * step;
+    const unsigned le = __ballot_sync(0xffffffffu, at < hi && (int64_t)ptr[at] <= key);
+    const int last = 31 - __clz((int)le);   // lane 0 always holds
+    const int64_t nlo = lo + last * step;
+    hi = nlo + step < hi ? nlo + step : hi;
+    lo = nlo;
+  }
+  return lo;
+}
+
+// Visits every entry k of the rows [0, rows) of a CSR with offsets ptr as
+// f(row, k): a block of kEntryThreads takes kEntryTile consecutive entries,
+// finds the rows they lie in, marks each row's first entry in shared memory
+// and spreads the marks by a running maximum. Every thread has the same work
+// whatever the row lengths, and accesses by k are coalesced. (Rows dealt to
+// warps left one warp on a row of thousands of entries: packing the 17.6M
+// incidences of the 1M-node workload took 283 us.) Launch with one block per
+// tile of the `total` entries; total = ptr[rows].
+constexpr int kEntryThreads = 256;
+constexpr int kEntryTile = 2048;
+inline unsigned entry_grid(int64_t total) {
+  return (unsigned)((total + kEntryTile - 1) / kEntryTile);
+}
+
+template <typename P, typename F>
+__device__ __forceinline__ void csr_entries_visit(int64_t rows, const P* __restrict__ ptr,
+                                                  int64_t total, F f) {
+  constexpr int PER = kEntryTile / kEntryThreads;
+  __shared__ int32_t mark[kEntryTile];
+  __shared__ int32_t wmax[kEntryThreads / 32];
+  __shared__ int64_t bounds[2];
+  const int64_t t0 = (int64_t)blockIdx.x * kEntryTile;
+  const int64_t t1 = t0 + kEntryTile < total ? t0 + kEntryTile : total;
+  if (t0 >= t1) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < 2) {
+    const int64_t r = warp_last_le(ptr, rows, w == 0 ? t0 : t1 - 1);
+    if (lane == 0) bounds[w] = r;
+  }
+  for (int i = threadIdx.x; i < kEntryTile; i += kEntryThreads) mark[i] = 0;
+  __syncthreads();
+  const int64_t r0 = bounds[0], r1 = bounds[1];
+  // (an empty row shares its start with the row after it: the larger wins)
+  for (int64_t r = r0 + 1 + threadIdx.x; r <= r1; r += kEntryThreads)
+    atomicMax(&mark[(int64_t)ptr[r] - t0], (int32_t)(r - r0));
+  __syncthreads();
+  int32_t x[PER], run = 0;
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int64_t sc = __shfl_sync(0xffffffffu, start, j + step);
-        if (sc <= k) j += step;
-      }
-      if (k < end) f(r0 + j, k);
-    }
+  for (int j = 0; j < PER; ++j) {
+    run = max(run, mark[threadIdx.x * PER + j]);
+    x[j] = run;
+  }
+  int32_t inc = run;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc = max(inc, y);
+  }
+  if (lane == 31) wmax[w] = inc;
+  int32_t before = __shfl_up_sync(0xffffffffu, inc, 1);
+  if (lane == 0) before = 0;
+  __syncthreads();
+  for (int q = 0; q < w; ++q) before = max(before, wmax[q]);
+#pragma unroll
+  for (int j = 0; j < PER; ++j) mark[threadIdx.x * PER + j] = max(x[j], before);
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = j * kEntryThreads + threadIdx.x;
+    if (t0 + i < t1) f(r0 + mark[i], t0 + i);
+  }
+}
+
+// Compaction of entries [0, n) chosen by a predicate, in order, without
+// materialised flags: compact_count writes the chosen per tile (and marks
+// nothing), the tile counts are scanned, compact_write recomputes the
+// predicate and calls put(k, position).
+constexpr int kCompactThreads = 256;
+constexpr int kCompactTile = 4096;
+inline int64_t compact_tiles(int64_t n) { return (n + kCompactTile - 1) / kCompactTile; }
+
+template <typename Pred>
+__device__ __forceinline__ void compact_count(int64_t n, int32_t* __restrict__ tile_count, Pred pred) {
+  const int64_t t0 = (int64_t)blockIdx.x * kCompactTile;
+  int32_t c = 0;
+#pragma unroll 4
+  for (int j = 0; j < kCompactTile / kCompactThreads; ++j) {
+    const int64_t k = t0 + j * kCompactThreads + threadIdx.x;
+    if (k < n && pred(k)) ++c;
+  }
+  __shared__ int32_t ws[kCompactThreads / 32];
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = c;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < kCompactThreads / 32; ++q) c += ws[q];
+    tile_count[blockIdx.x] = c;
+  }
+}
+
+template <typename Pred, typename Put>
+__device__ __forceinline__ void compact_write(int64_t n, const int32_t* __restrict__ tile_off,
+                                              Pred pred, Put put) {
+  // a warp takes 512 consecutive entries, 32 at a time: ballots rank them
+  constexpr int ROUNDS = kCompactTile / kCompactThreads;
+  __shared__ int32_t ws[kCompactThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * kCompactTile + (int64_t)w * (32 * ROUNDS) + lane;
+  unsigned bits[ROUNDS];
+  int32_t c = 0;
+#pragma unroll
+  for (int j = 0; j < ROUNDS; ++j) {
+    const int64_t k = base + j * 32;
+    bits[j] = __ballot_sync(0xffffffffu, k < n && pred(k));
+    c += __popc(bits[j]);
+  }
+  if (lane == 0) ws[w] = c;
+  __syncthreads();
+  int32_t at = tile_off[blockIdx.x];
+  for (int q = 0; q < w; ++q) at += ws[q];
+#pragma unroll
+  for (int j = 0; j < ROUNDS; ++j) {
+    if (bits[j] >> lane & 1u) put(base + j * 32, at + __popc(bits[j] & ((1u << lane) - 1u)));
+    at += __popc(bits[j]);
   }
 }
 
@@ -201,6 +306,14 @@ constexpr size_t kSegBitmapBytes = 160 * 1024;
 int segmented_sort_low32(int32_t segs, const int32_t* ptr32, const int64_t* ptr64,
                          int32_t max_len, int64_t total_keys, uint64_t* keys, cudaStream_t s,
                          uint32_t distinct_range = 0);
+
+// The distinct keys of n sorted (row << 32 | col) keys as a CSR, in two
+// steps: unique_count leaves the kept keys' offsets per tile in tiles
+// [compact_tiles(n)] and their number in *total (device); unique_csr writes
+// their cols and row_ptr[row] of every row that has keys.
+int unique_count(const uint64_t* keys, int64_t n, int32_t* tiles, int32_t* total, cudaStream_t s);
+int unique_csr(const uint64_t* keys, int64_t n, const int32_t* tiles, int32_t* cols,
+               int32_t* row_ptr, cudaStream_t s);
 
 int fill_i32(int32_t* p, int32_t value, int64_t n, cudaStream_t s);
 

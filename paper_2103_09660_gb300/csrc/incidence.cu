@@ -48,44 +48,20 @@ __global__ void check_weights_kernel(int32_t m, const float* __restrict__ w,
   }
 }
 
-// key = (e << 32) | node, warp per hyperedge; an out-of-range node sets the
-// error bit and is replaced by 0 so the sort stays in bounds.
-__global__ void pack_input_keys(int32_t m, int32_t n, const int64_t* __restrict__ ptr,
-                                const int32_t* __restrict__ nodes, uint64_t* __restrict__ keys,
-                                int32_t* __restrict__ err) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t e = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < m;
-       e += warps) {
-    const int64_t b = ptr[e], end = ptr[e + 1];
-    for (int64_t k = b + lane; k < end; k += 32) {
-      int32_t v = nodes[k];
-      if (v < 0 || v >= n) {
-        atomicOr(err, ERRBIT_NODE_RANGE);
-        v = 0;
-      }
-      keys[k] = ((uint64_t)(uint32_t)e << 32) | (uint32_t)v;
+// key = (e << 32) | node; an out-of-range node sets the error bit and is
+// replaced by 0 so the sort stays in bounds.
+__global__ void __launch_bounds__(kEntryThreads)
+pack_input_keys(int32_t m, int32_t n, int64_t nnz, const int64_t* __restrict__ ptr,
+                const int32_t* __restrict__ nodes, uint64_t* __restrict__ keys,
+                int32_t* __restrict__ err) {
+  csr_entries_visit(m, ptr, nnz, [&](int64_t e, int64_t k) {
+    int32_t v = nodes[k];
+    if (v < 0 || v >= n) {
+      atomicOr(err, ERRBIT_NODE_RANGE);
+      v = 0;
     }
-  }
-}
-
-__global__ void first_flags(const uint64_t* __restrict__ keys, int64_t n, int32_t* __restrict__ f) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    f[k] = (k == 0 || keys[k] != keys[k - 1]) ? 1 : 0;
-}
-
-// Unique (row, col) keys -> CSR columns + per-row counts.
-__global__ void csr_from_unique(const uint64_t* __restrict__ keys, int64_t n,
-                                const int32_t* __restrict__ first, const int32_t* __restrict__ pos,
-                                int32_t* __restrict__ cols, int32_t* __restrict__ row_cnt) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    if (!first[k]) continue;
-    const uint64_t key = keys[k];
-    cols[pos[k]] = (int32_t)(uint32_t)key;
-    atomicAdd(&row_cnt[(uint32_t)(key >> 32)], 1);
-  }
+    keys[k] = ((uint64_t)(uint32_t)e << 32) | (uint32_t)v;
+  });
 }
 
 __global__ void iota_kernel(int32_t* p, int32_t n) {
@@ -103,13 +79,7 @@ __global__ void inv_size_kernel(int32_t m, const int32_t* __restrict__ e_ptr,
   }
 }
 
-__global__ void csc_weights_kernel(int64_t nnz, const int32_t* __restrict__ v_edges,
-                                   const float* __restrict__ w, float* __restrict__ v_w) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz;
-       k += (int64_t)gridDim.x * blockDim.x)
-    v_w[k] = w[v_edges[k]];
-}
-
+// v_w[k] = w of CSC entry k's hyperedge, and
 // deg_v[v] = sum of the CSC row's weights: lane-strided partial sums, then a
 // fixed xor-shuffle tree (deterministic). Rows longer than kLongRow are
 // appended to `long_rows` and left to deg_long_kernel (a warp on a row of
@@ -117,7 +87,8 @@ __global__ void csc_weights_kernel(int64_t nnz, const int32_t* __restrict__ v_ed
 constexpr int32_t kLongRow = 4096;
 
 __global__ void deg_kernel(int32_t n, const int32_t* __restrict__ v_ptr,
-                           const float* __restrict__ v_w, float* __restrict__ deg,
+                           const int32_t* __restrict__ v_edges, const float* __restrict__ w,
+                           float* __restrict__ v_w, float* __restrict__ deg,
                            float* __restrict__ inv_deg, int32_t* __restrict__ long_rows,
                            int32_t* __restrict__ n_long) {
   const int lane = threadIdx.x & 31;
@@ -130,7 +101,11 @@ __global__ void deg_kernel(int32_t n, const int32_t* __restrict__ v_ptr,
       continue;
     }
     float s = 0.f;
-    for (int64_t k = b + lane; k < e; k += 32) s += v_w[k];
+    for (int64_t k = b + lane; k < e; k += 32) {
+      const float x = w[v_edges[k]];
+      v_w[k] = x;
+      s += x;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
     if (lane == 0) {
@@ -158,15 +133,30 @@ __device__ float block_sum_fixed(float x, float* sm) {
 
 __global__ void __launch_bounds__(kLongThreads)
 deg_long_kernel(const int32_t* __restrict__ long_rows, const int32_t* __restrict__ n_long,
-                const int32_t* __restrict__ v_ptr, const float* __restrict__ v_w,
-                float* __restrict__ deg, float* __restrict__ inv_deg) {
+                const int32_t* __restrict__ v_ptr, const int32_t* __restrict__ v_edges,
+                const float* __restrict__ w, float* __restrict__ v_w, float* __restrict__ deg,
+                float* __restrict__ inv_deg) {
   __shared__ float sm[kLongThreads];
   const int32_t count = *n_long;
   for (int32_t i = blockIdx.x; i < count; i += gridDim.x) {
     const int32_t v = long_rows[i];
     const int64_t b = v_ptr[v], e = v_ptr[v + 1];
     float s = 0.f;
-    for (int64_t k = b + threadIdx.x; k < e; k += kLongThreads) s += v_w[k];
+    // eight loads in flight, added in order
+    for (int64_t k = b + threadIdx.x; k < e; k += 8 * kLongThreads) {
+      float x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int64_t at = k + u * kLongThreads;
+        x[u] = at < e ? w[v_edges[at]] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int64_t at = k + u * kLongThreads;
+        if (at < e) v_w[at] = x[u];
+        s += x[u];   // (past the end: + 0, exact)
+      }
+    }
     s = block_sum_fixed(s, sm);
     if (threadIdx.x == 0) {
       deg[v] = s;
@@ -247,18 +237,21 @@ __global__ void long_chunk_counts(const uint64_t* __restrict__ keys, int32_t beg
   }
 }
 
+// (a warp per row: its lanes write the chunks)
 __global__ void fill_long(const uint64_t* __restrict__ keys, int32_t begin, int32_t count,
                           const int32_t* __restrict__ ptr, int32_t T,
                           const int32_t* __restrict__ chunk_off, int4* __restrict__ long_desc,
                           int4* __restrict__ chunk_items) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < count;
+       i += warps) {
     const int32_t r = (int32_t)(uint32_t)keys[begin + i];
     const int32_t b = ptr[r], e = ptr[r + 1];
     const int32_t c0 = chunk_off[i];
     const int32_t nc = (e - b + T - 1) / T;
-    long_desc[i] = make_int4(r, c0, nc, 0);
-    for (int32_t j = 0; j < nc; ++j) {
+    if (lane == 0) long_desc[i] = make_int4(r, c0, nc, 0);
+    for (int32_t j = lane; j < nc; j += 32) {
       const int32_t s = b + j * T;
       chunk_items[c0 + j] = make_int4(r, s, min(T, e - s), c0 + j);
     }
@@ -360,7 +353,7 @@ int build_split_plan(hnv_graph* g, std::vector<void*>* owned, const int32_t* ptr
                      (const uint64_t*)sorted, off[1], n_rows_items, ptr, plan->items));
   if (n_long > 0) {
     HNV_CHECK(owned_alloc(owned, (void**)&plan->long_desc, sizeof(int4) * (size_t)n_long, s));
-    HNV_CHECK(launch("fill_long", fill_long, grid_for(n_long, 256), 256, 0, s,
+    HNV_CHECK(launch("fill_long", fill_long, grid_for((int64_t)n_long * 32, 256), 256, 0, s,
                      (const uint64_t*)sorted, off[5], n_long, ptr, T, (const int32_t*)chunk_off,
                      plan->long_desc, plan->items + n_rows_items));
   }
@@ -623,19 +616,18 @@ int side_plan(hnv_graph* g, Level* lv, int side, size_t row_bytes, const SplitPl
 }
 
 int level_weight_arrays(Level* lv, cudaStream_t s) {
-  HNV_CHECK(launch("csc_weights", csc_weights_kernel, grid_for(lv->nnz, 256), 256, 0, s, lv->nnz,
-                   (const int32_t*)lv->v_edges, (const float*)lv->w, lv->v_w));
   TempPool pool(s);
   int32_t *long_rows = nullptr, *n_long = nullptr;
   HNV_CHECK(pool.get(&long_rows, (size_t)(lv->nnz / kLongRow + 1)));
   HNV_CHECK(pool.get(&n_long, 1));
   HNV_CUDA(cudaMemsetAsync(n_long, 0, sizeof(int32_t), s));
   HNV_CHECK(launch("deg", deg_kernel, grid_for((int64_t)lv->n * 32, 256), 256, 0, s, lv->n,
-                   (const int32_t*)lv->v_ptr, (const float*)lv->v_w, lv->deg_v, lv->inv_deg_v,
-                   long_rows, n_long));
+                   (const int32_t*)lv->v_ptr, (const int32_t*)lv->v_edges, (const float*)lv->w,
+                   lv->v_w, lv->deg_v, lv->inv_deg_v, long_rows, n_long));
   return launch("deg_long", deg_long_kernel, (unsigned)(2 * num_sms()), kLongThreads, 0, s,
                 (const int32_t*)long_rows, (const int32_t*)n_long, (const int32_t*)lv->v_ptr,
-                (const float*)lv->v_w, lv->deg_v, lv->inv_deg_v);
+                (const int32_t*)lv->v_edges, (const float*)lv->w, lv->v_w, lv->deg_v,
+                lv->inv_deg_v);
 }
 
 int finish_level(hnv_graph* g, Level* lv) {
@@ -690,11 +682,11 @@ int build_level0(hnv_graph* g, int32_t n, int32_t m, const int64_t* d_edge_ptr,
   // 2. sort (hyperedge, node) keys and drop repeats
   TempPool pool(s);
   uint64_t *k0 = nullptr, *k1 = nullptr, *sorted = nullptr;
-  int32_t *first = nullptr, *pos = nullptr, *cnt = nullptr;
+  int32_t* tiles = nullptr;
   HNV_CHECK(pool.get(&k0, (size_t)nnz_in));
   HNV_CHECK(pool.get(&k1, (size_t)nnz_in));
-  HNV_CHECK(launch("pack_input_keys", pack_input_keys, grid_for((int64_t)m * 32, 256), 256, 0, s,
-                   m, n, d_edge_ptr, d_edge_nodes, k0, g->d_err));
+  HNV_CHECK(launch("pack_input_keys", pack_input_keys, entry_grid(nnz_in), kEntryThreads, 0, s,
+                   m, n, nnz_in, d_edge_ptr, d_edge_nodes, k0, g->d_err));
   HNV_CHECK(read_and_clear_err(g, s, &bits));
   if (bits & ERRBIT_NODE_RANGE) HNV_FAIL(HNV_ERR_OUT_OF_RANGE, "a node ID is outside [0, n)");
   // the keys are grouped by hyperedge already: sorting every hyperedge's run
@@ -712,22 +704,15 @@ int build_level0(hnv_graph* g, int32_t n, int32_t m, const int64_t* d_edge_ptr,
     const int np = radix_shifts(bits_for_count(n), bits_for_count(m), shifts);
     HNV_CHECK(radix_sort_u64(k0, k1, nnz_in, shifts, np, s, &sorted));
   }
-  HNV_CHECK(pool.get(&first, (size_t)nnz_in));
-  HNV_CHECK(pool.get(&pos, (size_t)nnz_in));
-  HNV_CHECK(pool.get(&cnt, (size_t)m + 1));
-  HNV_CHECK(launch("first_flags", first_flags, grid_for(nnz_in, 256), 256, 0, s,
-                   (const uint64_t*)sorted, nnz_in, first));
-  HNV_CHECK(exclusive_scan_i32(first, pos, nnz_in, g->d_buf, s));
+  HNV_CHECK(pool.get(&tiles, (size_t)compact_tiles(nnz_in)));
+  HNV_CHECK(unique_count(sorted, nnz_in, tiles, g->d_buf, s));
   int32_t nnz = 0;
   HNV_CHECK(read_ints(g, g->d_buf, 1, &nnz, s));
   lv->nnz = nnz;
   HNV_CHECK(level_alloc(lv, (void**)&lv->e_ptr, sizeof(int32_t) * ((size_t)m + 1), s));
   HNV_CHECK(level_alloc(lv, (void**)&lv->e_nodes, sizeof(int32_t) * (size_t)nnz, s));
-  HNV_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * ((size_t)m + 1), s));
-  HNV_CHECK(launch("csr_from_unique", csr_from_unique, grid_for(nnz_in, 256), 256, 0, s,
-                   (const uint64_t*)sorted, nnz_in, (const int32_t*)first, (const int32_t*)pos,
-                   lv->e_nodes, cnt));
-  HNV_CHECK(exclusive_scan_i32(cnt, lv->e_ptr, (int64_t)m + 1, nullptr, s));
+  HNV_CHECK(unique_csr(sorted, nnz_in, tiles, lv->e_nodes, lv->e_ptr, s));
+  HNV_CHECK(fill_i32(lv->e_ptr + m, nnz, 1, s));
 
   // 3. weights (copy, or all ones) and level-0 IDs
   HNV_CHECK(level_alloc(lv, (void**)&lv->w, sizeof(float) * (size_t)m, s));

@@ -196,9 +196,10 @@ __global__ void fill_i32_kernel(int32_t* p, int32_t v, int64_t n) {
 }
 
 // key = (col << 32) | row for every CSR entry.
-__global__ void pack_col_row(int32_t n_rows, const int32_t* __restrict__ row_ptr,
-                             const int32_t* __restrict__ cols, uint64_t* __restrict__ keys) {
-  csr_rows_warp_visit(n_rows, row_ptr, [&](int64_t r, int64_t k) {
+__global__ void __launch_bounds__(kEntryThreads)
+pack_col_row(int32_t n_rows, int64_t nnz, const int32_t* __restrict__ row_ptr,
+             const int32_t* __restrict__ cols, uint64_t* __restrict__ keys) {
+  csr_entries_visit(n_rows, row_ptr, nnz, [&](int64_t r, int64_t k) {
     keys[k] = ((uint64_t)(uint32_t)cols[k] << 32) | (uint32_t)r;
   });
 }
@@ -215,6 +216,31 @@ __global__ void col_starts(const uint64_t* __restrict__ keys, int64_t n, int32_t
     const int64_t cur = i < n ? (int64_t)(uint32_t)(keys[i] >> 32) : (int64_t)n_cols;
     for (int64_t c = prev + 1; c <= cur; ++c) col_ptr[c] = (int32_t)i;
   }
+}
+
+// Unique (row, col) keys -> CSR columns and row offsets. An entry that is
+// kept and starts another row than the entry before it writes the offsets of
+// every row up to its own (rows are non-empty, so that is one).
+__device__ __forceinline__ bool first_of_run(const uint64_t* __restrict__ keys, int64_t k) {
+  return k == 0 || keys[k] != keys[k - 1];
+}
+
+__global__ void __launch_bounds__(kCompactThreads)
+unique_count_kernel(const uint64_t* __restrict__ keys, int64_t n, int32_t* __restrict__ tile_count) {
+  compact_count(n, tile_count, [&](int64_t k) { return first_of_run(keys, k); });
+}
+
+__global__ void __launch_bounds__(kCompactThreads)
+unique_csr_kernel(const uint64_t* __restrict__ keys, int64_t n, const int32_t* __restrict__ tile_off,
+                int32_t* __restrict__ cols, int32_t* __restrict__ row_ptr) {
+  compact_write(
+      n, tile_off, [&](int64_t k) { return first_of_run(keys, k); },
+      [&](int64_t k, int32_t at) {
+        const uint64_t key = keys[k];
+        cols[at] = (int32_t)(uint32_t)key;
+        const uint32_t row = (uint32_t)(key >> 32);
+        if (k == 0 || (uint32_t)(keys[k - 1] >> 32) != row) row_ptr[row] = at;
+      });
 }
 
 __global__ void low_words(const uint64_t* __restrict__ keys, int64_t n, int32_t* __restrict__ out) {
@@ -547,6 +573,19 @@ int exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int32_t* tota
                 (const int32_t*)sums, (int32_t*)nullptr);
 }
 
+int unique_count(const uint64_t* keys, int64_t n, int32_t* tiles, int32_t* total, cudaStream_t s) {
+  const int64_t nt = compact_tiles(n);
+  HNV_CHECK(launch("unique_count", unique_count_kernel, (unsigned)nt, kCompactThreads, 0, s, keys,
+                   n, tiles));
+  return exclusive_scan_i32(tiles, tiles, nt, total, s);
+}
+
+int unique_csr(const uint64_t* keys, int64_t n, const int32_t* tiles, int32_t* cols,
+               int32_t* row_ptr, cudaStream_t s) {
+  return launch("unique_csr", unique_csr_kernel, (unsigned)compact_tiles(n), kCompactThreads, 0, s,
+                keys, n, tiles, cols, row_ptr);
+}
+
 int bits_for_count(int64_t count) {
   int b = 0;
   while (b < 63 && (int64_t(1) << b) < count) ++b;
@@ -601,8 +640,8 @@ int transpose_csr(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* ro
   uint64_t *k0 = nullptr, *k1 = nullptr, *sorted = nullptr;
   HNV_CHECK(pool.get(&k0, (size_t)nnz));
   HNV_CHECK(pool.get(&k1, (size_t)nnz));
-  HNV_CHECK(launch("pack_col_row", pack_col_row, grid_for((int64_t)n_rows, 256), 256, 0, s,
-                   n_rows, row_ptr, cols, k0));
+  HNV_CHECK(launch("pack_col_row", pack_col_row, entry_grid(nnz), kEntryThreads, 0, s, n_rows,
+                   nnz, row_ptr, cols, k0));
   int shifts[16];
   int np = radix_shifts(0, bits_for_count(n_cols), shifts);
   HNV_CHECK(radix_sort_u64(k0, k1, nnz, shifts, np, s, &sorted));
