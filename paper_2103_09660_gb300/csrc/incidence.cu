@@ -188,14 +188,17 @@ __global__ void classify_rows(int32_t rows, const int32_t* __restrict__ ptr, int
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
        r += (int64_t)gridDim.x * blockDim.x) {
     const int32_t d = ptr[r + 1] - ptr[r];
-    int c;
+    int c, lo = 0, hi = 0;
     if (d == 0) c = 0;
     else if (d <= shape.a_max) c = 1;
-    else if (d <= shape.b_max) c = 2;
-    else if (d <= shape.c_max) c = 3;
-    else if (d <= T) c = 4;
+    else if (d <= shape.b_max) c = 2, lo = shape.a_max + 1, hi = shape.b_max;
+    else if (d <= shape.c_max) c = 3, lo = shape.b_max + 1, hi = shape.c_max;
+    else if (d <= T) c = 4, lo = shape.c_max + 1, hi = T;
     else c = ((d + T - 1) / T <= mid_chunks) ? 5 : 6;
-    keys[r] = ((uint64_t)c << 32) | (uint32_t)r;
+    // within B, C and D by eighths of the class's lengths, so that the rows a
+    // warp takes together need about as many rounds of loads
+    const int sub = hi > lo ? (d - lo) * 8 / (hi - lo + 1) : 0;
+    keys[r] = ((uint64_t)(c * 8 + sub) << 32) | (uint32_t)r;
     atomicAdd(&h[c], 1);
   }
   __syncthreads();
@@ -325,7 +328,7 @@ int build_split_plan(hnv_graph* g, std::vector<void*>* owned, const int32_t* ptr
   HNV_CHECK(launch("classify_rows", classify_rows, grid_for(rows, 256), 256, 0, s, rows, ptr, T,
                    kMidChunks, shape, k0, cnt));
   const int shift = 32;
-  HNV_CHECK(radix_sort_u64(k0, k1, rows, &shift, 1, s, &sorted));   // stable: rows ascend per class
+  HNV_CHECK(radix_sort_u64(k0, k1, rows, &shift, 1, s, &sorted));   // stable: rows ascend per class and eighth
   int32_t c[kClasses];
   HNV_CHECK(read_ints(g, cnt, kClasses, c, s));
   int32_t off[kClasses + 1] = {0};

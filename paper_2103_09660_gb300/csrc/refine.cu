@@ -44,7 +44,7 @@ constexpr int kGatherThreads = 64;
 // Passes per warp of the packed short-row kernel (see gather_packed_kernel).
 constexpr int kPackedPasses = 4;
 
-template <typename T, int G, int VPL, bool WEIGHTED, bool WIDE_U = false>
+template <typename T, int G, int VPL, bool WEIGHTED, bool LONG>
 __global__ void __launch_bounds__(256)
 gather_kernel(const int4* __restrict__ items, int32_t n_items, const int32_t* __restrict__ idx,
               const float* __restrict__ inc_w, const float* __restrict__ inv_norm,
@@ -60,8 +60,8 @@ gather_kernel(const int4* __restrict__ items, int32_t n_items, const int32_t* __
     const int64_t item = wbase + grp;
     int4 it = make_int4(-1, 0, 0, -1);
     if (item < n_items) it = __ldg(items + item);
-    dev::gather_item<T, G, VPL, WEIGHTED, false, WIDE_U>(it, lg, idx, inc_w, inv_norm, src,
-                                                         self_in, out, dv, keep, scale, partials);
+    dev::gather_item<T, G, VPL, WEIGHTED, false, LONG>(it, lg, idx, inc_w, inv_norm, src, self_in,
+                                                       out, dv, keep, scale, partials);
   }
 }
 
@@ -141,8 +141,10 @@ gather_packed_kernel(const int4* __restrict__ items, const void* __restrict__ me
     float nw;
     const int4 nn = load_it(k + 2);
     load_head(k + 2, ni, nw);
-    dev::gather_item<T, G, VPL, false, true>(cur, lg, idx, inc_w, inv_norm, src, self_in, out,
-                                             dv, keep, scale, partials, ci, cw);
+    // a row of 1-4 members takes one round of 4 loads; with 8 the short rows'
+    // instructions doubled where a lane has one vector
+    dev::gather_item<T, G, VPL, false, true, false, false, PK == 1 && VPL == 1 ? 4 : 0>(
+        cur, lg, idx, inc_w, inv_norm, src, self_in, out, dv, keep, scale, partials, ci, cw);
     cur = nxt;
     ci = xi;
     cw = xw;
@@ -245,8 +247,9 @@ bool use_tma(int d) {
   return mode == 1 && tma_supported(d);
 }
 
+// `lng`: the long classes (rows of 17 incidences and more, chunks).
 template <typename T, int G, int VPL>
-int launch_items(const HalfSweep& h, const int4* items, int32_t n_items, const void* src,
+int launch_items(const HalfSweep& h, const int4* items, int32_t n_items, bool lng, const void* src,
                  const void* self_in, void* out, int dv, float keep, float scale,
                  float* partials, cudaStream_t s) {
   if (n_items <= 0) return HNV_OK;
@@ -255,18 +258,11 @@ int launch_items(const HalfSweep& h, const int4* items, int32_t n_items, const v
   const int64_t warps = ((int64_t)n_items + R - 1) / R;
   const int64_t blocks64 = (warps + WPB - 1) / WPB;
   const unsigned blocks = (unsigned)(blocks64 > 0x7fffffff ? 0x7fffffff : blocks64);
-  // the weighted long-row kernel keeps 8 row loads in flight per lane (not
-  // the weighted default of 4): the coarse levels' node half-sweeps, bound
-  // by L2 latency, got 1-2% faster; level 0 is unchanged
-  if (h.inc_w && G == 32 && VPL == 1)
-    return launch("gather_w", gather_kernel<T, G, VPL, true, true>, blocks, kGatherThreads, 0, s,
-                  items, n_items, h.idx, h.inc_w, h.inv_norm, (const uint4*)src,
-                  (const uint4*)self_in, (uint4*)out, dv, keep, scale, partials);
-  if (h.inc_w)
-    return launch("gather_w", gather_kernel<T, G, VPL, true>, blocks, kGatherThreads, 0, s,
-                  items, n_items, h.idx, h.inc_w, h.inv_norm, (const uint4*)src,
-                  (const uint4*)self_in, (uint4*)out, dv, keep, scale, partials);
-  return launch("gather", gather_kernel<T, G, VPL, false>, blocks, kGatherThreads, 0, s, items,
+  auto kern = h.inc_w ? (lng ? gather_kernel<T, G, VPL, true, true>
+                             : gather_kernel<T, G, VPL, true, false>)
+                      : (lng ? gather_kernel<T, G, VPL, false, true>
+                             : gather_kernel<T, G, VPL, false, false>);
+  return launch(h.inc_w ? "gather_w" : "gather", kern, blocks, kGatherThreads, 0, s, items,
                 n_items, h.idx, h.inc_w, h.inv_norm, (const uint4*)src, (const uint4*)self_in,
                 (uint4*)out, dv, keep, scale, partials);
 }
@@ -320,11 +316,11 @@ int launch_packed16_dispatch(int G, int VPL, const HalfSweep& h, const int4* ite
 
 template <typename T>
 int launch_items_dispatch(int G, int VPL, const HalfSweep& h, const int4* items, int32_t n_items,
-                          const void* src, const void* self_in, void* out, int dv, float keep,
+                          bool lng, const void* src, const void* self_in, void* out, int dv, float keep,
                           float scale, float* partials, cudaStream_t s) {
 #define HNV_CASE(g, v)                                                                       \
   if (G == g && VPL == v)                                                                    \
-    return launch_items<T, g, v>(h, items, n_items, src, self_in, out, dv, keep, scale,     \
+    return launch_items<T, g, v>(h, items, n_items, lng, src, self_in, out, dv, keep, scale,     \
                                  partials, s);
   HNV_CASE(1, 1) HNV_CASE(2, 1) HNV_CASE(4, 1)
   HNV_CASE(8, 1) HNV_CASE(8, 2) HNV_CASE(8, 4) HNV_CASE(8, 8)
@@ -409,8 +405,8 @@ int run_half(const HalfSweep& h, const void* src, const void* self_in, void* out
         rc = launch_packed16_dispatch<T>(G, VPL, h, items + off, p.b_members, counts[1], src,
                                          self_in, out, dv, keep, scale, partials, cs[c]);
       if (rc == 1)
-        rc = launch_items_dispatch<T>(G, VPL, h, items + off, counts[c], src, self_in, out, dv,
-                                      keep, scale, partials, cs[c]);
+        rc = launch_items_dispatch<T>(G, VPL, h, items + off, counts[c], c == 2, src, self_in, out,
+                                      dv, keep, scale, partials, cs[c]);
       HNV_CHECK(rc);
       off += counts[c];
     }

@@ -106,9 +106,11 @@ __device__ __forceinline__ void diff_max(const uint4& stored, const float* old, 
 // PRE: the caller supplies this lane's first neighbour index (incidence
 // beg + lg, any value where lg >= len) in idx0 instead of it being loaded,
 // and for a weighted side that incidence's weight in w0.
+// LONG: an item of the long classes (rounds in which every group of the warp
+// has U more incidences go without predicates).
 // COH: see load_row. UO: row loads in flight per lane (0: the default).
 // DIFF: the largest change of a coordinate of the row goes to *diff (max).
-template <typename T, int G, int VPL, bool WEIGHTED, bool PRE = false, bool WIDE_U = false,
+template <typename T, int G, int VPL, bool WEIGHTED, bool PRE = false, bool LONG = false,
           bool COH = false, int UO = 0, bool DIFF = false>
 __device__ __forceinline__ void gather_item(int4 it, int lg, const int32_t* __restrict__ idx,
                                             const float* __restrict__ inc_w,
@@ -121,10 +123,15 @@ __device__ __forceinline__ void gather_item(int4 it, int lg, const int32_t* __re
   constexpr int N = V::N;
   // row loads in flight per lane (the weighted variant also holds a weight
   // per load, so it takes half as many to keep its register count down,
-  // unless WIDE_U)
+  // unless LONG)
   constexpr int UB0 = (VPL == 1) ? 8 : (VPL == 2 ? 4 : (VPL == 4 ? 2 : 1));
-  constexpr int UB = UO > 0 ? UO : ((WEIGHTED && UB0 > 1 && !WIDE_U) ? UB0 / 2 : UB0);
+  constexpr int UB = UO > 0 ? UO : ((WEIGHTED && UB0 > 1 && !LONG) ? UB0 / 2 : UB0);
   constexpr int U = UB < G ? UB : G;
+  // Full rounds pay where a warp has one row, or a bfloat16 row, whose
+  // conversions bind the issue slots (d = 128: V-cycle of 1M nodes 75.2 ->
+  // 67.3 ms in bfloat16, 94.5 -> 91.4 in float32); with two float32 rows per
+  // warp they cost 3-5% (d = 64).
+  constexpr bool FULL = LONG && (G == 32 || N == 8);
   const bool read_self = DIFF || keep != 0.f;
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
     const int32_t row = it.x, beg = it.y, len = it.z, slot = it.w;
@@ -153,27 +160,60 @@ __device__ __forceinline__ void gather_item(int4 it, int lg, const int32_t* __re
       for (int e = 0; e < N; ++e) acc[j][e] = 0.f;
 
     const int32_t maxlen = __reduce_max_sync(kFull, len);
-    int32_t nx_idx = 0;       // UO: the next G neighbours, loaded a round ahead
+    // full rounds (every group of the warp has U more incidences) need no
+    // predicates and no zeros: lanes past the row's width load its last vector
+    const int32_t minlen = !FULL ? 0 : (G == 32 ? maxlen : __reduce_min_sync(kFull, len));
+    const char* base[VPL];
+#pragma unroll
+    for (int j = 0; j < VPL; ++j)
+      base[j] = reinterpret_cast<const char*>(src + (lg + j * G < dv ? lg + j * G : dv - 1));
+    const uint32_t row_bytes = (uint32_t)dv * 16u;
+    int32_t nx_idx = 0;       // COH: the next G neighbours, loaded a round ahead
     float nx_w = 0.f;
     for (int32_t off = 0; off < maxlen; off += G) {
       const int32_t mine = len - off;
       const bool have = lg < mine;
       int32_t my_idx;
       float my_w = 0.f;
-      if (UO > 0 && off > 0) {
+      if (COH && off > 0) {
         my_idx = nx_idx;
         my_w = nx_w;
       } else {
         my_idx = have ? ((PRE && off == 0) ? idx0 : __ldg(idx + beg + off + lg)) : 0;
         if (WEIGHTED) my_w = have ? ((PRE && off == 0) ? w0 : __ldg(inc_w + beg + off + lg)) : 0.f;
       }
-      if (UO > 0) {
+      if (COH) {
         const bool more = lg + G < mine;
         nx_idx = more ? __ldg(idx + beg + off + G + lg) : 0;
         if (WEIGHTED) nx_w = more ? __ldg(inc_w + beg + off + G + lg) : 0.f;
       }
       const int32_t cnt = min(G, maxlen - off);
-      for (int32_t t = 0; t < cnt; t += U) {
+      const int32_t nfull = min(G, minlen - off);
+      int32_t t = 0;
+      for (; FULL && t + U <= nfull; t += U) {
+        uint4 x[U][VPL];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint32_t nb = (uint32_t)__shfl_sync(kFull, my_idx, t + u, G);
+#pragma unroll
+          for (int j = 0; j < VPL; ++j)
+            x[u][j] = load_row<COH>(
+                reinterpret_cast<const uint4*>(base[j] + (uint64_t)nb * row_bytes));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float w = WEIGHTED ? __shfl_sync(kFull, my_w, t + u, G) : 1.f;
+#pragma unroll
+          for (int j = 0; j < VPL; ++j) {
+            float xf[N];
+            V::unpack(x[u][j], xf);
+#pragma unroll
+            for (int e = 0; e < N; ++e)
+              acc[j][e] = WEIGHTED ? fmaf(w, xf[e], acc[j][e]) : acc[j][e] + xf[e];
+          }
+        }
+      }
+      for (; t < cnt; t += U) {
         uint4 x[U][VPL];
         float wt[U];
 #pragma unroll
