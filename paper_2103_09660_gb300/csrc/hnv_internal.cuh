@@ -493,6 +493,9 @@ int coarsen_step(hnv_graph* g, int level, const hnv_coarsen_params* p, const uin
 // dtype: HNV_F32 or HNV_BF16 row storage (sums in float32 either way).
 int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d, float omega,
                  int sweeps, int mode, cudaStream_t s);
+// One sweep from (v_in, e_in) into the buffers (v_out, e_out) (no overlap).
+int refine_sweep_into(hnv_graph* g, int level, const void* v_in, const void* e_in, void* v_out,
+                      void* e_out, int dtype, int d, float omega, int mode, cudaStream_t s);
 int project_level(const hnv_graph* g, int fine_level, const void* zc_v, const void* zc_e,
                   void* zf_v, void* zf_e, int dtype, int d, cudaStream_t s);
 // Sweeps until the largest change of any coordinate in a sweep is <= eps, or

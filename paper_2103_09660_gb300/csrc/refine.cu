@@ -24,6 +24,7 @@
 
 #include <algorithm>
 #include <cstdlib>
+#include <utility>
 
 #include "refine_device.cuh"
 
@@ -531,6 +532,51 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
   return team_launch(a, 1, dtype, d, s);
 }
 
+namespace {
+
+// Compulsory bytes of a half-sweep (0 hyperedge side, 1 node side).
+double half_bytes(const Level& lv, int side, int dtype, int d) {
+  const double es = (double)elem_size(dtype), n = lv.n, m = lv.m, nnz = (double)lv.nnz;
+  return side == 0 ? es * (n * d + 2.0 * m * d) + 4.0 * (nnz + 2.0 * m + 1.0)
+                   : es * (m * d + 2.0 * n * d) + 4.0 * (2.0 * nnz + 2.0 * n + 1.0);
+}
+
+// Both half-sweeps of a level on its plans for d, with scratch for their
+// split rows.
+int level_halves(hnv_graph* g, int level, int dtype, int d, HalfSweep* E, HalfSweep* V,
+                 cudaStream_t s) {
+  Level& lv = g->levels[level];
+  const size_t es = elem_size(dtype);
+  const SplitPlan* planE = &lv.planE;
+  const SplitPlan* planV = &lv.planV;
+  if (!use_tma(d)) {
+    HNV_CHECK(side_plan(g, &lv, 0, es * (size_t)d, &planE, s));
+    HNV_CHECK(side_plan(g, &lv, 1, es * (size_t)d, &planV, s));
+  }
+  const int64_t chunks = planE->n_chunks > planV->n_chunks ? planE->n_chunks : planV->n_chunks;
+  HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes,
+                           sizeof(float) * (size_t)(chunks > 0 ? chunks : 1) * d, s));
+  *E = HalfSweep{lv.e_nodes, nullptr, lv.inv_size_e, planE, lv.n, lv.m, g->d_err};
+  *V = HalfSweep{lv.v_edges, lv.v_w, lv.inv_deg_v, planV, lv.m, lv.n, g->d_err};
+  if (g->aux[0] && g->aux[1]) E->conc = V->conc = g;
+  return HNV_OK;
+}
+
+}  // namespace
+
+int refine_sweep_into(hnv_graph* g, int level, const void* v_in, const void* e_in, void* v_out,
+                      void* e_out, int dtype, int d, float omega, int mode, cudaStream_t s) {
+  HalfSweep E, V;
+  HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, s));
+  {
+    PhaseScope ps(HNV_PHASE_REFINE_E, s, half_bytes(g->levels[level], 0, dtype, d));
+    HNV_CHECK(run_half_dispatch(E, v_in, e_in, e_out, dtype, d, omega, g->partials, s));
+  }
+  PhaseScope ps(HNV_PHASE_REFINE_V, s, half_bytes(g->levels[level], 1, dtype, d));
+  return run_half_dispatch(V, mode == HNV_SWEEP_JACOBI ? e_in : e_out, v_in, v_out, dtype, d,
+                           omega, g->partials, s);
+}
+
 int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d, float omega,
                  int sweeps, int mode, cudaStream_t s) {
   NvtxRange nvtx("hnv refine level %d (%d sweeps)", level, sweeps);
@@ -543,25 +589,17 @@ int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d
     t.ze0 = static_cast<uint4*>(z_e);
     return team_run(g, t, dtype, d, omega, sweeps, mode, s);
   }
+  HalfSweep E, V;
+  HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, s));
   const size_t es = elem_size(dtype);
-  const SplitPlan* planE = &lv.planE;
-  const SplitPlan* planV = &lv.planV;
-  if (!use_tma(d)) {
-    HNV_CHECK(side_plan(g, &lv, 0, es * (size_t)d, &planE, s));
-    HNV_CHECK(side_plan(g, &lv, 1, es * (size_t)d, &planV, s));
-  }
-  const int64_t chunks = planE->n_chunks > planV->n_chunks ? planE->n_chunks : planV->n_chunks;
-  HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes,
-                           sizeof(float) * (size_t)(chunks > 0 ? chunks : 1) * d, s));
   if (mode == HNV_SWEEP_JACOBI)
     HNV_CHECK(ensure_scratch(&g->jacobi_tmp, &g->jacobi_bytes,
                              es * ((size_t)lv.m > 0 ? lv.m : 1) * d, s));
-  HalfSweep E{lv.e_nodes, nullptr, lv.inv_size_e, planE, lv.n, lv.m, g->d_err};
-  HalfSweep V{lv.v_edges, lv.v_w, lv.inv_deg_v, planV, lv.m, lv.n, g->d_err};
-  if (g->aux[0] && g->aux[1]) E.conc = V.conc = g;
-  const double n = lv.n, m = lv.m, nnz = (double)lv.nnz;
-  const double bytesE = (double)es * (n * d + 2.0 * m * d) + 4.0 * (nnz + 2.0 * m + 1.0);
-  const double bytesV = (double)es * (m * d + 2.0 * n * d) + 4.0 * (2.0 * nnz + 2.0 * n + 1.0);
+  const double bytesE = half_bytes(lv, 0, dtype, d), bytesV = half_bytes(lv, 1, dtype, d);
+  // Jacobi: the new hyperedge rows go to a second buffer, the nodes read the
+  // old ones, and the buffers change places (one copy back at most, not one a
+  // sweep)
+  void *e_cur = z_e, *e_nxt = g->jacobi_tmp;
   for (int it = 0; it < sweeps; ++it) {
     if (mode == HNV_SWEEP_TWO_PHASE) {
       {
@@ -575,17 +613,17 @@ int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d
     } else {
       {
         PhaseScope ps(HNV_PHASE_REFINE_E, s, bytesE);
-        HNV_CHECK(run_half_dispatch(E, z_v, z_e, g->jacobi_tmp, dtype, d, omega, g->partials, s));
+        HNV_CHECK(run_half_dispatch(E, z_v, e_cur, e_nxt, dtype, d, omega, g->partials, s));
       }
       {
         PhaseScope ps(HNV_PHASE_REFINE_V, s, bytesV);
-        HNV_CHECK(run_half_dispatch(V, z_e, z_v, z_v, dtype, d, omega, g->partials, s));
+        HNV_CHECK(run_half_dispatch(V, e_cur, z_v, z_v, dtype, d, omega, g->partials, s));
       }
-      if (lv.m > 0)
-        HNV_CUDA(cudaMemcpyAsync(z_e, g->jacobi_tmp, es * (size_t)lv.m * d,
-                                 cudaMemcpyDeviceToDevice, s));
+      std::swap(e_cur, e_nxt);
     }
   }
+  if (e_cur != z_e && lv.m > 0)
+    HNV_CUDA(cudaMemcpyAsync(z_e, e_cur, es * (size_t)lv.m * d, cudaMemcpyDeviceToDevice, s));
   return HNV_OK;
 }
 
