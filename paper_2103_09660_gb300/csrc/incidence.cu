@@ -177,13 +177,15 @@ deg_long_kernel(const int32_t* __restrict__ long_rows, const int32_t* __restrict
 // Row class for the refinement plan: 0 empty, 1 A (1..a_max), 2 B (..b_max),
 // 3 C (..c_max), 4 D (..T), 5 split into at most mid_chunks chunks, 6 split
 // into more.
+// counts[0..6]: rows per class; [7], [8]: chunks of the class 5 and 6 rows.
 constexpr int kClasses = 7;
+constexpr int kPlanCounts = 9;
 
 __global__ void classify_rows(int32_t rows, const int32_t* __restrict__ ptr, int32_t T,
                               int32_t mid_chunks, PlanShape shape, uint64_t* __restrict__ keys,
                               int32_t* __restrict__ counts) {
-  __shared__ int32_t h[kClasses];
-  if (threadIdx.x < kClasses) h[threadIdx.x] = 0;
+  __shared__ int32_t h[kPlanCounts];
+  if (threadIdx.x < kPlanCounts) h[threadIdx.x] = 0;
   __syncthreads();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
        r += (int64_t)gridDim.x * blockDim.x) {
@@ -200,9 +202,10 @@ __global__ void classify_rows(int32_t rows, const int32_t* __restrict__ ptr, int
     const int sub = hi > lo ? (d - lo) * 8 / (hi - lo + 1) : 0;
     keys[r] = ((uint64_t)(c * 8 + sub) << 32) | (uint32_t)r;
     atomicAdd(&h[c], 1);
+    if (c >= 5) atomicAdd(&h[c + 2], (d + T - 1) / T);
   }
   __syncthreads();
-  if (threadIdx.x < kClasses && h[threadIdx.x]) atomicAdd(&counts[threadIdx.x], h[threadIdx.x]);
+  if (threadIdx.x < kPlanCounts && h[threadIdx.x]) atomicAdd(&counts[threadIdx.x], h[threadIdx.x]);
 }
 
 __global__ void fill_row_items(const uint64_t* __restrict__ keys, int32_t begin, int32_t count,
@@ -313,24 +316,57 @@ static int owned_alloc(std::vector<void*>* owned, void** p, size_t bytes, cudaSt
   return HNV_OK;
 }
 
+namespace {
+
+// A plan in the making: its rows' (class, row) keys, sorted.
+struct PlanKeys {
+  uint64_t* sorted = nullptr;
+};
+
+// Classifies the rows into cnt[0 .. kPlanCounts) (device, zeroed by the
+// caller) and sorts them by class.
+int plan_classify(const int32_t* ptr, int32_t rows, const PlanShape& shape, int32_t* cnt,
+                  TempPool& pool, PlanKeys* out, cudaStream_t s) {
+  if (rows == 0) return HNV_OK;
+  uint64_t *k0 = nullptr, *k1 = nullptr;
+  HNV_CHECK(pool.get(&k0, (size_t)rows));
+  HNV_CHECK(pool.get(&k1, (size_t)rows));
+  HNV_CHECK(launch("classify_rows", classify_rows, grid_for(rows, 256), 256, 0, s, rows, ptr,
+                   kSplitT, kMidChunks, shape, k0, cnt));
+  const int shift = 32;
+  // stable: rows ascend per class and eighth
+  return radix_sort_u64(k0, k1, rows, &shift, 1, s, &out->sorted);
+}
+
+int plan_fill(std::vector<void*>* owned, const int32_t* ptr, int32_t rows, const PlanShape& shape,
+              const int32_t* idx, const int32_t* c, const PlanKeys& keys, TempPool& pool,
+              SplitPlan* plan, cudaStream_t s);
+
+}  // namespace
+
 int build_split_plan(hnv_graph* g, std::vector<void*>* owned, const int32_t* ptr, int32_t rows,
                      SplitPlan* plan, cudaStream_t s, const PlanShape& shape,
                      const int32_t* idx) {
   *plan = SplitPlan();
-  const int32_t T = plan->T;
   if (rows == 0) return HNV_OK;
   TempPool pool(s);
-  uint64_t *k0 = nullptr, *k1 = nullptr, *sorted = nullptr;
-  HNV_CHECK(pool.get(&k0, (size_t)rows));
-  HNV_CHECK(pool.get(&k1, (size_t)rows));
-  int32_t* cnt = g->d_buf;
-  HNV_CUDA(cudaMemsetAsync(cnt, 0, 16 * sizeof(int32_t), s));
-  HNV_CHECK(launch("classify_rows", classify_rows, grid_for(rows, 256), 256, 0, s, rows, ptr, T,
-                   kMidChunks, shape, k0, cnt));
-  const int shift = 32;
-  HNV_CHECK(radix_sort_u64(k0, k1, rows, &shift, 1, s, &sorted));   // stable: rows ascend per class and eighth
-  int32_t c[kClasses];
-  HNV_CHECK(read_ints(g, cnt, kClasses, c, s));
+  PlanKeys keys;
+  int32_t c[kPlanCounts];
+  HNV_CUDA(cudaMemsetAsync(g->d_buf, 0, kPlanCounts * sizeof(int32_t), s));
+  HNV_CHECK(plan_classify(ptr, rows, shape, g->d_buf, pool, &keys, s));
+  HNV_CHECK(read_ints(g, g->d_buf, kPlanCounts, c, s));
+  return plan_fill(owned, ptr, rows, shape, idx, c, keys, pool, plan, s);
+}
+
+namespace {
+
+int plan_fill(std::vector<void*>* owned, const int32_t* ptr, int32_t rows, const PlanShape& shape,
+              const int32_t* idx, const int32_t* c, const PlanKeys& keys, TempPool& pool,
+              SplitPlan* plan, cudaStream_t s) {
+  *plan = SplitPlan();
+  if (rows == 0) return HNV_OK;
+  const int32_t T = plan->T;
+  const uint64_t* sorted = keys.sorted;
   int32_t off[kClasses + 1] = {0};
   for (int i = 0; i < kClasses; ++i) off[i + 1] = off[i] + c[i];
   plan->n_zero = c[0];
@@ -347,15 +383,9 @@ int build_split_plan(hnv_graph* g, std::vector<void*>* owned, const int32_t* ptr
     HNV_CHECK(pool.get(&chunk_off, (size_t)n_long));
     HNV_CHECK(launch("long_chunk_counts", long_chunk_counts, grid_for(n_long, 256), 256, 0, s,
                      (const uint64_t*)sorted, off[5], n_long, ptr, T, chunk_off));
-    HNV_CHECK(exclusive_scan_i32(chunk_off, chunk_off, n_long, cnt + 8, s));
-    // the offset of the first row with many chunks = chunks of those before it
-    if (c[5] > 0 && c[6] > 0)
-      HNV_CUDA(cudaMemcpyAsync(cnt + 9, chunk_off + c[5], sizeof(int32_t),
-                               cudaMemcpyDeviceToDevice, s));
-    int32_t ch[2];
-    HNV_CHECK(read_ints(g, cnt + 8, 2, ch, s));
-    plan->n_chunks = ch[0];
-    plan->n_mid_chunks = c[6] == 0 ? ch[0] : (c[5] > 0 ? ch[1] : 0);
+    HNV_CHECK(exclusive_scan_i32(chunk_off, chunk_off, n_long, nullptr, s));
+    plan->n_mid_chunks = c[7];
+    plan->n_chunks = c[7] + c[8];
   }
   const int64_t n_items = (int64_t)n_rows_items + plan->n_chunks;
   if (n_items > 0)
@@ -388,6 +418,8 @@ int build_split_plan(hnv_graph* g, std::vector<void*>* owned, const int32_t* ptr
   }
   return HNV_OK;
 }
+
+}  // namespace
 
 // ---------------------------------------------------------------------------
 // Panel plans
@@ -659,10 +691,18 @@ int finish_level(hnv_graph* g, Level* lv) {
   HNV_CHECK(launch("inv_size", inv_size_kernel, grid_for(m, 256), 256, 0, s, m,
                    (const int32_t*)lv->e_ptr, lv->inv_size_e));
   HNV_CHECK(level_weight_arrays(lv, s));
-  HNV_CHECK(build_split_plan(g, &lv->owned, lv->e_ptr, m, &lv->planE, s, PlanShape(),
-                             lv->e_nodes));
-  HNV_CHECK(build_split_plan(g, &lv->owned, lv->v_ptr, n, &lv->planV, s));
-  return HNV_OK;
+  // both plans' counts in one read
+  TempPool pool(s);
+  PlanKeys ke, kv;
+  int32_t c[2 * kPlanCounts];
+  HNV_CUDA(cudaMemsetAsync(g->d_buf, 0, sizeof(c), s));
+  HNV_CHECK(plan_classify(lv->e_ptr, m, PlanShape(), g->d_buf, pool, &ke, s));
+  HNV_CHECK(plan_classify(lv->v_ptr, n, PlanShape(), g->d_buf + kPlanCounts, pool, &kv, s));
+  HNV_CHECK(read_ints(g, g->d_buf, 2 * kPlanCounts, c, s));
+  HNV_CHECK(plan_fill(&lv->owned, lv->e_ptr, m, PlanShape(), lv->e_nodes, c, ke, pool, &lv->planE,
+                      s));
+  return plan_fill(&lv->owned, lv->v_ptr, n, PlanShape(), nullptr, c + kPlanCounts, kv, pool,
+                   &lv->planV, s);
 }
 
 int build_level0(hnv_graph* g, int32_t n, int32_t m, const int64_t* d_edge_ptr,
