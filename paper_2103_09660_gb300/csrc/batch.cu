@@ -474,8 +474,8 @@ int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
   std::vector<std::vector<int>> best;
   double best_us = -1.0;
   int best_blocks = 1;
-  for (int blocks = sms; blocks >= 1; blocks /= 2) {
-    const int teams = std::min<int>(sms / blocks, (int)own.size());
+  for (int teams = 1; teams <= std::min<int>(sms, (int)own.size()); ++teams) {
+    const int blocks = sms / teams;
     std::vector<std::pair<double, int>> cost;
     for (int i : own) {
       double us = 0.0;
@@ -498,7 +498,6 @@ int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       best = deal;
       best_blocks = blocks;
     }
-    if (teams == (int)own.size()) break;
   }
   const int teams = (int)best.size();
   std::vector<TeamGraph> hg;

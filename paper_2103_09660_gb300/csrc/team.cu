@@ -608,11 +608,12 @@ int team_blocks_for(const Level& lv, int dtype, int d) {
 }
 
 double team_sweep_us(const Level& lv, int dtype, int d, int blocks) {
-  // measured on the 41K-node workload: about 10 us of dependent loads and
-  // barriers a sweep, and 80 GB/s of gathered rows per SM beyond it
+  // fitted to a batch of 64 graphs of 1K-100K nodes (d = 64, 9 blocks a
+  // team): 12 us of dependent loads and barriers a sweep, 52 GB/s of rows per
+  // SM beyond it
   const double bytes = (double)(dtype == HNV_BF16 ? 2 : 4) * d *
                        (2.0 * lv.nnz + 3.0 * ((double)lv.n + lv.m));
-  return 10.0 + bytes / (80e3 * blocks);
+  return 12.0 + bytes / (52e3 * blocks);
 }
 
 int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s) {
