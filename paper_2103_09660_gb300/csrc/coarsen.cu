@@ -109,17 +109,21 @@ __global__ void segment_mean_kernel(int32_t rows, int32_t k, const int32_t* __re
   }
 }
 
-// The listed rows, 32 dimensions a task: the block loads kMeanTile members'
-// values at a time into shared memory (the next tile's loads are out while
-// this one is added), one warp adds them in list order. A thread walking a
-// 5,000-member list alone, one dependent load after the other, took 660 us.
+// The listed rows, 32 dimensions a task: the block copies kMeanTile members'
+// values at a time into shared memory, kMeanStages - 1 tiles ahead of the
+// warp that adds them in list order (cp.async; the member IDs of a tile are
+// loaded one tile before its copies). A thread walking a 5,000-member list
+// alone, one dependent load after the other, took 660 us; tiles loaded through
+// registers, the loads of a tile exposed, 268 us.
+constexpr int kMeanStages = 3;
+
 __global__ void __launch_bounds__(kMeanThreads)
 segment_mean_long_kernel(int32_t k, const int32_t* __restrict__ ptr,
                          const int32_t* __restrict__ idx, const float* __restrict__ X,
                          float* __restrict__ out, const int32_t* __restrict__ long_rows,
                          const int32_t* __restrict__ n_long) {
-  constexpr int PER = kMeanTile * 32 / kMeanThreads;   // loads per thread and tile
-  __shared__ float tile[kMeanTile][32];
+  constexpr int W = kMeanThreads / 32, PER = kMeanTile / W;   // copies per thread and tile
+  __shared__ float tile[kMeanStages][kMeanTile][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int32_t slabs = (k + 31) / 32;
   const int64_t tasks = (int64_t)*n_long * slabs;
@@ -127,34 +131,53 @@ segment_mean_long_kernel(int32_t k, const int32_t* __restrict__ ptr,
     const int32_t r = long_rows[q / slabs];
     const int32_t col = (int32_t)(q % slabs) * 32 + lane;
     const int32_t b = ptr[r], e = ptr[r + 1];
-    float x[PER], acc = 0.f;
-    auto load = [&](int32_t j0) {
+    const int32_t tiles = (e - b + kMeanTile - 1) / kMeanTile;
+    int32_t id[PER];
+    auto ids = [&](int32_t t) {
 #pragma unroll
       for (int u = 0; u < PER; ++u) {
-        const int32_t j = j0 + w + u * (kMeanThreads / 32);
-        x[u] = j < e && col < k ? X[(size_t)idx[j] * k + col] : 0.f;
+        const int32_t j = b + t * kMeanTile + w + u * W;
+        id[u] = j < e ? idx[j] : -1;
       }
     };
-    load(b);
-    for (int32_t j0 = b; j0 < e; j0 += kMeanTile) {
-      __syncthreads();   // the adder is done with the tile
+    // copies tile t (its IDs in id) and loads the IDs of tile t + 1
+    auto copy = [&](int32_t t) {
 #pragma unroll
-      for (int u = 0; u < PER; ++u) tile[w + u * (kMeanThreads / 32)][lane] = x[u];
-      __syncthreads();
-      if (j0 + kMeanTile < e) load(j0 + kMeanTile);
+      for (int u = 0; u < PER; ++u) {
+        const uint32_t dst =
+            (uint32_t)__cvta_generic_to_shared(&tile[t % kMeanStages][w + u * W][lane]);
+        if (id[u] >= 0 && col < k)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst),
+                       "l"(X + (size_t)id[u] * k + col)
+                       : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      ids(t + 1);
+    };
+    ids(0);
+    __syncthreads();   // the adder is done with the row before
+#pragma unroll
+    for (int t = 0; t < kMeanStages - 1; ++t) copy(t);   // (empty past the row's end)
+    float acc = 0.f;
+    for (int32_t t = 0; t < tiles; ++t) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kMeanStages - 2) : "memory");
+      __syncthreads();   // tile t is there, tile t - 1 has been added
+      copy(t + kMeanStages - 1);
       if (w == 0) {
-        const int32_t cnt = min(kMeanTile, e - j0);
+        const float (*x)[32] = tile[t % kMeanStages];
+        const int32_t cnt = min(kMeanTile, e - b - t * kMeanTile);
         int32_t j = 0;
-        for (; j + 8 <= cnt; j += 8) {
-          float y[8];
+        for (; j + 16 <= cnt; j += 16) {
+          float y[16];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) y[u] = tile[j + u][lane];
+          for (int u = 0; u < 16; ++u) y[u] = x[j + u][lane];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) acc = __fadd_rn(acc, y[u]);
+          for (int u = 0; u < 16; ++u) acc = __fadd_rn(acc, y[u]);
         }
-        for (; j < cnt; ++j) acc = __fadd_rn(acc, tile[j][lane]);
+        for (; j < cnt; ++j) acc = __fadd_rn(acc, x[j][lane]);
       }
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (w == 0 && col < k) out[(size_t)r * k + col] = __fdiv_rn(acc, (float)(e - b));
   }
 }
