@@ -482,6 +482,8 @@ typedef enum {
   HNV_PHASE_ADJOINT_PROJECT = 7,  /* weight gradients out, projection reversed */
   HNV_PHASE_COUNT = 8
 } hnv_phase;
+/* While timing is on, small graphs too run a launch per half-sweep (otherwise
+ * their V-cycles are one launch); the results are the same bits. */
 int hnv_timing_enable(int enable);
 /* Clears the recorded events. */
 int hnv_timing_reset(void);

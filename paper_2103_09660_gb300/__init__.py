@@ -542,8 +542,9 @@ class Graph:
 
 
 class Batch:
-    """Many hypergraphs refined together (hnv_batch_*): one launch per row
-    class (or one persistent launch) per half-sweep covers every graph, the
+    """Many hypergraphs refined together (hnv_batch_*): small graphs are dealt
+    over teams of blocks in one launch; for the others one launch per row
+    class (or one persistent launch) per half-sweep covers every graph. The
     V-cycle is captured into a CUDA graph. The graphs must stay alive while
     the batch is used."""
 
