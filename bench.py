@@ -417,7 +417,9 @@ def _half_sweeps(csv_path):
         if "gather_packed" in name:             # the packed short rows: hyperedge side
             side = "E"
         elif "gather_kernel<" in name and "batched" not in name:
-            side = "V" if name.split("<", 1)[1].split(">", 1)[0].rstrip().endswith("1") else "E"
+            # template arguments: type, lanes, vectors, weighted (the node side), ...
+            weighted = name.split("<", 1)[1].split(">", 1)[0].split(",")[3].strip()
+            side = "V" if weighted == "1" else "E"
         elif (("finalize_kernel<" in name or "combine_kernel<" in name) and phase is not None
               and "batched" not in name):
             side = phase
