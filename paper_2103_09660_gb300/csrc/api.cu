@@ -222,7 +222,7 @@ int hnv_build_incidence(int32_t n_nodes, int32_t n_edges, const int64_t* edge_pt
       break;
     }
     if ((rc = dev_alloc((void**)&g->d_err, sizeof(int32_t), s)) != HNV_OK) break;
-    if ((rc = dev_alloc((void**)&g->d_buf, (kBufWords + kTeamWords) * sizeof(int32_t), s)) != HNV_OK) break;
+    if ((rc = dev_alloc((void**)&g->d_buf, 64 * sizeof(int32_t), s)) != HNV_OK) break;
     {
       cudaError_t e = cudaEventCreateWithFlags(&g->fork_ev, cudaEventDisableTiming);
       for (int i = 0; i < 2 && e == cudaSuccess; ++i) {

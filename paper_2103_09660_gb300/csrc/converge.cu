@@ -53,6 +53,9 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
   const Level& lv = g->levels[level];
   if (max_sweeps > 0 && team_enabled(d) && team_fits(lv, dtype, d) && team_ready(g, s)) {
     // sweeps, changes and the test in one launch (at most kTeamMaxSweeps each)
+    TempPool pool(s);
+    int32_t* words = nullptr;
+    HNV_CHECK(pool.get(&words, kTeamWords));
     int32_t done = 0, res[2] = {0, 0};
     float delta = 0.f;
     do {
@@ -61,8 +64,8 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
       t.zv0 = static_cast<uint4*>(z_v);
       t.ze0 = static_cast<uint4*>(z_e);
       const int k = max_sweeps - done < kTeamMaxSweeps ? max_sweeps - done : kTeamMaxSweeps;
-      HNV_CHECK(team_run(g, t, dtype, d, omega, k, mode, s, &eps));
-      HNV_CHECK(read_ints(g, g->d_buf + kTeamResult, 2, res, s));
+      HNV_CHECK(team_run(g, t, dtype, d, omega, k, mode, s, &eps, words));
+      HNV_CHECK(read_ints(g, words + kTeamResult, 2, res, s));
       if (res[0] <= 0) HNV_FAIL(HNV_ERR_TIMEOUT, "a bounded wait of a refinement kernel gave up");
       done += res[0];
       std::memcpy(&delta, &res[1], sizeof(float));

@@ -419,10 +419,10 @@ struct Level {
 };
 
 struct TeamLevel;
-// 32-bit words of hnv_graph::d_buf: 64 of scratch, then the team kernel's
-// barrier line, the stopping rule's 3 running maxima and its 2 results.
-constexpr int kBufWords = 64, kTeamBarrier = 64, kTeamDelta = 96, kTeamResult = 100,
-              kTeamWords = 64;
+// 32-bit words a one-graph team launch owns (calls on other streams may run
+// beside it): the barrier line, the stopping rule's 3 running maxima and its 2
+// results.
+constexpr int kTeamWords = 64, kTeamDelta = 32, kTeamResult = 36;
 
 }  // namespace hnv
 
@@ -432,7 +432,7 @@ struct hnv_graph {
   std::vector<hnv::Level> levels;
   int32_t* d_err = nullptr;      // device error word
   int32_t* h_buf = nullptr;      // pinned host scratch (64 ints)
-  int32_t* d_buf = nullptr;      // device scratch (64 ints), then the team kernel's (kTeamWords)
+  int32_t* d_buf = nullptr;      // device scratch (64 ints)
   hnv::TeamLevel* team_levels = nullptr;   // device, one per level (team.cu)
   float* partials = nullptr;     // split-row partial sums
   size_t partials_bytes = 0;
@@ -599,10 +599,10 @@ int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s);
 // an environment switch asks for another gather).
 bool team_enabled(int d);
 // Levels top .. bottom of g (all of which fit) in one launch on s.
-// With eps, the stopping rule: the sweeps done and the last change are left
-// in d_buf + kTeamResult.
+// With eps, the stopping rule: the caller brings the kTeamWords words, and
+// the sweeps done and the last change are left at words + kTeamResult.
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
-             cudaStream_t s, const float* eps = nullptr);
+             cudaStream_t s, const float* eps = nullptr, int32_t* words = nullptr);
 // Uploads the hierarchy's TeamLevels on first use (dropped with the
 // hierarchy). False where it cannot: under capture, or out of memory; the
 // caller then takes the per-launch path.

@@ -499,7 +499,9 @@ bool team_ready(hnv_graph* g, cudaStream_t s) {
 }
 
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
-             cudaStream_t s, const float* eps) {
+             cudaStream_t s, const float* eps, int32_t* words) {
+  TempPool pool(s);
+  if (!words) HNV_CHECK(pool.get(&words, kTeamWords));
   int64_t chunks = 1, m = 1;
   int blocks = 1;
   for (int l = t.bottom; l <= t.top; ++l) {
@@ -511,7 +513,7 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
   HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes, sizeof(float) * (size_t)chunks * d, s));
   if (mode == HNV_SWEEP_JACOBI)
     HNV_CHECK(ensure_scratch(&g->jacobi_tmp, &g->jacobi_bytes, elem_size(dtype) * (size_t)m * d, s));
-  HNV_CUDA(cudaMemsetAsync(g->d_buf + kBufWords, 0, sizeof(int32_t) * kTeamWords, s));
+  HNV_CUDA(cudaMemsetAsync(words, 0, sizeof(int32_t) * kTeamWords, s));
   t.levels = g->team_levels;
   t.err = g->d_err;
   t.partials = g->partials;
@@ -523,10 +525,10 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
   a.jacobi = mode == HNV_SWEEP_JACOBI;
   a.keep = 1.0f - omega;
   a.omega = omega;
-  a.barriers = reinterpret_cast<uint32_t*>(g->d_buf + kTeamBarrier);
+  a.barriers = reinterpret_cast<uint32_t*>(words);
   if (eps) {
-    a.delta = reinterpret_cast<unsigned*>(g->d_buf + kTeamDelta);
-    a.result = g->d_buf + kTeamResult;
+    a.delta = reinterpret_cast<unsigned*>(words + kTeamDelta);
+    a.result = words + kTeamResult;
     a.eps = *eps;
   }
   return team_launch(a, 1, dtype, d, s);

@@ -163,3 +163,35 @@ def test_saved_rows_gradients_and_capture(H):
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(zv, want[0]) and torch.equal(ze, want[1])
+
+
+def test_two_streams_on_one_graph(H):
+    """Calls on two streams may run beside each other (no split rows, so they
+    share no scratch): each launch has its own barrier words."""
+    import torch
+    hg = _hub_graph(40, [])
+    keep = [e for e in range(hg.m) if hg.edge_ptr[e + 1] - hg.edge_ptr[e] <= 128]
+    edges = [hg.edge_nodes[hg.edge_ptr[e]:hg.edge_ptr[e + 1]] for e in keep]
+    ptr = np.concatenate([[0], np.cumsum([len(e) for e in edges])]).astype(np.int64)
+    with H.Graph(hg.n, len(edges), ptr, np.concatenate(edges).astype(np.int32)) as G:
+        z = torch.randn((2, hg.n + len(edges), 16), device="cuda")
+
+        def run(k, stream):
+            v, e = z[k, :hg.n].clone(), z[k, hg.n:].clone()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                H.hnv_refine(G.handle, 0, v, e, 0.3, 400, H.SWEEP_TWO_PHASE, stream)
+            return v, e
+        s = [torch.cuda.Stream(), torch.cuda.Stream()]
+        want = []
+        for k in range(2):
+            want.append(run(k, s[0]))
+            torch.cuda.synchronize()
+        pairs = [(z[k, :hg.n].clone(), z[k, hg.n:].clone()) for k in range(2)]
+        torch.cuda.synchronize()
+        for k in range(2):
+            H.hnv_refine(G.handle, 0, pairs[k][0], pairs[k][1], 0.3, 400, H.SWEEP_TWO_PHASE, s[k])
+        torch.cuda.synchronize()
+        G.sync_status()
+        for k in range(2):
+            assert torch.equal(pairs[k][0], want[k][0]) and torch.equal(pairs[k][1], want[k][1])
