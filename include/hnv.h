@@ -440,6 +440,19 @@ int hnv_sync_status(hnv_graph* g, hnv_stream_t stream);
  * Errors: HNV_ERR_INVALID_ARG (NULL graph, limit out of range), HNV_ERR_CUDA. */
 int hnv_selftest_wait_timeout(hnv_graph* g, uint32_t limit_us, hnv_stream_t stream);
 
+/* Self-test of the one-launch path's failure handling (a library service; the
+ * paper has no counterpart). Small levels run many sweeps in one launch, with
+ * bounded barriers between the half-sweeps. After this call barrier number
+ * `barrier` (counted from 1) of each such launch on the graph waits for an
+ * arrival that never comes, and every barrier wait of the graph gives up
+ * after limit_us microseconds (1 .. 1000000); the launch then ends and the
+ * timeout is reported as that of a real failure is: hnv_refine_until returns
+ * HNV_ERR_TIMEOUT, the asynchronous calls leave it to hnv_sync_status.
+ * barrier = 0 restores the normal waits (limit_us is not read). A batch takes
+ * the setting of its graphs when it builds its work lists. Not a device
+ * operation. Errors: HNV_ERR_INVALID_ARG. */
+int hnv_selftest_team_timeout(hnv_graph* g, int32_t barrier, uint32_t limit_us);
+
 /* Releases the hierarchy (stream-ordered on the graph's stream). NULL is a no-op. */
 void hnv_graph_free(hnv_graph* g);
 

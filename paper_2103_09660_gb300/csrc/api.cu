@@ -653,6 +653,17 @@ int hnv_selftest_wait_timeout(hnv_graph* g, uint32_t limit_us, hnv_stream_t stre
                        reinterpret_cast<cudaStream_t>(stream));
 }
 
+int hnv_selftest_team_timeout(hnv_graph* g, int32_t barrier, uint32_t limit_us) {
+  clear_error_detail();
+  if (!g) HNV_FAIL(HNV_ERR_INVALID_ARG, "graph is NULL");
+  if (barrier < 0) HNV_FAIL(HNV_ERR_INVALID_ARG, "barrier < 0");
+  if (barrier > 0 && (limit_us < 1 || limit_us > 1000000))
+    HNV_FAIL(HNV_ERR_INVALID_ARG, "limit_us = %u: need 1 .. 1000000", limit_us);
+  g->team_stop_at = barrier;
+  g->team_wait_ns = barrier > 0 ? (uint64_t)limit_us * 1000ull : kTeamWaitNs;
+  return HNV_OK;
+}
+
 void hnv_graph_free(hnv_graph* g) {
   if (!g) return;
   DeviceGuard dgd(g->device);

@@ -523,6 +523,8 @@ int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       t.zv0 = (uint4*)(zv0 + (size_t)b->v_off[i] * rb);
       t.ze0 = (uint4*)(ze0 + (size_t)b->e_off[i] * rb);
       t.err = g->d_err;
+      t.wait_ns = g->team_wait_ns;
+      t.stop_at = g->team_stop_at;
       hg.push_back(t);
     }
     first.push_back((int32_t)hg.size());

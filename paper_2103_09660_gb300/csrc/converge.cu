@@ -56,7 +56,7 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
     TempPool pool(s);
     int32_t* words = nullptr;
     HNV_CHECK(pool.get(&words, kTeamWords));
-    int32_t done = 0, res[2] = {0, 0};
+    int32_t done = 0, res[3] = {0, 0, 0};
     float delta = 0.f;
     do {
       TeamGraph t;
@@ -65,8 +65,9 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
       t.ze0 = static_cast<uint4*>(z_e);
       const int k = max_sweeps - done < kTeamMaxSweeps ? max_sweeps - done : kTeamMaxSweeps;
       HNV_CHECK(team_run(g, t, dtype, d, omega, k, mode, s, &eps, words));
-      HNV_CHECK(read_ints(g, words + kTeamResult, 2, res, s));
-      if (res[0] <= 0) HNV_FAIL(HNV_ERR_TIMEOUT, "a bounded wait of a refinement kernel gave up");
+      HNV_CHECK(read_ints(g, words + kTeamResult, 3, res, s));
+      // in whichever sweep: the rows are then half-written
+      if (res[2]) HNV_FAIL(HNV_ERR_TIMEOUT, "a bounded wait of a refinement kernel gave up");
       done += res[0];
       std::memcpy(&delta, &res[1], sizeof(float));
     } while (done < max_sweeps && !(delta <= eps));

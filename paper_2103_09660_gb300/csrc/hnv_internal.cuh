@@ -419,8 +419,10 @@ struct Level {
 };
 
 struct TeamLevel;
+// Limit of one barrier wait of the team kernel.
+constexpr uint64_t kTeamWaitNs = 4000000000ull;
 // 32-bit words a one-graph team launch owns (calls on other streams may run
-// beside it): the barrier line, the stopping rule's 3 running maxima and its 2
+// beside it): the barrier line, the stopping rule's 3 running maxima and its 3
 // results.
 constexpr int kTeamWords = 64, kTeamDelta = 32, kTeamResult = 36;
 
@@ -434,6 +436,9 @@ struct hnv_graph {
   int32_t* h_buf = nullptr;      // pinned host scratch (64 ints)
   int32_t* d_buf = nullptr;      // device scratch (64 ints)
   hnv::TeamLevel* team_levels = nullptr;   // device, one per level (team.cu)
+  // hnv_selftest_team_timeout: of the one-launch calls' barriers
+  uint64_t team_wait_ns = hnv::kTeamWaitNs;
+  int32_t team_stop_at = 0;
   float* partials = nullptr;     // split-row partial sums
   size_t partials_bytes = 0;
   float* jacobi_tmp = nullptr;   // Jacobi: next hyperedge rows
@@ -565,6 +570,8 @@ struct TeamGraph {
   uint4* jtmp = nullptr;               // Jacobi: m rows of the largest level
   uint4* ckpt = nullptr;               // every level's starting rows, or null
   int32_t* err = nullptr;              // the graph's error word
+  uint64_t wait_ns = kTeamWaitNs;      // limit of a barrier wait
+  int32_t stop_at = 0;                 // self-test: the barrier that is never complete, or 0
 };
 
 struct TeamArgs {
@@ -576,7 +583,8 @@ struct TeamArgs {
   float keep = 0.f, omega = 0.f;
   uint32_t* barriers = nullptr;        // 32 words per team, zeroed before the launch
   // stopping rule (result != null): delta holds 3 words, zeroed before the
-  // launch; result receives {sweeps done, bits of the last largest change}
+  // launch; result (zeroed too) receives {sweeps done, bits of the last largest
+  // change, ERRBIT_TIMEOUT if a wait gave up}
   unsigned* delta = nullptr;
   int32_t* result = nullptr;
   float eps = 0.f;
@@ -600,7 +608,8 @@ int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s);
 bool team_enabled(int d);
 // Levels top .. bottom of g (all of which fit) in one launch on s.
 // With eps, the stopping rule: the caller brings the kTeamWords words, and
-// the sweeps done and the last change are left at words + kTeamResult.
+// the sweeps done, the last change and whether a wait gave up are left at words
+// + kTeamResult.
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
              cudaStream_t s, const float* eps = nullptr, int32_t* words = nullptr);
 // Uploads the hierarchy's TeamLevels on first use (dropped with the

@@ -516,6 +516,8 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
   HNV_CUDA(cudaMemsetAsync(words, 0, sizeof(int32_t) * kTeamWords, s));
   t.levels = g->team_levels;
   t.err = g->d_err;
+  t.wait_ns = g->team_wait_ns;
+  t.stop_at = g->team_stop_at;
   t.partials = g->partials;
   t.jtmp = reinterpret_cast<uint4*>(g->jacobi_tmp);
   TeamArgs a;

@@ -40,7 +40,9 @@
 // Rows written in one step are read in the next by other blocks, so row and
 // partial loads are plain (never the read-only path); the barrier's
 // acquire/release pair orders them. Every wait is bounded: a block that gives
-// up records ERRBIT_TIMEOUT and returns, and so does the rest of its team.
+// up records ERRBIT_TIMEOUT and returns, and so does the rest of its team. It
+// goes to the graph's error word (read by hnv_sync_status), or, with the
+// stopping rule, to the launch's own result, which that call reads anyway.
 #include <algorithm>
 #include <cstring>
 
@@ -54,7 +56,6 @@ using dev::VecT;
 
 constexpr int kTeamThreads = 512;
 constexpr int kTeamWarps = kTeamThreads / 32;
-constexpr uint64_t kBarrierLimitNs = 4000000000ull;   // of one barrier wait
 constexpr int kFinSlots = 1024;   // (slice, vector) pairs of a split row's reduction, as in
                                   // finalize_kernel's 1,024-thread blocks
 
@@ -65,30 +66,35 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // A barrier among the `blocks` blocks that share `counter` (0 at launch).
-// False once a wait gave up (the whole block sees the same answer).
+// False once a wait gave up (the whole block sees the same answer). A wait is
+// limited to g->wait_ns; the barrier at target *stop waits for one arrival
+// more than comes (TeamGraph::stop_at).
 struct TeamBarrier {
   uint32_t* counter;
   uint32_t blocks;
   uint32_t target;
   int32_t* err;
-  int* dead;   // shared memory
+  int* dead;             // shared memory, as g and stop
+  const TeamGraph* g;
+  const uint32_t* stop;
 
   __device__ __forceinline__ bool wait() {
     __syncthreads();
     if (threadIdx.x == 0) {
       target += blocks;
+      const uint32_t want = target == *stop ? target + 1 : target;
       asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
       uint64_t t0 = 0;
       int spins = 0;
       for (;;) {
         uint32_t v;
         asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-        if ((int32_t)(v - target) >= 0) break;
+        if ((int32_t)(v - want) >= 0) break;
         if ((++spins & 1023) == 0) {
           const uint64_t now = global_ns();
           if (t0 == 0) {
             t0 = now;
-          } else if (now - t0 > kBarrierLimitNs) {
+          } else if (now - t0 > g->wait_ns) {
             *dead = 1;
             atomicOr(err, (int32_t)ERRBIT_TIMEOUT);
             break;
@@ -467,19 +473,23 @@ template <typename T, int G, int VPL, bool DIFF>
 __global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(const TeamArgs a) {
   __shared__ __align__(16) float sm[kFinSlots * VecT<T>::N];
   __shared__ int dead;
+  __shared__ uint32_t stop;
   __shared__ TeamGraph g;
   if (threadIdx.x == 0) dead = 0;
   const int team = blockIdx.x / a.blocks, block = blockIdx.x - team * a.blocks;
   const int warp = (threadIdx.x >> 5) * a.blocks + block, warps = kTeamWarps * a.blocks;
   const int64_t thread = (int64_t)warp * 32 + (threadIdx.x & 31), threads = (int64_t)warps * 32;
-  TeamBarrier bar{a.barriers + 32 * team, (uint32_t)a.blocks, 0u, nullptr, &dead};
+  TeamBarrier bar{a.barriers + 32 * team, (uint32_t)a.blocks, 0u, nullptr, &dead, &g, &stop};
   const int32_t q0 = a.graphs ? a.team_first[team] : 0, q1 = a.graphs ? a.team_first[team + 1] : 1;
   const int dv = a.dv;
   for (int32_t q = q0; q < q1; ++q) {
     __syncthreads();
-    if (threadIdx.x == 0) g = a.graphs ? a.graphs[q] : a.one;
+    if (threadIdx.x == 0) {
+      g = a.graphs ? a.graphs[q] : a.one;
+      stop = g.stop_at > 0 ? bar.target + (uint32_t)g.stop_at * bar.blocks : 0u;
+    }
     __syncthreads();
-    bar.err = g.err;
+    bar.err = DIFF ? a.result + 2 : g.err;
     for (int l = g.top; l >= g.bottom; --l) {
       const TeamLevel& lv = g.levels[l];
       uint4* zv = l == g.bottom ? g.zv0 : g.buf[l & 1];

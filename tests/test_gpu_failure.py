@@ -85,3 +85,55 @@ def test_release_cached_memory_keeps_graphs_working(H):
         G.vcycle(zc, zv, ze, 0.5, 3)                      # allocates afresh
         torch.cuda.synchronize()
         assert torch.equal(a[0], zv) and torch.equal(a[1], ze)
+
+
+def _no_split_rows():
+    """A small hypergraph whose rows all have at most 128 incidences (so that a
+    sweep of the one-launch path has two barriers)."""
+    rng = np.random.default_rng(4)
+    return hypergen.random_small_hypergraph(rng, 400, 300, 6)
+
+
+# barrier 1 starts the first sweep; sweep k ends at barrier 1 + 2 k
+@pytest.mark.parametrize("barrier", [1, 2, 6, 7])
+def test_stopping_rule_reports_a_barrier_that_gave_up(H, barrier):
+    """A barrier of the one-launch path runs out, before the first sweep ends or
+    after some have: the call returns HNV_ERR_TIMEOUT either way, and leaves
+    nothing for hnv_sync_status to report again."""
+    import torch
+    hg = _no_split_rows()
+    L = H.lib()
+    with H.Graph.from_hypergraph(hg) as G:
+        z = torch.randn((hg.n + hg.m, 32), device="cuda")
+
+        def until():
+            v, e = z[:hg.n].clone(), z[hg.n:].clone()
+            return v, e, G.refine_until(0, v, e, 0.5, 8, -1.0)
+        want = until()
+        assert L.hnv_selftest_team_timeout(G.handle, barrier, 2000) == 0
+        with pytest.raises(H.HNVError) as ei:
+            until()
+        assert ei.value.code == -6
+        G.sync_status()
+        assert L.hnv_selftest_team_timeout(G.handle, 0, 0) == 0
+        got = until()
+        assert got[2] == want[2] and got[2][0] == 8
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+def test_asynchronous_calls_leave_a_barrier_that_gave_up_to_sync_status(H):
+    import torch
+    hg = _no_split_rows()
+    L = H.lib()
+    with H.Graph.from_hypergraph(hg) as G:
+        z = torch.randn((hg.n + hg.m, 32), device="cuda")
+        assert L.hnv_selftest_team_timeout(G.handle, 4, 2000) == 0
+        G.refine(0, z[:hg.n], z[hg.n:], 0.5, 8)
+        with pytest.raises(H.HNVError) as ei:
+            G.sync_status()
+        assert ei.value.code == -6
+        G.sync_status()
+        assert L.hnv_selftest_team_timeout(G.handle, -1, 2000) == -1
+        assert L.hnv_selftest_team_timeout(G.handle, 1, 0) == -1
+        assert L.hnv_selftest_team_timeout(G.handle, 1, 1_000_001) == -1
+        assert L.hnv_selftest_team_timeout(None, 1, 2000) == -1
