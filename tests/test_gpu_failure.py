@@ -137,3 +137,34 @@ def test_asynchronous_calls_leave_a_barrier_that_gave_up_to_sync_status(H):
         assert L.hnv_selftest_team_timeout(G.handle, 1, 0) == -1
         assert L.hnv_selftest_team_timeout(G.handle, 1, 1_000_001) == -1
         assert L.hnv_selftest_team_timeout(None, 1, 2000) == -1
+
+
+def test_a_team_that_gives_up_reports_every_graph_it_did_not_run(H):
+    """More graphs than SMs, so that some teams run several: a barrier that
+    runs out in a team's first graph leaves the later ones without results, and
+    each of them says so."""
+    import torch
+    L = H.lib()
+    count = torch.cuda.get_device_properties(0).multi_processor_count + 8
+    rng = np.random.default_rng(6)
+    Gs = [H.Graph.from_hypergraph(hypergen.random_small_hypergraph(rng, 40, 30, 5))
+          for _ in range(count)]
+
+    def run():
+        with H.Batch(Gs) as B:
+            co, vo, eo = (int(a[-1]) for a in B.offsets())
+            B.vcycle(torch.ones((co, 8), device="cuda"), torch.empty((vo, 8), device="cuda"),
+                     torch.empty((eo, 8), device="cuda"), 0.5, 3)
+            torch.cuda.synchronize()
+        codes = []
+        for G in Gs:
+            codes.append(L.hnv_sync_status(G.handle, H._stream_handle(G.stream)))
+        return codes
+    for G in Gs:
+        assert L.hnv_selftest_team_timeout(G.handle, 3, 2000) == 0
+    assert run() == [-6] * count
+    for G in Gs:
+        assert L.hnv_selftest_team_timeout(G.handle, 0, 0) == 0
+    assert run() == [0] * count
+    for G in Gs:
+        G.close()
