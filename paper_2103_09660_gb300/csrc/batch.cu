@@ -339,22 +339,13 @@ int next_pow2(int x) {
 
 using namespace hnv;
 
-struct hnv_batch {
-  std::vector<hnv_graph*> graphs;
-  std::vector<uint64_t> generation;   // each graph's hierarchy generation at creation
-  int device = 0;
-  cudaStream_t cap_stream = nullptr;
-  // side streams: a half-sweep's row classes run concurrently (see enqueue_half)
-  cudaStream_t aux[2] = {nullptr, nullptr};
-  cudaEvent_t fork_ev = nullptr;
-  cudaEvent_t used_ev = nullptr;   // after the last V-cycle (what it used is freed after it)
-  bool used = false;
-  cudaEvent_t join_ev[2] = {nullptr, nullptr};
-  std::vector<int> top;            // coarsest level of each graph
-  std::vector<int> step_top;       // the same, -1 for a graph the teams run
-  int Lmax = 0, step_lmax = -1;    // deepest level of all graphs, of the step lists
-  PlanShape shape;
-  int lanes[3] = {0, 0, 0};        // lanes per row of classes A, B, rest (0: default)
+// Which graphs the teams run, and all that is built for that: plans, work
+// lists for one (dtype, d, buffers) and the captured V-cycle. A batch keeps two,
+// so that a call that takes the other one (more sweeps than a team's launch
+// runs, the other kernel) leaves what was built for these pointers in place.
+struct BatchDeal {
+  std::vector<int> step_top;       // coarsest level of each graph, -1 for one the teams run
+  int step_lmax = -1;              // deepest level of the step lists
   // per-graph plans for `shape`: plans[side][graph][level]
   std::vector<std::vector<SplitPlan>> plans[2];
   std::vector<void*> plan_owned;
@@ -369,7 +360,6 @@ struct hnv_batch {
   const void* built_zc = nullptr;
   const void* built_zv = nullptr;
   const void* built_ze = nullptr;
-  int built_kernel = -1;
   // the teams' graphs (device, in team order) and barrier words
   TeamArgs team;
   int teams = 0;
@@ -379,6 +369,25 @@ struct hnv_batch {
   int exec_sweeps = -1;
   int64_t exec_kernels = 0;        // kernel nodes of the captured V-cycle
   int exec_kernel = -1;            // the half-sweep kernel it was captured with
+};
+
+struct hnv_batch {
+  std::vector<hnv_graph*> graphs;
+  std::vector<uint64_t> generation;   // each graph's hierarchy generation at creation
+  int device = 0;
+  cudaStream_t cap_stream = nullptr;
+  // side streams: a half-sweep's row classes run concurrently (see enqueue_half)
+  cudaStream_t aux[2] = {nullptr, nullptr};
+  cudaEvent_t fork_ev = nullptr;
+  cudaEvent_t used_ev = nullptr;   // after the last V-cycle (what it used is freed after it)
+  bool used = false;
+  cudaEvent_t join_ev[2] = {nullptr, nullptr};
+  std::vector<int> top;            // coarsest level of each graph
+  int Lmax = 0;                    // deepest level of all graphs
+  PlanShape shape;
+  int lanes[3] = {0, 0, 0};        // lanes per row of classes A, B, rest (0: default)
+  // [0] small graphs run by teams, [1] every graph in the step lists
+  BatchDeal deal[2];
   // half-sweep kernel: 0 one launch per row class, 1 one persistent launch
   int kernel = HNV_BATCH_KERNEL_PER_CLASS;
   // task counters of the persistent launches, one per half-sweep of a V-cycle
@@ -404,71 +413,100 @@ int alloc_into(std::vector<void*>& owned, void** p, size_t bytes, cudaStream_t s
   return HNV_OK;
 }
 
+void free_steps(const hnv_batch* b, BatchDeal& D, cudaStream_t s) {
+  if (b->used) cudaStreamWaitEvent(s, b->used_ev, 0);
+  free_list(D.step_owned, s);
+  D.steps.clear();
+  D.partials = nullptr;
+  D.arena[0] = D.arena[1] = nullptr;
+  D.built_dt = D.built_d = -1;
+  D.teams = 0;
+  if (D.exec) {
+    cudaGraphExecDestroy(D.exec);
+    D.exec = nullptr;
+  }
+}
+
+// Everything built for a deal is dropped.
+void drop_deal(const hnv_batch* b, BatchDeal& D, cudaStream_t s) {
+  free_steps(b, D, s);
+  free_list(D.plan_owned, s);
+  D.plans_ready = false;
+}
+
+// The deal a call takes. The teams run the graphs all of whose levels are
+// small, with the per-class setting and at most kTeamMaxSweeps sweeps.
+BatchDeal& pick_deal(hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
+  std::vector<int> top = b->top;
+  bool any = false;
+  if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && team_enabled(d) && sweeps <= kTeamMaxSweeps)
+    for (size_t i = 0; i < b->graphs.size(); ++i) {
+      bool fits = true;
+      for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
+      if (!fits || !team_ready(b->graphs[i], s)) continue;
+      top[i] = -1;
+      any = true;
+    }
+  BatchDeal& D = b->deal[any ? 0 : 1];
+  if (D.step_top != top) {
+    drop_deal(b, D, s);
+    D.step_top = top;
+    D.step_lmax = -1;
+    for (int t : top) D.step_lmax = std::max(D.step_lmax, t);
+  }
+  return D;
+}
+
 // Row-class plans of every graph and level. Where the single-graph path
 // cuts long rows into panels (a neighbour table far larger than L2), the
 // batch builds the same panel plan from the level's own regular plan, so
 // both sum every row in the same order; elsewhere it uses its tuned shape.
-int build_plans(hnv_batch* b, size_t row_bytes, cudaStream_t s, int only_level = -1) {
+int build_plans(hnv_batch* b, BatchDeal& D, size_t row_bytes, cudaStream_t s,
+                int only_level = -1) {
   BTRACE("build_plans row_bytes=%zu only_level=%d", row_bytes, only_level);
+  D.plans_ready = false;   // (also where building them fails)
   if (b->used) cudaStreamWaitEvent(s, b->used_ev, 0);
-  free_list(b->plan_owned, s);
-  for (int side = 0; side < 2; ++side) b->plans[side].assign(b->graphs.size(), {});
+  free_list(D.plan_owned, s);
+  for (int side = 0; side < 2; ++side) D.plans[side].assign(b->graphs.size(), {});
   for (size_t i = 0; i < b->graphs.size(); ++i) {
     hnv_graph* g = b->graphs[i];
-    const int L = b->step_top[i] + 1;   // none for a team's graph
-    for (int side = 0; side < 2; ++side) b->plans[side][i].assign(L, SplitPlan());
+    const int L = D.step_top[i] + 1;   // none for a team's graph
+    for (int side = 0; side < 2; ++side) D.plans[side][i].assign(L, SplitPlan());
     for (int l = 0; l < L; ++l) {
       if (only_level >= 0 && l != only_level) continue;
       Level& lv = g->levels[l];
       for (int side = 0; side < 2; ++side) {
         const int32_t rows = side == 0 ? lv.m : lv.n, cols = side == 0 ? lv.n : lv.m;
         const int32_t* ptr = side == 0 ? lv.e_ptr : lv.v_ptr;
-        SplitPlan& out = b->plans[side][i][l];
+        SplitPlan& out = D.plans[side][i][l];
         int P = 1;
         if (rows > 0 && cols > 0)
-          HNV_CHECK(build_panel_plan(g, &b->plan_owned, side == 0 ? lv.planE : lv.planV, ptr,
+          HNV_CHECK(build_panel_plan(g, &D.plan_owned, side == 0 ? lv.planE : lv.planV, ptr,
                                      side == 0 ? lv.e_nodes : lv.v_edges, cols,
                                      (int64_t)cols * (int64_t)row_bytes, &out, &P, s));
-        if (P <= 1) HNV_CHECK(build_split_plan(g, &b->plan_owned, ptr, rows, &out, s, b->shape));
+        if (P <= 1) HNV_CHECK(build_split_plan(g, &D.plan_owned, ptr, rows, &out, s, b->shape));
         BTRACE("plan graph %zu level %d side %d: P=%d a=%d b=%d c=%d d=%d chunks=%d mid=%d huge=%d",
                i, l, side, P, out.n_a, out.n_b, out.n_c, out.n_d, out.n_chunks, out.n_mid,
                out.n_huge);
       }
     }
   }
-  b->plans_ready = only_level < 0;
-  b->plans_row_bytes = row_bytes;
+  D.plans_ready = only_level < 0;
+  D.plans_row_bytes = row_bytes;
   return HNV_OK;
-}
-
-// Which graphs the teams run: every level small, and the per-class setting.
-// Returns whether that changed (plans and steps are then stale).
-bool choose_teams(hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
-  std::vector<int> top = b->top;
-  if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && team_enabled(d) && sweeps <= kTeamMaxSweeps)
-    for (size_t i = 0; i < b->graphs.size(); ++i) {
-      bool fits = true;
-      for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
-      if (fits && team_ready(b->graphs[i], s)) top[i] = -1;
-    }
-  if (top == b->step_top) return false;
-  b->step_top = top;
-  b->step_lmax = -1;
-  for (int t : top) b->step_lmax = std::max(b->step_lmax, t);
-  return true;
 }
 
 // Deals the teams' graphs (longest first, each to the team with the least
 // work so far) over the number of teams with the shortest longest team, and
 // uploads their descriptors. Row buffers and partials belong to a team, so
 // that its next graph finds them in L2.
-int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, uint8_t* ze0,
+int build_teams(const hnv_batch* b, BatchDeal& D, int dt, int d, const uint8_t* zc, uint8_t* zv0, uint8_t* ze0,
                 cudaStream_t s) {
   const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
   std::vector<int> own;
   for (size_t i = 0; i < b->graphs.size(); ++i)
-    if (b->step_top[i] < 0) own.push_back((int)i);
-  b->teams = 0;
+    if (D.step_top[i] < 0) own.push_back((int)i);
+  D.teams = 0;
   if (own.empty()) return HNV_OK;
   const int sms = num_sms();
   std::vector<std::vector<int>> best;
@@ -513,8 +551,8 @@ int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       }
     TeamGraph t;
     for (int k = 0; k < 2 && rows > 0; ++k)
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&t.buf[k], rows * rb, s));
-    HNV_CHECK(alloc_into(b->step_owned, (void**)&t.partials, sizeof(float) * (size_t)chunks * d, s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&t.buf[k], rows * rb, s));
+    HNV_CHECK(alloc_into(D.step_owned, (void**)&t.partials, sizeof(float) * (size_t)chunks * d, s));
     for (int i : list) {
       const hnv_graph* g = b->graphs[i];
       t.levels = g->team_levels;
@@ -531,70 +569,56 @@ int build_teams(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
   }
   TeamGraph* dg = nullptr;
   int32_t* df = nullptr;
-  b->team = TeamArgs();
-  HNV_CHECK(alloc_into(b->step_owned, (void**)&dg, sizeof(TeamGraph) * hg.size(), s));
-  HNV_CHECK(alloc_into(b->step_owned, (void**)&df, sizeof(int32_t) * first.size(), s));
-  HNV_CHECK(alloc_into(b->step_owned, (void**)&b->team.barriers, sizeof(uint32_t) * 32 * teams, s));
+  D.team = TeamArgs();
+  HNV_CHECK(alloc_into(D.step_owned, (void**)&dg, sizeof(TeamGraph) * hg.size(), s));
+  HNV_CHECK(alloc_into(D.step_owned, (void**)&df, sizeof(int32_t) * first.size(), s));
+  HNV_CHECK(alloc_into(D.step_owned, (void**)&D.team.barriers, sizeof(uint32_t) * 32 * teams, s));
   HNV_CUDA(cudaMemcpyAsync(dg, hg.data(), sizeof(TeamGraph) * hg.size(), cudaMemcpyHostToDevice, s));
   HNV_CUDA(cudaMemcpyAsync(df, first.data(), sizeof(int32_t) * first.size(), cudaMemcpyHostToDevice, s));
   HNV_CUDA(cudaStreamSynchronize(s));   // the host vectors die here
-  b->team.graphs = dg;
-  b->team.team_first = df;
-  b->team.blocks = best_blocks;
-  b->teams = teams;
+  D.team.graphs = dg;
+  D.team.team_first = df;
+  D.team.blocks = best_blocks;
+  D.teams = teams;
   return HNV_OK;
-}
-
-void free_steps(hnv_batch* b, cudaStream_t s) {
-  if (b->used) cudaStreamWaitEvent(s, b->used_ev, 0);
-  free_list(b->step_owned, s);
-  b->steps.clear();
-  b->partials = nullptr;
-  b->arena[0] = b->arena[1] = nullptr;
-  b->built_dt = b->built_d = -1;
-  b->teams = 0;
-  if (b->exec) {
-    cudaGraphExecDestroy(b->exec);
-    b->exec = nullptr;
-  }
 }
 
 // Work lists, pointer tables and buffers of every step for (dt, d) and the
 // caller's buffers. `only_step` >= 0 builds that step only (the autotuner
 // times step 0).
-int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, uint8_t* ze0,
-                cudaStream_t s, int only_step = -1) {
-  BTRACE("build_steps dt=%d d=%d only_step=%d Lmax=%d", dt, d, only_step, b->step_lmax);
-  free_steps(b, s);
+int build_steps(const hnv_batch* b, BatchDeal& D, int dt, int d, const uint8_t* zc, uint8_t* zv0,
+                uint8_t* ze0, cudaStream_t s, int only_step = -1) {
+  BTRACE("build_steps dt=%d d=%d only_step=%d Lmax=%d", dt, d, only_step, D.step_lmax);
+  free_steps(b, D, s);
   const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
   const int32_t dv = (int32_t)(rb / 16);
   const size_t G = b->graphs.size();
-  b->steps.assign(b->step_lmax + 1, BStep());
+  D.steps.assign(D.step_lmax + 1, BStep());
   // arenas for levels >= 1 (parity of the level)
   size_t arena_rows = 0;
-  for (int st = 1; st <= b->step_lmax; ++st) {
+  for (int st = 1; st <= D.step_lmax; ++st) {
     size_t rows = 0;
     for (size_t i = 0; i < G; ++i)
-      if (b->step_top[i] >= st) rows += (size_t)b->graphs[i]->levels[st].n + b->graphs[i]->levels[st].m;
+      if (D.step_top[i] >= st) rows += (size_t)b->graphs[i]->levels[st].n + b->graphs[i]->levels[st].m;
     arena_rows = std::max(arena_rows, rows);
   }
   if (arena_rows > 0 && only_step != 0) {
-    HNV_CHECK(alloc_into(b->step_owned, (void**)&b->arena[0], arena_rows * rb, s));
-    HNV_CHECK(alloc_into(b->step_owned, (void**)&b->arena[1], arena_rows * rb, s));
+    HNV_CHECK(alloc_into(D.step_owned, (void**)&D.arena[0], arena_rows * rb, s));
+    HNV_CHECK(alloc_into(D.step_owned, (void**)&D.arena[1], arena_rows * rb, s));
   }
   // row pointers of graph i at level st
-  std::vector<std::vector<uint8_t*>> zvp(b->step_lmax + 1, std::vector<uint8_t*>(G, nullptr));
+  std::vector<std::vector<uint8_t*>> zvp(D.step_lmax + 1, std::vector<uint8_t*>(G, nullptr));
   std::vector<std::vector<uint8_t*>> zep = zvp;
-  for (int st = 0; st <= b->step_lmax; ++st) {
+  for (int st = 0; st <= D.step_lmax; ++st) {
     size_t off = 0;
     for (size_t i = 0; i < G; ++i) {
-      if (b->step_top[i] < st) continue;
+      if (D.step_top[i] < st) continue;
       const Level& lv = b->graphs[i]->levels[st];
       if (st == 0) {
         zvp[st][i] = zv0 + (size_t)b->v_off[i] * rb;
         zep[st][i] = ze0 + (size_t)b->e_off[i] * rb;
       } else {
-        zvp[st][i] = b->arena[st & 1] + off * rb;
+        zvp[st][i] = D.arena[st & 1] + off * rb;
         zep[st][i] = zvp[st][i] + (size_t)lv.n * rb;
         off += (size_t)lv.n + lv.m;
       }
@@ -602,18 +626,18 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
   }
   // partials: the largest step-side total
   size_t max_chunks = 1;
-  for (int st = 0; st <= b->step_lmax; ++st)
+  for (int st = 0; st <= D.step_lmax; ++st)
     for (int side = 0; side < 2; ++side) {
       size_t c = 0;
       for (size_t i = 0; i < G; ++i)
-        if (b->step_top[i] >= st) c += b->plans[side][i][st].n_chunks;
+        if (D.step_top[i] >= st) c += D.plans[side][i][st].n_chunks;
       max_chunks = std::max(max_chunks, c);
     }
-  HNV_CHECK(alloc_into(b->step_owned, (void**)&b->partials, max_chunks * sizeof(float) * d, s));
+  HNV_CHECK(alloc_into(D.step_owned, (void**)&D.partials, max_chunks * sizeof(float) * d, s));
 
-  for (int st = 0; st <= b->step_lmax; ++st) {
+  for (int st = 0; st <= D.step_lmax; ++st) {
     if (only_step >= 0 && st != only_step) continue;
-    BStep& S = b->steps[st];
+    BStep& S = D.steps[st];
     for (int side = 0; side < 2; ++side) {
       BSide& B = S.side[side];
       B.weighted = side == 1;
@@ -621,9 +645,9 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       B.n_graphs = (int32_t)G;
       int64_t n_items = 0, n_long = 0, chunk_base = 0;
       for (size_t i = 0; i < G; ++i) {
-        if (b->step_top[i] < st) continue;
+        if (D.step_top[i] < st) continue;
         const Level& lv = b->graphs[i]->levels[st];
-        const SplitPlan& p = b->plans[side][i][st];
+        const SplitPlan& p = D.plans[side][i][st];
         GraphSide& gs = hs[i];
         if (side == 0) {
           gs.idx = lv.e_nodes;
@@ -645,17 +669,17 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
         gs.nnz = lv.nnz;
         gs.n_slots = p.n_chunks;
         gs.err = b->graphs[i]->d_err;
-        gs.partials = b->partials + (size_t)chunk_base * d;
+        gs.partials = D.partials + (size_t)chunk_base * d;
         chunk_base += p.n_chunks;
         n_items += (int64_t)p.n_a + p.n_b + p.n_c + p.n_d + p.n_chunks;
         n_long += (int64_t)p.n_mid + p.n_huge;
       }
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&B.sides, sizeof(GraphSide) * G, s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&B.sides, sizeof(GraphSide) * G, s));
       HNV_CUDA(cudaMemcpyAsync(B.sides, hs.data(), sizeof(GraphSide) * G, cudaMemcpyHostToDevice, s));
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&B.items, sizeof(int4) * (size_t)n_items, s));
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&B.item_g, sizeof(int32_t) * (size_t)n_items, s));
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&B.long_desc, sizeof(int4) * (size_t)n_long, s));
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&B.long_g, sizeof(int32_t) * (size_t)n_long, s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&B.items, sizeof(int4) * (size_t)n_items, s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&B.item_g, sizeof(int32_t) * (size_t)n_items, s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&B.long_desc, sizeof(int4) * (size_t)n_long, s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&B.long_g, sizeof(int32_t) * (size_t)n_long, s));
       std::vector<int32_t> hg_items, hg_long;
       hg_items.reserve(n_items);
       hg_long.reserve(n_long);
@@ -663,8 +687,8 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       for (int cls = 0; cls < 3; ++cls) {
         int64_t cls_count = 0;
         for (size_t i = 0; i < G; ++i) {
-          if (b->step_top[i] < st) continue;
-          const SplitPlan& p = b->plans[side][i][st];
+          if (D.step_top[i] < st) continue;
+          const SplitPlan& p = D.plans[side][i][st];
           int64_t first = 0, count = 0;
           if (cls == 0) { first = 0; count = p.n_a; }
           else if (cls == 1) { first = p.n_a; count = p.n_b; }
@@ -682,8 +706,8 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
       for (int part = 0; part < 2; ++part) {   // rows with few chunks first, then the rest
         int64_t cnt_part = 0;
         for (size_t i = 0; i < G; ++i) {
-          if (b->step_top[i] < st) continue;
-          const SplitPlan& p = b->plans[side][i][st];
+          if (D.step_top[i] < st) continue;
+          const SplitPlan& p = D.plans[side][i][st];
           const int64_t first = part == 0 ? 0 : p.n_mid;
           const int64_t count = part == 0 ? p.n_mid : p.n_huge;
           if (count == 0) continue;
@@ -713,9 +737,9 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
     std::vector<CopyDesc> cd;
     std::vector<int64_t> cpre{0};
     for (size_t i = 0; i < G; ++i) {
-      if (b->step_top[i] < st) continue;
+      if (D.step_top[i] < st) continue;
       const Level& lv = b->graphs[i]->levels[st];
-      if (b->step_top[i] > st) {
+      if (D.step_top[i] > st) {
         pd.push_back(ProjDesc{lv.rep_v, lv.rep_e, lv.n, lv.m, (const uint4*)zvp[st + 1][i],
                               (const uint4*)zep[st + 1][i], (uint4*)zvp[st][i],
                               (uint4*)zep[st][i]});
@@ -737,25 +761,24 @@ int build_steps(hnv_batch* b, int dt, int d, const uint8_t* zc, uint8_t* zv0, ui
     S.proj_total = ppre.back();
     S.copy_total = cpre.back();
     if (S.n_proj) {
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&S.proj, sizeof(ProjDesc) * pd.size(), s));
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&S.proj_prefix, sizeof(int64_t) * ppre.size(), s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&S.proj, sizeof(ProjDesc) * pd.size(), s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&S.proj_prefix, sizeof(int64_t) * ppre.size(), s));
       HNV_CUDA(cudaMemcpyAsync(S.proj, pd.data(), sizeof(ProjDesc) * pd.size(), cudaMemcpyHostToDevice, s));
       HNV_CUDA(cudaMemcpyAsync(S.proj_prefix, ppre.data(), sizeof(int64_t) * ppre.size(),
                                cudaMemcpyHostToDevice, s));
     }
     if (S.n_copies) {
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&S.copies, sizeof(CopyDesc) * cd.size(), s));
-      HNV_CHECK(alloc_into(b->step_owned, (void**)&S.copy_prefix, sizeof(int64_t) * cpre.size(), s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&S.copies, sizeof(CopyDesc) * cd.size(), s));
+      HNV_CHECK(alloc_into(D.step_owned, (void**)&S.copy_prefix, sizeof(int64_t) * cpre.size(), s));
       HNV_CUDA(cudaMemcpyAsync(S.copies, cd.data(), sizeof(CopyDesc) * cd.size(), cudaMemcpyHostToDevice, s));
       HNV_CUDA(cudaMemcpyAsync(S.copy_prefix, cpre.data(), sizeof(int64_t) * cpre.size(),
                                cudaMemcpyHostToDevice, s));
     }
     HNV_CUDA(cudaStreamSynchronize(s));
   }
-  if (only_step < 0) HNV_CHECK(build_teams(b, dt, d, zc, zv0, ze0, s));
-  b->built_dt = dt;
-  b->built_d = d;
-  b->built_kernel = b->kernel;
+  if (only_step < 0) HNV_CHECK(build_teams(b, D, dt, d, zc, zv0, ze0, s));
+  D.built_dt = dt;
+  D.built_d = d;
   return HNV_OK;
 }
 
@@ -921,24 +944,25 @@ int ensure_counters(hnv_batch* b, int64_t n, cudaStream_t s, cudaStream_t user) 
 }
 
 template <typename T>
-int enqueue_vcycle(const hnv_batch* b, int d, float omega, int sweeps, cudaStream_t s) {
+int enqueue_vcycle(const hnv_batch* b, const BatchDeal& D, int d, float omega, int sweeps, cudaStream_t s) {
   const int dv = (int)(d * sizeof(T) / 16);
+  if ((int)D.steps.size() != D.step_lmax + 1) HNV_FAIL(HNV_ERR_STATE, "work lists not built");
   int32_t* counter = b->counters;
   if (b->kernel == HNV_BATCH_KERNEL_PERSISTENT) {
     const int64_t need = (int64_t)(b->Lmax + 1) * sweeps * 2 * kCountersPerHalf;
     if (need > b->counters_n) HNV_FAIL(HNV_ERR_STATE, "persistent counters not allocated");
     if (need > 0) HNV_CUDA(cudaMemsetAsync(counter, 0, sizeof(int32_t) * (size_t)need, s));
   }
-  if (b->teams > 0) {
-    HNV_CUDA(cudaMemsetAsync(b->team.barriers, 0, sizeof(uint32_t) * 32 * b->teams, s));
-    TeamArgs a = b->team;
+  if (D.teams > 0) {
+    HNV_CUDA(cudaMemsetAsync(D.team.barriers, 0, sizeof(uint32_t) * 32 * D.teams, s));
+    TeamArgs a = D.team;
     a.sweeps = sweeps;
     a.keep = 1.0f - omega;
     a.omega = omega;
-    HNV_CHECK(team_launch(a, b->teams, sizeof(T) == 2 ? HNV_BF16 : HNV_F32, d, s));
+    HNV_CHECK(team_launch(a, D.teams, sizeof(T) == 2 ? HNV_BF16 : HNV_F32, d, s));
   }
-  for (int st = b->step_lmax; st >= 0; --st) {
-    const BStep& S = b->steps[st];
+  for (int st = D.step_lmax; st >= 0; --st) {
+    const BStep& S = D.steps[st];
     BTRACE("enqueue step %d copies %d proj %d", st, S.n_copies, S.n_proj);
     if (S.n_copies) {
       BTRACE("launch copy step %d n=%d total=%lld", st, S.n_copies, (long long)S.copy_total);
@@ -961,14 +985,16 @@ int enqueue_vcycle(const hnv_batch* b, int d, float omega, int sweeps, cudaStrea
   return HNV_OK;
 }
 
-int enqueue(const hnv_batch* b, int dt, int d, float omega, int sweeps, cudaStream_t s) {
-  return dt == HNV_BF16 ? enqueue_vcycle<__nv_bfloat16>(b, d, omega, sweeps, s)
-                        : enqueue_vcycle<float>(b, d, omega, sweeps, s);
+int enqueue(const hnv_batch* b, const BatchDeal& D, int dt, int d, float omega, int sweeps,
+            cudaStream_t s) {
+  return dt == HNV_BF16 ? enqueue_vcycle<__nv_bfloat16>(b, D, d, omega, sweeps, s)
+                        : enqueue_vcycle<float>(b, D, d, omega, sweeps, s);
 }
 
 // milliseconds of one V-cycle of the batch with one sweep per level (median
 // of the timed repetitions; the first run warms the caches)
-int time_vcycle1(const hnv_batch* b, int dt, int d, float omega, cudaStream_t s, float* ms) {
+int time_vcycle1(const hnv_batch* b, const BatchDeal& D, int dt, int d, float omega, cudaStream_t s,
+                 float* ms) {
   cudaEvent_t e0, e1;
   HNV_CUDA(cudaEventCreate(&e0));
   HNV_CUDA(cudaEventCreate(&e1));
@@ -976,7 +1002,7 @@ int time_vcycle1(const hnv_batch* b, int dt, int d, float omega, cudaStream_t s,
   int rc = HNV_OK;
   for (int r = 0; r < 4 && rc == HNV_OK; ++r) {
     cudaEventRecord(e0, s);
-    rc = enqueue(b, dt, d, omega, 1, s);
+    rc = enqueue(b, D, dt, d, omega, 1, s);
     cudaEventRecord(e1, s);
     cudaEventSynchronize(e1);
     float x = 0.f;
@@ -1044,7 +1070,6 @@ int hnv_batch_create(hnv_graph* const* graphs, int32_t count, hnv_batch** out) {
   b->graphs.assign(graphs, graphs + count);
   for (int32_t i = 0; i < count; ++i) b->generation.push_back(graphs[i]->generation);
   b->device = dev0;
-  b->step_top.assign(count, -2);   // not dealt yet
   b->coarse_off.assign(count + 1, 0);
   b->v_off.assign(count + 1, 0);
   b->e_off.assign(count + 1, 0);
@@ -1133,10 +1158,10 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       b->shape = shapes[si];
       std::fill(b->lanes, b->lanes + 3, 0);
       b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
-      choose_teams(b, dt, d, 1, s);
-      rc = build_plans(b, rb, s);
+      BatchDeal& D = pick_deal(b, dt, d, 1, s);
+      rc = build_plans(b, D, rb, s);
       if (rc == HNV_OK)
-        rc = build_steps(b, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
+        rc = build_steps(b, D, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
       const int cand_a[3] = {2, 4, 8}, cand_b[3] = {4, 8, 16};
       for (int ia = 0; ia < 3 && rc == HNV_OK; ++ia)
         for (int ib = 0; ib < 3 && rc == HNV_OK; ++ib) {
@@ -1145,7 +1170,7 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
           b->lanes[2] = 0;
           if (class_lanes(b, 0, dv) != cand_a[ia] || class_lanes(b, 1, dv) != cand_b[ib]) continue;
           float ms = 0.f;
-          rc = time_vcycle1(b, dt, d, omega, s, &ms);
+          rc = time_vcycle1(b, D, dt, d, omega, s, &ms);
           if (rc == HNV_OK && (best_ms < 0.f || ms < best_ms)) {
             best_ms = ms;
             best_shape = shapes[si];
@@ -1156,12 +1181,13 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       if (si == 0 && rc == HNV_OK) {
         std::fill(b->lanes, b->lanes + 3, 0);
         b->kernel = HNV_BATCH_KERNEL_PERSISTENT;
-        if (choose_teams(b, dt, d, 1, s)) {
-          rc = build_plans(b, rb, s);
+        BatchDeal& P = pick_deal(b, dt, d, 1, s);
+        if (&P != &D) {
+          rc = build_plans(b, P, rb, s);
           if (rc == HNV_OK)
-            rc = build_steps(b, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
+            rc = build_steps(b, P, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
         }
-        if (rc == HNV_OK) rc = time_vcycle1(b, dt, d, omega, s, &persistent_ms);
+        if (rc == HNV_OK) rc = time_vcycle1(b, P, dt, d, omega, s, &persistent_ms);
         if (rc == HNV_OK && (best_ms < 0.f || persistent_ms < best_ms)) {
           best_ms = persistent_ms;
           best_shape = shapes[si];
@@ -1169,6 +1195,8 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
         }
       }
     }
+    // (what was built refers to the scratch rows)
+    for (BatchDeal& D : b->deal) drop_deal(b, D, s);
     if (zbuf) dev_free(zbuf, s);
     if (rc == HNV_OK) {
       std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -1179,8 +1207,7 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
     b->shape = best_shape;
     for (int c = 0; c < 3; ++c) b->lanes[c] = best_lanes[c];
     b->kernel = best_lanes[3];
-    free_steps(b, s);
-    b->plans_ready = false;
+    for (BatchDeal& D : b->deal) drop_deal(b, D, s);
     if (chosen) {
       chosen->kernel = best_lanes[3];
       chosen->persistent_ms = persistent_ms;
@@ -1225,19 +1252,19 @@ int hnv_batch_vcycle(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* 
   int rc = HNV_OK;
   do {
     const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
-    const bool dealt = choose_teams(b, (int)dt, d, sweeps_per_level, cs);
-    if (dealt || !b->plans_ready || b->plans_row_bytes != rb) {
-      if ((rc = build_plans(b, rb, cs)) != HNV_OK) break;
-      free_steps(b, cs);
+    BatchDeal& D = pick_deal(b, (int)dt, d, sweeps_per_level, cs);
+    if (!D.plans_ready || D.plans_row_bytes != rb) {
+      free_steps(b, D, cs);   // built from the plans
+      if ((rc = build_plans(b, D, rb, cs)) != HNV_OK) break;
     }
-    if (b->built_dt != (int)dt || b->built_d != d || b->built_zc != z_coarsest ||
-        b->built_zv != z_v_out || b->built_ze != z_e_out || b->built_kernel != b->kernel) {
-      if ((rc = build_steps(b, dt, d, (const uint8_t*)z_coarsest, (uint8_t*)z_v_out,
+    if (D.built_dt != (int)dt || D.built_d != d || D.built_zc != z_coarsest ||
+        D.built_zv != z_v_out || D.built_ze != z_e_out) {
+      if ((rc = build_steps(b, D, dt, d, (const uint8_t*)z_coarsest, (uint8_t*)z_v_out,
                             (uint8_t*)z_e_out, cs)) != HNV_OK)
         break;
-      b->built_zc = z_coarsest;
-      b->built_zv = z_v_out;
-      b->built_ze = z_e_out;
+      D.built_zc = z_coarsest;
+      D.built_zv = z_v_out;
+      D.built_ze = z_e_out;
     }
     if (b->kernel == HNV_BATCH_KERNEL_PERSISTENT &&
         (rc = ensure_counters(b, (int64_t)(b->Lmax + 1) * sweeps_per_level * 2 * kCountersPerHalf,
@@ -1252,44 +1279,45 @@ int hnv_batch_vcycle(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* 
       }
     }
     if (!use_cuda_graph) {
-      rc = enqueue(b, (int)dt, d, omega, sweeps_per_level, s);
+      rc = enqueue(b, D, (int)dt, d, omega, sweeps_per_level, s);
       BTRACE("direct enqueue rc=%d", rc);
       break;
     }
-    if (!b->exec || b->exec_omega != omega || b->exec_sweeps != sweeps_per_level ||
-        b->exec_kernel != b->kernel) {
-      if (b->exec) {
-        cudaGraphExecDestroy(b->exec);
-        b->exec = nullptr;
+    if (!D.exec || D.exec_omega != omega || D.exec_sweeps != sweeps_per_level ||
+        D.exec_kernel != b->kernel) {
+      if (D.exec) {
+        cudaGraphExecDestroy(D.exec);
+        D.exec = nullptr;
       }
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       if (e != cudaSuccess) { rc = cuda_status(e, "cudaStreamBeginCapture"); break; }
       const int64_t before = hnv_kernel_launch_count();
-      const int erc = enqueue(b, (int)dt, d, omega, sweeps_per_level, cs);
+      const int erc = enqueue(b, D, (int)dt, d, omega, sweeps_per_level, cs);
       // captured launches run at replay: count them there, not here
-      b->exec_kernels = hnv_kernel_launch_count() - before;
-      note_launches(-b->exec_kernels);
+      D.exec_kernels = hnv_kernel_launch_count() - before;
+      note_launches(-D.exec_kernels);
       e = cudaStreamEndCapture(cs, &graph);
       if (erc != HNV_OK) { if (graph) cudaGraphDestroy(graph); rc = erc; break; }
       if (e != cudaSuccess) { rc = cuda_status(e, "cudaStreamEndCapture"); break; }
-      e = cudaGraphInstantiate(&b->exec, graph, 0);
+      e = cudaGraphInstantiate(&D.exec, graph, 0);
       cudaGraphDestroy(graph);
-      if (e != cudaSuccess) { b->exec = nullptr; rc = cuda_status(e, "cudaGraphInstantiate"); break; }
-      b->exec_omega = omega;
-      b->exec_sweeps = sweeps_per_level;
-      b->exec_kernel = b->kernel;
+      if (e != cudaSuccess) { D.exec = nullptr; rc = cuda_status(e, "cudaGraphInstantiate"); break; }
+      D.exec_omega = omega;
+      D.exec_sweeps = sweeps_per_level;
+      D.exec_kernel = b->kernel;
     }
-    BTRACE("graph launch (%lld kernels)", (long long)b->exec_kernels);
-    cudaError_t e = cudaGraphLaunch(b->exec, s);
+    BTRACE("graph launch (%lld kernels)", (long long)D.exec_kernels);
+    cudaError_t e = cudaGraphLaunch(D.exec, s);
     if (e != cudaSuccess) rc = cuda_status(e, "cudaGraphLaunch");
-    else note_launches(b->exec_kernels);
+    else note_launches(D.exec_kernels);
   } while (0);
-  if (rc == HNV_OK) {
+  {
+    // also after a failure, which may have come after some launches
     // (an event recorded under capture cannot order later work)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
-      b->used = cudaEventRecord(b->used_ev, s) == cudaSuccess;
+      b->used = cudaEventRecord(b->used_ev, s) == cudaSuccess || b->used;
   }
   if (prev >= 0) cudaSetDevice(prev);
   return rc;
@@ -1312,8 +1340,7 @@ void hnv_batch_free(hnv_batch* b) {
   cudaGetDevice(&prev);
   cudaSetDevice(b->device);
   if (b->cap_stream) {
-    free_steps(b, b->cap_stream);
-    free_list(b->plan_owned, b->cap_stream);
+    for (BatchDeal& D : b->deal) drop_deal(b, D, b->cap_stream);
     if (b->counters) dev_free(b->counters, b->cap_stream);
     cudaStreamSynchronize(b->cap_stream);
     cudaStreamDestroy(b->cap_stream);

@@ -198,3 +198,153 @@ def test_batch_goes_stale_when_a_graph_is_coarsened_again(H):
         assert ei.value.code == -8
     for G in Gs:
         G.close()
+
+
+def _buffers(B, d, dt, seed=0):
+    import torch
+    co, vo, eo = B.offsets()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    zc = torch.randn((int(co[-1]), d), generator=g, device="cuda").to(dt)
+    return zc, torch.empty((int(vo[-1]), d), dtype=dt, device="cuda"), \
+        torch.empty((int(eo[-1]), d), dtype=dt, device="cuda")
+
+
+def _launches(H, f):
+    import torch
+    before = H.kernel_launch_count()
+    f()
+    torch.cuda.synchronize()
+    return H.kernel_launch_count() - before
+
+
+class _StepLists:
+    """Phase timing selects a launch per half-sweep: every graph in the step
+    lists of the batch, and the per-launch path for a single graph."""
+
+    def __init__(self, H):
+        self.H = H
+
+    def __enter__(self):
+        self.H.timing_enable(True)
+
+    def __exit__(self, *exc):
+        self.H.timing_enable(False)
+        self.H.timing_reset()
+
+
+@pytest.mark.parametrize("dtname,d", [("f32", 256), ("bf16", 512)])
+def test_batch_of_teams_and_stepped_graphs(H, dtname, d):
+    """One graph too large for a team among small ones; calls of more sweeps
+    than a team's launch takes in between, on the same buffers. A caller's
+    captured V-cycle stays valid through them (the lists it uses are kept)."""
+    import torch
+    dt = torch.float32 if dtname == "f32" else torch.bfloat16
+    hgs, Gs = _graphs(H, 4, seed=7)
+    big = hypergen.planted_hypergraph(60_000, 50_000, C=8, alpha=1.8, cap=500, p_in=0.8,
+                                      weighted=True, seed=1)
+    G = H.Graph.from_hypergraph(big)
+    G.coarsen(min_nodes=3000, max_levels=2)
+    assert G.level_info(0)[2] * 1024 > 250_000_000
+    Gs.insert(2, G)
+    with H.Batch(Gs) as B:
+        zc, zv, ze = _buffers(B, d, dt)
+
+        def run(sweeps, graph):
+            zv.fill_(float("nan"))
+            ze.fill_(float("nan"))
+            n = _launches(H, lambda: B.vcycle(zc, zv, ze, 0.5, sweeps, use_cuda_graph=graph))
+            for G in Gs:
+                G.sync_status()
+            return n, zv.clone(), ze.clone()
+        with _StepLists(H):
+            want = {k: run(k, False) for k in (3, 513)}
+        own = None
+        for k, graph in ((3, False), (3, True), (513, False), (3, False), (513, True), (3, True)):
+            got = run(k, graph)
+            assert torch.equal(got[1], want[k][1]) and torch.equal(got[2], want[k][2])
+            assert (got[0] < want[k][0]) == (k == 3)
+            if own is None:
+                own = torch.cuda.CUDAGraph()
+                s = torch.cuda.Stream()
+                s.wait_stream(torch.cuda.current_stream())
+                stream, B.stream = B.stream, s
+                with torch.cuda.graph(own, stream=s, capture_error_mode="relaxed"):
+                    B.vcycle(zc, zv, ze, 0.5, 3, use_cuda_graph=False)
+                B.stream = stream
+        zv.fill_(float("nan"))
+        ze.fill_(float("nan"))
+        own.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(zv, want[3][1]) and torch.equal(ze, want[3][2])
+    for G in Gs:
+        G.close()
+
+
+class _Allocator:
+    """A device allocator hook that refuses once `left` requests were granted."""
+
+    def __init__(self, H):
+        import ctypes
+        self.H, self.held, self.left = H, [], None
+        AF = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p)
+        FF = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+        self.fns = AF(self._alloc), FF(lambda p, s, ctx: None)
+        self.ptrs = [ctypes.cast(f, ctypes.c_void_p) for f in self.fns]
+
+    def _alloc(self, nbytes, s, ctx):
+        import torch
+        if self.left is not None:
+            if self.left == 0:
+                return None
+            self.left -= 1
+        self.held.append(torch.empty(nbytes, dtype=torch.uint8, device="cuda"))
+        return self.held[-1].data_ptr()
+
+    def __enter__(self):
+        assert self.H.lib().hnv_set_allocator(self.ptrs[0], self.ptrs[1], None) == 0
+        return self
+
+    def __exit__(self, *exc):
+        import torch
+        torch.cuda.synchronize()
+        assert self.H.lib().hnv_set_allocator(None, None, None) == 0
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_batch_survives_a_build_that_fails(H, graph):
+    """Work lists for another dealing of the graphs (more sweeps than a team's
+    launch takes), with the allocator refusing at every point of the build in
+    turn: each call fails with HNV_ERR_OOM, the next tries again, and what was
+    built before keeps working."""
+    import torch
+    d = 16
+    with _Allocator(H) as hook:
+        hgs, Gs = _graphs(H, 3, seed=21)
+        with H.Batch(Gs) as B:
+            zc, zv, ze = _buffers(B, d, torch.float32)
+            B.vcycle(zc, zv, ze, 0.5, 4, use_cuda_graph=graph)
+            few = zv.clone(), ze.clone()
+            for granted in range(10_000):
+                hook.left = granted
+                try:
+                    B.vcycle(zc, zv, ze, 0.5, 513, use_cuda_graph=graph)
+                    break
+                except H.HNVError as e:
+                    assert e.code == -4
+                hook.left = None
+                if granted % 16 == 0:
+                    B.vcycle(zc, zv, ze, 0.5, 4, use_cuda_graph=graph)
+                    assert torch.equal(zv, few[0]) and torch.equal(ze, few[1])
+            assert granted > 16
+            hook.left = None
+            co, vo, eo = B.offsets()
+            for i, G in enumerate(Gs):
+                G.sync_status()
+                sv, se = _run_single(H, G, zc[co[i]:co[i + 1]].contiguous(), d, torch.float32, 513)
+                assert torch.equal(sv, zv[vo[i]:vo[i + 1]]) and torch.equal(se, ze[eo[i]:eo[i + 1]])
+            B.vcycle(zc, zv, ze, 0.5, 4, use_cuda_graph=graph)
+            torch.cuda.synchronize()
+            assert torch.equal(zv, few[0]) and torch.equal(ze, few[1])
+        for G in Gs:
+            G.close()
