@@ -233,6 +233,43 @@ class _StepLists:
         self.H.timing_reset()
 
 
+@pytest.mark.parametrize("dtname,d", [("f32", 8), ("f32", 64), ("bf16", 64), ("bf16", 512)])
+def test_teams_and_step_lists_give_the_same_bits(H, dtname, d):
+    """Small graphs run by teams in one launch, and lined up in the step lists
+    of the per-class kernels (direct, captured, replayed, and with the row
+    classes and lanes of the autotuner)."""
+    import torch
+    dt = torch.float32 if dtname == "f32" else torch.bfloat16
+    hgs, Gs = _graphs(H, 9, seed=40 + d)
+    with H.Batch(Gs) as B:
+        zc, zv, ze = _buffers(B, d, dt)
+
+        def run(graph):
+            zv.fill_(float("nan"))
+            ze.fill_(float("nan"))
+            n = _launches(H, lambda: B.vcycle(zc, zv, ze, 0.5, 4, use_cuda_graph=graph))
+            for G in Gs:
+                G.sync_status()
+            return n, zv.clone(), ze.clone()
+        want = run(False)
+        assert want[0] == 1
+        for graph in (True, True):
+            got = run(graph)
+            assert got[0] == 1 and torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+        for tuned in (False, True):
+            if tuned:
+                B.autotune(H.F32 if dtname == "f32" else H.BF16, d)
+                B.kernel = H.BATCH_KERNEL_PER_CLASS
+            for graph in (False, True, True):
+                with _StepLists(H):
+                    got = run(graph)
+                assert got[0] > 8 and torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+        got = run(True)
+        assert got[0] == 1 and torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+    for G in Gs:
+        G.close()
+
+
 @pytest.mark.parametrize("dtname,d", [("f32", 256), ("bf16", 512)])
 def test_batch_of_teams_and_stepped_graphs(H, dtname, d):
     """One graph too large for a team among small ones; calls of more sweeps
