@@ -389,9 +389,12 @@ int hnv_batch_offsets(const hnv_batch* b, int64_t* coarsest_rows, int64_t* node_
 
 /* Times candidate row-class boundaries and lanes per row of the per-class
  * kernel, and the persistent kernel, on a whole V-cycle of the batch with one
- * sweep per level, and keeps the fastest (cached per dtype, d and the batch's
- * level-0 row-length histogram). Uses scratch rows of the batch's level-0
- * size while it runs. Synchronises. */
+ * sweep per level, and keeps the fastest (cached per dtype, d, the batch's
+ * level-0 row-length histogram and the number of its graphs that teams run).
+ * The boundaries and lanes are timed with every graph lined up by level, and
+ * serve the calls and graphs that are; where the per-class setting gives graphs
+ * to teams, that is what the persistent kernel is compared with. Uses scratch
+ * rows of the batch's level-0 size while it runs. Synchronises. */
 int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch_tuning* chosen);
 
 /* Selects the half-sweep kernel (HNV_BATCH_KERNEL_*) of later hnv_batch_vcycle

@@ -434,20 +434,23 @@ void drop_deal(const hnv_batch* b, BatchDeal& D, cudaStream_t s) {
   D.plans_ready = false;
 }
 
-// The deal a call takes. The teams run the graphs all of whose levels are
-// small, with the per-class setting and at most kTeamMaxSweeps sweeps.
-BatchDeal& pick_deal(hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
+// The coarsest level of each graph, -1 for those the teams run: the graphs all
+// of whose levels are small, with the per-class setting and at most
+// kTeamMaxSweeps sweeps.
+std::vector<int> deal_teams(const hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
   std::vector<int> top = b->top;
-  bool any = false;
   if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && team_enabled(d) && sweeps <= kTeamMaxSweeps)
     for (size_t i = 0; i < b->graphs.size(); ++i) {
       bool fits = true;
       for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
-      if (!fits || !team_ready(b->graphs[i], s)) continue;
-      top[i] = -1;
-      any = true;
+      if (fits && team_ready(b->graphs[i], s)) top[i] = -1;
     }
-  BatchDeal& D = b->deal[any ? 0 : 1];
+  return top;
+}
+
+// The deal that belongs to `top` (the second if no graph is with the teams).
+BatchDeal& use_deal(hnv_batch* b, const std::vector<int>& top, cudaStream_t s) {
+  BatchDeal& D = b->deal[top == b->top ? 1 : 0];
   if (D.step_top != top) {
     drop_deal(b, D, s);
     D.step_top = top;
@@ -1017,8 +1020,9 @@ int time_vcycle1(const hnv_batch* b, const BatchDeal& D, int dt, int d, float om
   return HNV_OK;
 }
 
-std::vector<int64_t> tune_key(const hnv_batch* b, int dt, int d) {
-  std::vector<int64_t> k{dt, d, (int64_t)b->graphs.size()};
+// `teamed`: the graphs that the teams run with the per-class setting.
+std::vector<int64_t> tune_key(const hnv_batch* b, int dt, int d, int64_t teamed) {
+  std::vector<int64_t> k{dt, d, (int64_t)b->graphs.size(), teamed};
   int64_t hist[2][24] = {{0}};
   for (hnv_graph* g : b->graphs) {
     const Level& lv = g->levels[0];
@@ -1124,19 +1128,26 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
   cudaSetDevice(b->device);
   cudaStream_t s = b->cap_stream;
   int rc = HNV_OK;
-  const std::vector<int64_t> key = tune_key(b, dt, d);
+  const PlanShape old_shape = b->shape;
+  const int old_kernel = b->kernel;
+  const std::vector<int> old_lanes(b->lanes, b->lanes + 3);
+  b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
+  const std::vector<int> teams_top = deal_teams(b, dt, d, 1, s);
+  const int64_t teamed = std::count(teams_top.begin(), teams_top.end(), -1);
+  const std::vector<int64_t> key = tune_key(b, dt, d, teamed);
   PlanShape best_shape = b->shape;
   std::vector<int> best_lanes(4, 0);   // lanes of classes A, B, rest; [3]: kernel
   float best_ms = -1.f, persistent_ms = -1.f;
+  bool cached = false;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
       best_shape = it->second.first;
       best_lanes = it->second.second;
+      cached = true;
     }
   }
-  const bool cached = best_lanes[0] != 0 || best_lanes[3] == HNV_BATCH_KERNEL_PERSISTENT;
   const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
   const int dv = (int)(rb / 16);
   uint8_t* zbuf = nullptr;
@@ -1150,18 +1161,20 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       const cudaError_t e = cudaMemsetAsync(zbuf, 0, rows * rb, s);
       if (e != cudaSuccess) rc = cuda_status(e, "cudaMemsetAsync");
     }
-    const PlanShape shapes[3] = {{4, 16, 64}, {2, 8, 32}, {8, 32, 64}};
     if (rc == HNV_OK) rc = ensure_counters(b, (int64_t)(b->Lmax + 1) * 2 * kCountersPerHalf, s, s);
+    // builds for the current shape; lanes and kernel only change the launches
+    auto build = [&](BatchDeal& D) -> int {
+      HNV_CHECK(build_plans(b, D, rb, s));
+      return build_steps(b, D, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
+    };
+    // the candidates are timed with every graph in the step lists: the teams'
+    // launch would be the same for all of them
+    BatchDeal& S = use_deal(b, b->top, s);
+    const PlanShape shapes[3] = {{4, 16, 64}, {2, 8, 32}, {8, 32, 64}};
     for (int si = 0; si < 3 && rc == HNV_OK; ++si) {
-      // plans and work lists depend on the class boundaries only; the lanes
-      // per row and the kernel only change the launches
       b->shape = shapes[si];
-      std::fill(b->lanes, b->lanes + 3, 0);
       b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
-      BatchDeal& D = pick_deal(b, dt, d, 1, s);
-      rc = build_plans(b, D, rb, s);
-      if (rc == HNV_OK)
-        rc = build_steps(b, D, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
+      rc = build(S);
       const int cand_a[3] = {2, 4, 8}, cand_b[3] = {4, 8, 16};
       for (int ia = 0; ia < 3 && rc == HNV_OK; ++ia)
         for (int ib = 0; ib < 3 && rc == HNV_OK; ++ib) {
@@ -1170,7 +1183,7 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
           b->lanes[2] = 0;
           if (class_lanes(b, 0, dv) != cand_a[ia] || class_lanes(b, 1, dv) != cand_b[ib]) continue;
           float ms = 0.f;
-          rc = time_vcycle1(b, D, dt, d, omega, s, &ms);
+          rc = time_vcycle1(b, S, dt, d, omega, s, &ms);
           if (rc == HNV_OK && (best_ms < 0.f || ms < best_ms)) {
             best_ms = ms;
             best_shape = shapes[si];
@@ -1181,33 +1194,39 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       if (si == 0 && rc == HNV_OK) {
         std::fill(b->lanes, b->lanes + 3, 0);
         b->kernel = HNV_BATCH_KERNEL_PERSISTENT;
-        BatchDeal& P = pick_deal(b, dt, d, 1, s);
-        if (&P != &D) {
-          rc = build_plans(b, P, rb, s);
-          if (rc == HNV_OK)
-            rc = build_steps(b, P, dt, d, zbuf, zbuf, zbuf + (size_t)b->v_off.back() * rb, s);
-        }
-        if (rc == HNV_OK) rc = time_vcycle1(b, P, dt, d, omega, s, &persistent_ms);
-        if (rc == HNV_OK && (best_ms < 0.f || persistent_ms < best_ms)) {
-          best_ms = persistent_ms;
-          best_shape = shapes[si];
-          best_lanes = {0, 0, 0, HNV_BATCH_KERNEL_PERSISTENT};
-        }
+        rc = time_vcycle1(b, S, dt, d, omega, s, &persistent_ms);
       }
     }
-    // (what was built refers to the scratch rows)
-    for (BatchDeal& D : b->deal) drop_deal(b, D, s);
-    if (zbuf) dev_free(zbuf, s);
+    // what the per-class setting runs where it has graphs for the teams
+    if (rc == HNV_OK && teamed > 0) {
+      b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
+      b->shape = best_ms >= 0.f ? best_shape : shapes[0];
+      for (int c = 0; c < 3; ++c) b->lanes[c] = best_lanes[c];
+      BatchDeal& D = use_deal(b, teams_top, s);
+      rc = build(D);
+      if (rc == HNV_OK) rc = time_vcycle1(b, D, dt, d, omega, s, &best_ms);
+    }
+    if (rc == HNV_OK && (best_ms < 0.f || persistent_ms < best_ms)) {
+      best_ms = persistent_ms;
+      best_shape = shapes[0];
+      best_lanes = {0, 0, 0, HNV_BATCH_KERNEL_PERSISTENT};
+    }
     if (rc == HNV_OK) {
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tune_cache[key] = {best_shape, best_lanes};
     }
   }
-  if (rc == HNV_OK) {
+  // (what was built is for another shape, or for the scratch rows)
+  for (BatchDeal& D : b->deal) drop_deal(b, D, s);
+  if (zbuf) dev_free(zbuf, s);
+  if (rc != HNV_OK) {
+    b->shape = old_shape;
+    b->kernel = old_kernel;
+    std::copy(old_lanes.begin(), old_lanes.end(), b->lanes);
+  } else {
     b->shape = best_shape;
     for (int c = 0; c < 3; ++c) b->lanes[c] = best_lanes[c];
     b->kernel = best_lanes[3];
-    for (BatchDeal& D : b->deal) drop_deal(b, D, s);
     if (chosen) {
       chosen->kernel = best_lanes[3];
       chosen->persistent_ms = persistent_ms;
@@ -1252,7 +1271,7 @@ int hnv_batch_vcycle(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* 
   int rc = HNV_OK;
   do {
     const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
-    BatchDeal& D = pick_deal(b, (int)dt, d, sweeps_per_level, cs);
+    BatchDeal& D = use_deal(b, deal_teams(b, (int)dt, d, sweeps_per_level, cs), cs);
     if (!D.plans_ready || D.plans_row_bytes != rb) {
       free_steps(b, D, cs);   // built from the plans
       if ((rc = build_plans(b, D, rb, cs)) != HNV_OK) break;

@@ -385,3 +385,38 @@ def test_batch_survives_a_build_that_fails(H, graph):
             assert torch.equal(zv, few[0]) and torch.equal(ze, few[1])
         for G in Gs:
             G.close()
+
+
+def test_autotune_times_the_step_lists(H):
+    """The row classes and lanes only matter to graphs in the step lists: they
+    are timed there, also for a batch whose graphs the teams run, and what is
+    found with the teams is not taken for a batch without them."""
+    import torch
+    d = 32
+    hgs, Gs = _graphs(H, 7, seed=77)
+    with H.Batch(Gs) as B:
+        zc, zv, ze = _buffers(B, d, torch.float32)
+        launches = []
+
+        def one():
+            launches.append(_launches(H, lambda: B.vcycle(zc, zv, ze, 0.5, 1)))
+            return zv.clone(), ze.clone()
+        want = one()
+        one()
+        tuned = {}
+        n = _launches(H, lambda: tuned.update(B.autotune(H.F32, d)))
+        assert tuned["from_cache"] == 0
+        with _StepLists(H):
+            B.kernel = H.BATCH_KERNEL_PER_CLASS
+            one()                                        # (builds the lists)
+            got = one()
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+            t = B.autotune(H.F32, d)
+            assert t["from_cache"] == 0                  # no graph goes to the teams now
+            assert B.autotune(H.F32, d)["from_cache"] == 1
+        t = B.autotune(H.F32, d)
+        assert t["from_cache"] == 1 and t["kernel"] == tuned["kernel"] == B.kernel
+        # 4 timed V-cycles of each candidate (18 at this width)
+        assert launches[1] == 1 and n > 4 * 18 * launches[3]
+    for G in Gs:
+        G.close()
