@@ -114,6 +114,7 @@ def _declare(L):
         "hnv_release_cached_memory": (ctypes.c_int, []),
         "hnv_selftest_wait_timeout": (ctypes.c_int, [_P, ctypes.c_uint32, _P]),
         "hnv_selftest_team_timeout": (ctypes.c_int, [_P, i32, ctypes.c_uint32]),
+        "hnv_selftest_team_refuse": (ctypes.c_int, [_P, ctypes.c_int]),
         "hnv_batch_get_kernel": (ctypes.c_int, [_P]),
         "hnv_set_weights": (ctypes.c_int, [_P, _P, ctypes.c_int, _P]),
         "hnv_checkpoint_floats": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(i64)]),

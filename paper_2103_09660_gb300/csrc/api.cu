@@ -144,8 +144,12 @@ int vcycle_impl(hnv_graph* g, const void* z_coarsest, void* z_v_out, void* z_e_o
     t.buf[0] = reinterpret_cast<uint4*>(buf[0]);
     t.buf[1] = reinterpret_cast<uint4*>(buf[1]);
     t.ckpt = reinterpret_cast<uint4*>(ckpt);
-    HNV_CHECK(team_run(g, t, dtype, d, omega, sweeps, mode, s));
-  } else if (top.n > 0) HNV_CUDA(cudaMemcpyAsync(zv(L), zc, row_bytes * top.n, kind, s));
+    const int rc = team_run(g, t, dtype, d, omega, sweeps, mode, s);
+    if (rc == kTeamRefused) first_big = L;
+    else HNV_CHECK(rc);
+  }
+  if (first_big == L && top.n > 0)
+    HNV_CUDA(cudaMemcpyAsync(zv(L), zc, row_bytes * top.n, kind, s));
   if (first_big == L && top.m > 0)
     HNV_CUDA(cudaMemcpyAsync(ze(L), zc + (size_t)top.n * row_bytes, row_bytes * top.m, kind, s));
   std::vector<size_t> off(L + 2, 0);
@@ -661,6 +665,13 @@ int hnv_selftest_team_timeout(hnv_graph* g, int32_t barrier, uint32_t limit_us) 
     HNV_FAIL(HNV_ERR_INVALID_ARG, "limit_us = %u: need 1 .. 1000000", limit_us);
   g->team_stop_at = barrier;
   g->team_wait_ns = barrier > 0 ? (uint64_t)limit_us * 1000ull : kTeamWaitNs;
+  return HNV_OK;
+}
+
+int hnv_selftest_team_refuse(hnv_graph* g, int refuse) {
+  clear_error_detail();
+  if (!g) HNV_FAIL(HNV_ERR_INVALID_ARG, "graph is NULL");
+  g->team_refuse = refuse != 0;
   return HNV_OK;
 }
 

@@ -388,6 +388,7 @@ struct hnv_batch {
   int lanes[3] = {0, 0, 0};        // lanes per row of classes A, B, rest (0: default)
   // [0] small graphs run by teams, [1] every graph in the step lists
   BatchDeal deal[2];
+  bool no_teams = false;           // the device refused the teams' launch
   // half-sweep kernel: 0 one launch per row class, 1 one persistent launch
   int kernel = HNV_BATCH_KERNEL_PER_CLASS;
   // task counters of the persistent launches, one per half-sweep of a V-cycle
@@ -439,7 +440,8 @@ void drop_deal(const hnv_batch* b, BatchDeal& D, cudaStream_t s) {
 // kTeamMaxSweeps sweeps.
 std::vector<int> deal_teams(const hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
   std::vector<int> top = b->top;
-  if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && team_enabled(d) && sweeps <= kTeamMaxSweeps)
+  if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && !b->no_teams && team_enabled(d) &&
+      sweeps <= kTeamMaxSweeps)
     for (size_t i = 0; i < b->graphs.size(); ++i) {
       bool fits = true;
       for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
@@ -946,8 +948,10 @@ int ensure_counters(hnv_batch* b, int64_t n, cudaStream_t s, cudaStream_t user) 
   return HNV_OK;
 }
 
+// (kTeamRefused: see team_launch; nothing was enqueued that counts)
 template <typename T>
-int enqueue_vcycle(const hnv_batch* b, const BatchDeal& D, int d, float omega, int sweeps, cudaStream_t s) {
+int enqueue_vcycle(const hnv_batch* b, const BatchDeal& D, int d, float omega, int sweeps,
+                   cudaStream_t s) {
   const int dv = (int)(d * sizeof(T) / 16);
   if ((int)D.steps.size() != D.step_lmax + 1) HNV_FAIL(HNV_ERR_STATE, "work lists not built");
   int32_t* counter = b->counters;
@@ -957,6 +961,8 @@ int enqueue_vcycle(const hnv_batch* b, const BatchDeal& D, int d, float omega, i
     if (need > 0) HNV_CUDA(cudaMemsetAsync(counter, 0, sizeof(int32_t) * (size_t)need, s));
   }
   if (D.teams > 0) {
+    for (size_t i = 0; i < b->graphs.size(); ++i)
+      if (D.step_top[i] < 0 && b->graphs[i]->team_refuse) return kTeamRefused;
     HNV_CUDA(cudaMemsetAsync(D.team.barriers, 0, sizeof(uint32_t) * 32 * D.teams, s));
     TeamArgs a = D.team;
     a.sweeps = sweeps;
@@ -1045,6 +1051,69 @@ std::vector<int64_t> tune_key(const hnv_batch* b, int dt, int d, int64_t teamed)
     for (int64_t x : hist[side]) k.push_back(tot ? (100 * x) / tot : 0);
   }
   return k;
+}
+
+// One hnv_batch_vcycle with the graphs dealt as they are, or kTeamRefused.
+int vcycle_once(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* z_e_out, int dt, int d,
+                float omega, int sweeps, int use_cuda_graph, cudaStream_t s) {
+  cudaStream_t cs = b->cap_stream;
+  const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
+  BatchDeal& D = use_deal(b, deal_teams(b, dt, d, sweeps, cs), cs);
+  if (!D.plans_ready || D.plans_row_bytes != rb) {
+    free_steps(b, D, cs);   // built from the plans
+    HNV_CHECK(build_plans(b, D, rb, cs));
+  }
+  if (D.built_dt != dt || D.built_d != d || D.built_zc != z_coarsest || D.built_zv != z_v_out ||
+      D.built_ze != z_e_out) {
+    HNV_CHECK(build_steps(b, D, dt, d, (const uint8_t*)z_coarsest, (uint8_t*)z_v_out,
+                          (uint8_t*)z_e_out, cs));
+    D.built_zc = z_coarsest;
+    D.built_zv = z_v_out;
+    D.built_ze = z_e_out;
+  }
+  if (b->kernel == HNV_BATCH_KERNEL_PERSISTENT)
+    HNV_CHECK(ensure_counters(b, (int64_t)(b->Lmax + 1) * sweeps * 2 * kCountersPerHalf, cs, s));
+  // the caller's stream must see the set-up work done on the batch stream
+  HNV_CUDA(cudaStreamSynchronize(cs));
+  if (!use_cuda_graph) return enqueue(b, D, dt, d, omega, sweeps, s);
+  // (the launches inside a graph may be refused when it is instantiated or launched)
+  auto status = [&](cudaError_t e, const char* what) {
+    cudaGetLastError();
+    return D.teams > 0 && team_refused(e) ? kTeamRefused : cuda_status(e, what);
+  };
+  if (!D.exec || D.exec_omega != omega || D.exec_sweeps != sweeps || D.exec_kernel != b->kernel) {
+    if (D.exec) {
+      cudaGraphExecDestroy(D.exec);
+      D.exec = nullptr;
+    }
+    cudaGraph_t graph = nullptr;
+    HNV_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    const int64_t before = hnv_kernel_launch_count();
+    const int rc = enqueue(b, D, dt, d, omega, sweeps, cs);
+    // captured launches run at replay: count them there, not here
+    D.exec_kernels = hnv_kernel_launch_count() - before;
+    note_launches(-D.exec_kernels);
+    cudaError_t e = cudaStreamEndCapture(cs, &graph);
+    if (rc != HNV_OK || e != cudaSuccess) {
+      if (graph) cudaGraphDestroy(graph);
+      cudaGetLastError();
+      return rc != HNV_OK ? rc : cuda_status(e, "cudaStreamEndCapture");
+    }
+    e = cudaGraphInstantiate(&D.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+      D.exec = nullptr;
+      return status(e, "cudaGraphInstantiate");
+    }
+    D.exec_omega = omega;
+    D.exec_sweeps = sweeps;
+    D.exec_kernel = b->kernel;
+  }
+  BTRACE("graph launch (%lld kernels)", (long long)D.exec_kernels);
+  const cudaError_t e = cudaGraphLaunch(D.exec, s);
+  if (e != cudaSuccess) return status(e, "cudaGraphLaunch");
+  note_launches(D.exec_kernels);
+  return HNV_OK;
 }
 
 }  // namespace
@@ -1204,14 +1273,20 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
       for (int c = 0; c < 3; ++c) b->lanes[c] = best_lanes[c];
       BatchDeal& D = use_deal(b, teams_top, s);
       rc = build(D);
-      if (rc == HNV_OK) rc = time_vcycle1(b, D, dt, d, omega, s, &best_ms);
+      float ms = 0.f;
+      if (rc == HNV_OK) rc = time_vcycle1(b, D, dt, d, omega, s, &ms);
+      if (rc == HNV_OK) best_ms = ms;
+      if (rc == kTeamRefused) {
+        b->no_teams = true;
+        rc = HNV_OK;
+      }
     }
     if (rc == HNV_OK && (best_ms < 0.f || persistent_ms < best_ms)) {
       best_ms = persistent_ms;
       best_shape = shapes[0];
       best_lanes = {0, 0, 0, HNV_BATCH_KERNEL_PERSISTENT};
     }
-    if (rc == HNV_OK) {
+    if (rc == HNV_OK && !(teamed > 0 && b->no_teams)) {   // (the key has the teams' graphs)
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tune_cache[key] = {best_shape, best_lanes};
     }
@@ -1267,70 +1342,13 @@ int hnv_batch_vcycle(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* 
   cudaGetDevice(&prev);
   cudaSetDevice(b->device);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  cudaStream_t cs = b->cap_stream;
-  int rc = HNV_OK;
-  do {
-    const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
-    BatchDeal& D = use_deal(b, deal_teams(b, (int)dt, d, sweeps_per_level, cs), cs);
-    if (!D.plans_ready || D.plans_row_bytes != rb) {
-      free_steps(b, D, cs);   // built from the plans
-      if ((rc = build_plans(b, D, rb, cs)) != HNV_OK) break;
-    }
-    if (D.built_dt != (int)dt || D.built_d != d || D.built_zc != z_coarsest ||
-        D.built_zv != z_v_out || D.built_ze != z_e_out) {
-      if ((rc = build_steps(b, D, dt, d, (const uint8_t*)z_coarsest, (uint8_t*)z_v_out,
-                            (uint8_t*)z_e_out, cs)) != HNV_OK)
-        break;
-      D.built_zc = z_coarsest;
-      D.built_zv = z_v_out;
-      D.built_ze = z_e_out;
-    }
-    if (b->kernel == HNV_BATCH_KERNEL_PERSISTENT &&
-        (rc = ensure_counters(b, (int64_t)(b->Lmax + 1) * sweeps_per_level * 2 * kCountersPerHalf,
-                              cs, s)) != HNV_OK)
-      break;
-    // the caller's stream must see the set-up work done on the batch stream
-    {
-      const cudaError_t e = cudaStreamSynchronize(cs);
-      if (e != cudaSuccess) {
-        rc = cuda_status(e, "cudaStreamSynchronize");
-        break;
-      }
-    }
-    if (!use_cuda_graph) {
-      rc = enqueue(b, D, (int)dt, d, omega, sweeps_per_level, s);
-      BTRACE("direct enqueue rc=%d", rc);
-      break;
-    }
-    if (!D.exec || D.exec_omega != omega || D.exec_sweeps != sweeps_per_level ||
-        D.exec_kernel != b->kernel) {
-      if (D.exec) {
-        cudaGraphExecDestroy(D.exec);
-        D.exec = nullptr;
-      }
-      cudaGraph_t graph = nullptr;
-      cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) { rc = cuda_status(e, "cudaStreamBeginCapture"); break; }
-      const int64_t before = hnv_kernel_launch_count();
-      const int erc = enqueue(b, D, (int)dt, d, omega, sweeps_per_level, cs);
-      // captured launches run at replay: count them there, not here
-      D.exec_kernels = hnv_kernel_launch_count() - before;
-      note_launches(-D.exec_kernels);
-      e = cudaStreamEndCapture(cs, &graph);
-      if (erc != HNV_OK) { if (graph) cudaGraphDestroy(graph); rc = erc; break; }
-      if (e != cudaSuccess) { rc = cuda_status(e, "cudaStreamEndCapture"); break; }
-      e = cudaGraphInstantiate(&D.exec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (e != cudaSuccess) { D.exec = nullptr; rc = cuda_status(e, "cudaGraphInstantiate"); break; }
-      D.exec_omega = omega;
-      D.exec_sweeps = sweeps_per_level;
-      D.exec_kernel = b->kernel;
-    }
-    BTRACE("graph launch (%lld kernels)", (long long)D.exec_kernels);
-    cudaError_t e = cudaGraphLaunch(D.exec, s);
-    if (e != cudaSuccess) rc = cuda_status(e, "cudaGraphLaunch");
-    else note_launches(D.exec_kernels);
-  } while (0);
+  int rc = vcycle_once(b, z_coarsest, z_v_out, z_e_out, (int)dt, d, omega, sweeps_per_level,
+                       use_cuda_graph, s);
+  if (rc == kTeamRefused) {
+    b->no_teams = true;
+    rc = vcycle_once(b, z_coarsest, z_v_out, z_e_out, (int)dt, d, omega, sweeps_per_level,
+                     use_cuda_graph, s);
+  }
   {
     // also after a failure, which may have come after some launches
     // (an event recorded under capture cannot order later work)

@@ -51,29 +51,35 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
                        float omega, int max_sweeps, float eps, int mode, int32_t* sweeps_done,
                        float* last_delta, cudaStream_t s) {
   const Level& lv = g->levels[level];
+  int32_t done = 0;
+  float delta = 0.f;
   if (max_sweeps > 0 && team_enabled(d) && team_fits(lv, dtype, d) && team_ready(g, s)) {
     // sweeps, changes and the test in one launch (at most kTeamMaxSweeps each)
     TempPool pool(s);
     int32_t* words = nullptr;
     HNV_CHECK(pool.get(&words, kTeamWords));
-    int32_t done = 0, res[3] = {0, 0, 0};
-    float delta = 0.f;
+    int32_t res[3] = {0, 0, 0};
+    int rc = HNV_OK;
     do {
       TeamGraph t;
       t.top = t.bottom = level;
       t.zv0 = static_cast<uint4*>(z_v);
       t.ze0 = static_cast<uint4*>(z_e);
       const int k = max_sweeps - done < kTeamMaxSweeps ? max_sweeps - done : kTeamMaxSweeps;
-      HNV_CHECK(team_run(g, t, dtype, d, omega, k, mode, s, &eps, words));
+      rc = team_run(g, t, dtype, d, omega, k, mode, s, &eps, words);
+      if (rc == kTeamRefused) break;
+      HNV_CHECK(rc);
       HNV_CHECK(read_ints(g, words + kTeamResult, 3, res, s));
       // in whichever sweep: the rows are then half-written
       if (res[2]) HNV_FAIL(HNV_ERR_TIMEOUT, "a bounded wait of a refinement kernel gave up");
       done += res[0];
       std::memcpy(&delta, &res[1], sizeof(float));
     } while (done < max_sweeps && !(delta <= eps));
-    *sweeps_done = done;
-    *last_delta = delta;
-    return HNV_OK;
+    if (rc != kTeamRefused) {
+      *sweeps_done = done;
+      *last_delta = delta;
+      return HNV_OK;
+    }
   }
   const size_t rb = (dtype == HNV_BF16 ? 2 : 4) * (size_t)d;
   const int64_t vec_v = (int64_t)lv.n * (int64_t)(rb / 16), vec_e = (int64_t)lv.m * (int64_t)(rb / 16);
@@ -82,13 +88,11 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
   HNV_CHECK(pool.get(&pv, (size_t)lv.n * rb));
   HNV_CHECK(pool.get(&pe, (size_t)lv.m * rb));
   unsigned* dmax = reinterpret_cast<unsigned*>(g->d_buf + 32);
-  int32_t done = 0;
-  float delta = 0.f;
   // Iterates alternate between the caller's buffers and these: a sweep writes
   // the other pair, so the previous iterate needs no copy (copying it took 30
   // of 330 us a sweep at 200K nodes, d = 64).
   void *cv = z_v, *ce = z_e, *ov = pv, *oe = pe;
-  for (int it = 0; it < max_sweeps; ++it) {
+  for (int it = done; it < max_sweeps; ++it) {
     HNV_CHECK(refine_sweep_into(g, level, cv, ce, ov, oe, dtype, d, omega, mode, s));
     std::swap(cv, ov);
     std::swap(ce, oe);

@@ -57,7 +57,7 @@ enum : int32_t {
 
 void note_launch();
 void note_launches(int64_t k);   // k kernels at once (a replayed CUDA graph)
-int num_sms();
+int num_sms();   // of the current device
 
 // Launches kernel<<<grid, block, smem, s>>>(args...) and counts it. A launch
 // with no blocks is skipped.
@@ -439,6 +439,7 @@ struct hnv_graph {
   // hnv_selftest_team_timeout: of the one-launch calls' barriers
   uint64_t team_wait_ns = hnv::kTeamWaitNs;
   int32_t team_stop_at = 0;
+  bool team_refuse = false;      // hnv_selftest_team_refuse
   float* partials = nullptr;     // split-row partial sums
   size_t partials_bytes = 0;
   float* jacobi_tmp = nullptr;   // Jacobi: next hyperedge rows
@@ -602,11 +603,17 @@ void team_level(const Level& lv, int64_t row0, TeamLevel* out);
 int team_blocks_for(const Level& lv, int dtype, int d);
 // Estimated microseconds of one sweep of a level by a team of `blocks`.
 double team_sweep_us(const Level& lv, int dtype, int d, int blocks);
+// kTeamRefused: the device would not run the blocks at once (it has fewer SMs
+// for this process than it says, or no cooperative launches), and nothing was
+// launched; the caller takes the per-launch path.
+constexpr int kTeamRefused = 1;
+bool team_refused(cudaError_t e);   // the error that says so
 int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s);
 // The team path applies at all (it is off while phases are timed, and where
 // an environment switch asks for another gather).
 bool team_enabled(int d);
-// Levels top .. bottom of g (all of which fit) in one launch on s.
+// Levels top .. bottom of g (all of which fit) in one launch on s, or
+// kTeamRefused.
 // With eps, the stopping rule: the caller brings the kTeamWords words, and
 // the sweeps done, the last change and whether a wait gave up are left at words
 // + kTeamResult.

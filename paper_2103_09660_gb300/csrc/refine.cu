@@ -500,6 +500,7 @@ bool team_ready(hnv_graph* g, cudaStream_t s) {
 
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
              cudaStream_t s, const float* eps, int32_t* words) {
+  if (g->team_refuse) return kTeamRefused;
   TempPool pool(s);
   if (!words) HNV_CHECK(pool.get(&words, kTeamWords));
   int64_t chunks = 1, m = 1;
@@ -591,7 +592,8 @@ int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d
     t.top = t.bottom = level;
     t.zv0 = static_cast<uint4*>(z_v);
     t.ze0 = static_cast<uint4*>(z_e);
-    return team_run(g, t, dtype, d, omega, sweeps, mode, s);
+    const int rc = team_run(g, t, dtype, d, omega, sweeps, mode, s);
+    if (rc != kTeamRefused) return rc;
   }
   HalfSweep E, V;
   HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, s));

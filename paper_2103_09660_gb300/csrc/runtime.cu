@@ -57,16 +57,18 @@ void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 void note_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
+constexpr int kMaxDevices = 64;
+
 int num_sms() {
-  static int cached = 0;
-  if (cached == 0) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 148;
-    cached = v;
-  }
-  return cached;
+  static std::atomic<int> cached[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) dev = 0;
+  int v = dev < kMaxDevices ? cached[dev].load(std::memory_order_relaxed) : 0;
+  if (v > 0) return v;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+    return 148;
+  if (dev < kMaxDevices) cached[dev].store(v, std::memory_order_relaxed);
+  return v;
 }
 
 unsigned grid_for(int64_t items, int64_t per_block, int waves) {
@@ -90,15 +92,14 @@ static void* g_alloc_ctx = nullptr;
 // next (the default pool returns it to the system at every synchronisation,
 // and a V-cycle step allocates and frees about 1.5 GB at the 1M-node size).
 // hnv_release_cached_memory() gives the unused part back.
-constexpr int kMaxPoolDevices = 64;
 static std::mutex g_pool_mu;
-static cudaMemPool_t g_pools[kMaxPoolDevices] = {nullptr};
+static cudaMemPool_t g_pools[kMaxDevices] = {nullptr};
 
 static int device_pool(cudaMemPool_t* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_status(e, "cudaGetDevice");
-  if (dev < 0 || dev >= kMaxPoolDevices) HNV_FAIL(HNV_ERR_INVALID_ARG, "device %d", dev);
+  if (dev < 0 || dev >= kMaxDevices) HNV_FAIL(HNV_ERR_INVALID_ARG, "device %d", dev);
   std::lock_guard<std::mutex> lk(g_pool_mu);
   if (!g_pools[dev]) {
     cudaMemPoolProps props = {};
@@ -227,7 +228,7 @@ int hnv_set_allocator(hnv_alloc_fn alloc_fn, hnv_free_fn free_fn, void* ctx) {
 
 int hnv_release_cached_memory(void) {
   std::lock_guard<std::mutex> lk(g_pool_mu);
-  for (int d = 0; d < kMaxPoolDevices; ++d) {
+  for (int d = 0; d < kMaxDevices; ++d) {
     if (!g_pools[d]) continue;
     const cudaError_t e = cudaMemPoolTrimTo(g_pools[d], 0);
     if (e != cudaSuccess) return cuda_status(e, "cudaMemPoolTrimTo");

@@ -565,11 +565,12 @@ int launch_team(const TeamArgs& a, int teams, cudaStream_t s) {
   void* params[] = {&args};
   const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)(teams * a.blocks)),
                                                     dim3(kTeamThreads), params, 0, s);
-  note_launch();
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (team_refused(e)) return kTeamRefused;
     return cuda_status(e, "team_kernel");
   }
+  note_launch();
   return HNV_OK;
 }
 
@@ -583,6 +584,10 @@ int launch_team_dispatch(const TeamArgs& a, int teams, cudaStream_t s) {
 }
 
 }  // namespace
+
+bool team_refused(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported;
+}
 
 void team_level(const Level& lv, int64_t row0, TeamLevel* out) {
   *out = TeamLevel();

@@ -195,3 +195,82 @@ def test_two_streams_on_one_graph(H):
         G.sync_status()
         for k in range(2):
             assert torch.equal(pairs[k][0], want[k][0]) and torch.equal(pairs[k][1], want[k][1])
+
+
+@pytest.mark.parametrize("dtname,d", [("f32", 36), ("bf16", 72)])
+def test_refused_launch_takes_the_per_launch_path(H, dtname, d):
+    """Where the device refuses the cooperative launch, every entry point that
+    would use it runs a launch per half-sweep instead and gives the same bits."""
+    import torch
+    dt = torch.float32 if dtname == "f32" else torch.bfloat16
+    hg = _hub_graph(4200, [129, 300])
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    with H.Graph.from_hypergraph(hg) as G:
+        L = G.coarsen(min_nodes=30, max_levels=3)
+        top = G.level_info(L - 1)
+        zc = torch.randn((top[0] + top[1], d), generator=g, device="cuda").to(dt)
+        zv, ze = torch.empty((hg.n, d), dtype=dt, device="cuda"), \
+            torch.empty((hg.m, d), dtype=dt, device="cuda")
+        z = torch.randn((hg.n + hg.m, d), generator=g, device="cuda").to(dt)
+
+        def work():
+            out, n = [], []
+
+            def call(f):
+                before = H.kernel_launch_count()
+                out.extend(f())
+                torch.cuda.synchronize()
+                n.append(H.kernel_launch_count() - before)
+
+            def vcycle():
+                zv.fill_(float("nan"))
+                ze.fill_(float("nan"))
+                G.vcycle(zc, zv, ze, 0.3, 3)
+                return zv.clone(), ze.clone()
+            call(vcycle)
+            for mode in (H.SWEEP_TWO_PHASE, H.SWEEP_JACOBI):
+                def refine():
+                    v, e = z[:hg.n].clone(), z[hg.n:].clone()
+                    G.refine(0, v, e, 0.3, 3, mode)
+                    return v, e
+
+                def until():
+                    v, e = z[:hg.n].clone(), z[hg.n:].clone()
+                    return (v, e) + tuple(G.refine_until(0, v, e, 0.3, 12, 0.2, mode))
+                call(refine)
+                call(until)
+            G.sync_status()
+            return out, n
+
+        def batch(graph):
+            zv.fill_(float("nan"))
+            ze.fill_(float("nan"))
+            before = H.kernel_launch_count()
+            B.vcycle(zc, zv, ze, 0.3, 3, use_cuda_graph=graph)
+            torch.cuda.synchronize()
+            return zv.clone(), ze.clone(), H.kernel_launch_count() - before
+        want, one = work()
+        assert one == [1] * 5
+        assert H.lib().hnv_selftest_team_refuse(G.handle, 1) == 0
+        got, many = work()
+        assert all(k > 1 for k in many)
+        same = lambda a, b: torch.equal(a, b) if torch.is_tensor(a) else a == b
+        assert all(same(a, b) for a, b in zip(got, want))
+        for graph in (False, True):
+            if d % 8:
+                break
+            with H.Batch([G]) as B:
+                first = batch(graph)
+                again = batch(graph)
+                assert first[2] > again[2] > 1           # the first call builds the lists
+                for r in (first, again):
+                    assert torch.equal(r[0], want[0]) and torch.equal(r[1], want[1])
+            with H.Batch([G]) as B:                      # the tuner meets it first
+                assert B.autotune(H.BF16, d)["lanes_a"] > 0
+                r = batch(graph)
+                assert torch.equal(r[0], want[0]) and torch.equal(r[1], want[1])
+        assert H.lib().hnv_selftest_team_refuse(G.handle, 0) == 0
+        got, back = work()
+        assert back == one and all(same(a, b) for a, b in zip(got, want))
+        assert H.lib().hnv_selftest_team_refuse(None, 1) == -1
