@@ -35,9 +35,10 @@ void destroy_graph(hnv_graph* g) {
   dev_free(g->team_levels, s);
   dev_free(g->partials, s);
   dev_free(g->jacobi_tmp, s);
-  dev_free(g->d_err, s);
-  dev_free(g->d_buf, s);
+  dev_free(g->d_words, s);
   cudaStreamSynchronize(s);
+  for (TeamSlot& t : g->team_slots)
+    if (t.done) cudaEventDestroy(t.done);
   for (int i = 0; i < 2; ++i) {
     if (g->aux[i]) {
       cudaStreamSynchronize(g->aux[i]);
@@ -225,8 +226,14 @@ int hnv_build_incidence(int32_t n_nodes, int32_t n_edges, const int64_t* edge_pt
       rc = HNV_ERR_OOM;
       break;
     }
-    if ((rc = dev_alloc((void**)&g->d_err, sizeof(int32_t), s)) != HNV_OK) break;
-    if ((rc = dev_alloc((void**)&g->d_buf, 64 * sizeof(int32_t), s)) != HNV_OK) break;
+    // the error word, the scratch words and the sets of team words, each on
+    // lines of its own
+    if ((rc = dev_alloc((void**)&g->d_words, (96 + kTeamSlots * kTeamWords) * sizeof(int32_t),
+                        s)) != HNV_OK)
+      break;
+    g->d_err = g->d_words;
+    g->d_buf = g->d_words + 32;
+    g->team_words = g->d_words + 96;
     {
       cudaError_t e = cudaEventCreateWithFlags(&g->fork_ev, cudaEventDisableTiming);
       for (int i = 0; i < 2 && e == cudaSuccess; ++i) {

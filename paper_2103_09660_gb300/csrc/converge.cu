@@ -55,9 +55,7 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
   float delta = 0.f;
   if (max_sweeps > 0 && team_enabled(d) && team_fits(lv, dtype, d) && team_ready(g, s)) {
     // sweeps, changes and the test in one launch (at most kTeamMaxSweeps each)
-    TempPool pool(s);
-    int32_t* words = nullptr;
-    HNV_CHECK(pool.get(&words, kTeamWords));
+    const int32_t* result = nullptr;
     int32_t res[3] = {0, 0, 0};
     int rc = HNV_OK;
     do {
@@ -66,10 +64,10 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
       t.zv0 = static_cast<uint4*>(z_v);
       t.ze0 = static_cast<uint4*>(z_e);
       const int k = max_sweeps - done < kTeamMaxSweeps ? max_sweeps - done : kTeamMaxSweeps;
-      rc = team_run(g, t, dtype, d, omega, k, mode, s, &eps, words);
+      rc = team_run(g, t, dtype, d, omega, k, mode, s, &eps, &result);
       if (rc == kTeamRefused) break;
       HNV_CHECK(rc);
-      HNV_CHECK(read_ints(g, words + kTeamResult, 3, res, s));
+      HNV_CHECK(read_ints(g, result, 3, res, s));
       // in whichever sweep: the rows are then half-written
       if (res[2]) HNV_FAIL(HNV_ERR_TIMEOUT, "a bounded wait of a refinement kernel gave up");
       done += res[0];

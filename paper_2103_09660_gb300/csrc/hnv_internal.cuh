@@ -421,10 +421,23 @@ struct Level {
 struct TeamLevel;
 // Limit of one barrier wait of the team kernel.
 constexpr uint64_t kTeamWaitNs = 4000000000ull;
-// 32-bit words a one-graph team launch owns (calls on other streams may run
-// beside it): the barrier line, the stopping rule's 3 running maxima and its 3
-// results.
+// 32-bit words a one-graph team launch owns: the barrier line, the stopping
+// rule's 3 running maxima and its 3 results.
 constexpr int kTeamWords = 64, kTeamDelta = 32, kTeamResult = 36;
+
+// Whose launches use a graph's k-th set of these words. Launches on one stream
+// follow each other and share a set; launches on other streams may run beside
+// them (a graph without split rows shares no other scratch), and so may the
+// replays of a capture, whose set is its own for the graph's lifetime. A call
+// neither allocates the words nor gives them back.
+struct TeamSlot {
+  bool taken = false;
+  unsigned long long stream = 0;    // cudaStreamGetId (not reused); in a capture the handle
+  unsigned long long capture = 0;   // id of the capture, 0: none
+  uint64_t used = 0;                // turn of the last launch (none captured)
+  cudaEvent_t done = nullptr;       // after it: another stream may take the set
+};
+constexpr int kTeamSlots = 32, kTeamStreamSlots = 8;   // sets; of them kept for streams
 
 }  // namespace hnv
 
@@ -435,6 +448,11 @@ struct hnv_graph {
   int32_t* d_err = nullptr;      // device error word
   int32_t* h_buf = nullptr;      // pinned host scratch (64 ints)
   int32_t* d_buf = nullptr;      // device scratch (64 ints)
+  // one allocation: d_err, d_buf and kTeamSlots x kTeamWords team_words
+  int32_t* d_words = nullptr;
+  int32_t* team_words = nullptr;
+  hnv::TeamSlot team_slots[hnv::kTeamSlots];
+  uint64_t team_turn = 0;
   hnv::TeamLevel* team_levels = nullptr;   // device, one per level (team.cu)
   // hnv_selftest_team_timeout: of the one-launch calls' barriers
   uint64_t team_wait_ns = hnv::kTeamWaitNs;
@@ -614,11 +632,10 @@ int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s);
 bool team_enabled(int d);
 // Levels top .. bottom of g (all of which fit) in one launch on s, or
 // kTeamRefused.
-// With eps, the stopping rule: the caller brings the kTeamWords words, and
-// the sweeps done, the last change and whether a wait gave up are left at words
-// + kTeamResult.
+// With eps, the stopping rule: the sweeps done, the last change and whether a
+// wait gave up are left at *result (device; until the next launch on s).
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
-             cudaStream_t s, const float* eps = nullptr, int32_t* words = nullptr);
+             cudaStream_t s, const float* eps = nullptr, const int32_t** result = nullptr);
 // Uploads the hierarchy's TeamLevels on first use (dropped with the
 // hierarchy). False where it cannot: under capture, or out of memory; the
 // caller then takes the per-launch path.

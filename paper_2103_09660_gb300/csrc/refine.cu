@@ -498,11 +498,61 @@ bool team_ready(hnv_graph* g, cudaStream_t s) {
   return true;
 }
 
+namespace {
+
+// The set of words of a launch on s, or kTeamRefused: every set for captures is
+// taken, or the stream's state cannot be read.
+int team_slot(hnv_graph* g, cudaStream_t s, int* slot) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  unsigned long long capture = 0, stream = 0;
+  cudaError_t e = cudaStreamGetCaptureInfo(s, &cap, &capture);
+  if (cap == cudaStreamCaptureStatusNone) {
+    capture = 0;
+    if (e == cudaSuccess) e = cudaStreamGetId(s, &stream);
+  } else {
+    // (cudaStreamGetId would end the capture; its streams live as long as it)
+    stream = (unsigned long long)reinterpret_cast<uintptr_t>(s);
+  }
+  if (e != cudaSuccess || cap == cudaStreamCaptureStatusInvalidated) {
+    cudaGetLastError();
+    return kTeamRefused;
+  }
+  TeamSlot* t = g->team_slots;
+  int free_k = -1, oldest = -1, streams = 0, captures = 0;
+  for (int k = 0; k < kTeamSlots; ++k) {
+    if (!t[k].taken) {
+      if (free_k < 0) free_k = k;
+    } else if (t[k].stream == stream && t[k].capture == capture) {
+      *slot = k;
+      return HNV_OK;
+    } else if (t[k].capture) {
+      ++captures;
+    } else {
+      ++streams;
+      if (oldest < 0 || t[k].used < t[oldest].used) oldest = k;
+    }
+  }
+  if (capture) {
+    if (captures >= kTeamSlots - kTeamStreamSlots) return kTeamRefused;
+  } else if (streams >= kTeamStreamSlots) {
+    // another stream's: its last launch comes first
+    HNV_CUDA(cudaStreamWaitEvent(s, t[oldest].done, 0));
+    free_k = oldest;
+  } else if (!t[free_k].done) {
+    HNV_CUDA(cudaEventCreateWithFlags(&t[free_k].done, cudaEventDisableTiming));
+  }
+  t[free_k].taken = true;
+  t[free_k].stream = stream;
+  t[free_k].capture = capture;
+  *slot = free_k;
+  return HNV_OK;
+}
+
+}  // namespace
+
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
-             cudaStream_t s, const float* eps, int32_t* words) {
+             cudaStream_t s, const float* eps, const int32_t** result) {
   if (g->team_refuse) return kTeamRefused;
-  TempPool pool(s);
-  if (!words) HNV_CHECK(pool.get(&words, kTeamWords));
   int64_t chunks = 1, m = 1;
   int blocks = 1;
   for (int l = t.bottom; l <= t.top; ++l) {
@@ -514,6 +564,10 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
   HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes, sizeof(float) * (size_t)chunks * d, s));
   if (mode == HNV_SWEEP_JACOBI)
     HNV_CHECK(ensure_scratch(&g->jacobi_tmp, &g->jacobi_bytes, elem_size(dtype) * (size_t)m * d, s));
+  int k = 0;
+  HNV_CHECK(team_slot(g, s, &k));
+  TeamSlot& slot = g->team_slots[k];
+  int32_t* words = g->team_words + k * kTeamWords;
   HNV_CUDA(cudaMemsetAsync(words, 0, sizeof(int32_t) * kTeamWords, s));
   t.levels = g->team_levels;
   t.err = g->d_err;
@@ -533,8 +587,14 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
     a.delta = reinterpret_cast<unsigned*>(words + kTeamDelta);
     a.result = words + kTeamResult;
     a.eps = *eps;
+    *result = a.result;
   }
-  return team_launch(a, 1, dtype, d, s);
+  HNV_CHECK(team_launch(a, 1, dtype, d, s));
+  if (!slot.capture) {
+    slot.used = ++g->team_turn;
+    HNV_CUDA(cudaEventRecord(slot.done, s));
+  }
+  return HNV_OK;
 }
 
 namespace {

@@ -274,3 +274,128 @@ def test_refused_launch_takes_the_per_launch_path(H, dtname, d):
         got, back = work()
         assert back == one and all(same(a, b) for a, b in zip(got, want))
         assert H.lib().hnv_selftest_team_refuse(None, 1) == -1
+
+
+class _Refuser:
+    """A device allocator hook that grants nothing and counts the requests."""
+
+    def __init__(self, H):
+        import ctypes
+        self.H, self.calls = H, []
+        AF = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p)
+        FF = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+        self.fns = AF(lambda n, s, ctx: self.calls.append(n)), \
+            FF(lambda p, s, ctx: self.calls.append(-1))
+        self.ptrs = [ctypes.cast(f, ctypes.c_void_p) for f in self.fns]
+
+    def __enter__(self):
+        assert self.H.lib().hnv_set_allocator(self.ptrs[0], self.ptrs[1], None) == 0
+        return self
+
+    def __exit__(self, *exc):
+        assert self.H.lib().hnv_set_allocator(None, None, None) == 0
+
+
+def test_warmed_calls_allocate_nothing(H):
+    """After the first call of its kind (which may allocate scratch), refining a
+    small level asks the allocator for nothing, also under capture: a captured
+    call then owns everything that its replays use."""
+    import torch
+    hg = _hub_graph(4200, [129, 300])
+    with H.Graph.from_hypergraph(hg) as G:
+        z = torch.randn((hg.n + hg.m, 36), device="cuda")
+
+        def calls():
+            out = []
+            for mode in (H.SWEEP_TWO_PHASE, H.SWEEP_JACOBI):
+                v, e = z[:hg.n].clone(), z[hg.n:].clone()
+                G.refine(0, v, e, 0.3, 3, mode)
+                out += [v, e]
+                v, e = z[:hg.n].clone(), z[hg.n:].clone()
+                G.refine_until(0, v, e, 0.3, 3, -1.0, mode)
+                out += [v, e]
+            return out
+        want = calls()
+        v, e = z[:hg.n].clone(), z[hg.n:].clone()
+        graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with _Refuser(H) as hook:
+            got = calls()
+            with torch.cuda.graph(graph, stream=s):
+                H.hnv_refine(G.handle, 0, v, e, 0.3, 3, H.SWEEP_TWO_PHASE, s)
+            assert hook.calls == []
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+        for _ in range(2):
+            v.copy_(z[:hg.n])
+            e.copy_(z[hg.n:])
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(v, want[0]) and torch.equal(e, want[1])
+
+
+def _rows_up_to_128():
+    """A hypergraph without split rows (calls on it share no scratch)."""
+    hg = _hub_graph(40, [])
+    edges = [hg.edge_nodes[hg.edge_ptr[e]:hg.edge_ptr[e + 1]] for e in range(hg.m)
+             if hg.edge_ptr[e + 1] - hg.edge_ptr[e] <= 128]
+    ptr = np.concatenate([[0], np.cumsum([len(e) for e in edges])]).astype(np.int64)
+    return hg.n, len(edges), ptr, np.concatenate(edges).astype(np.int32)
+
+
+def test_more_streams_than_sets_of_barrier_words(H):
+    """Launches on 20 streams, three rounds of them: a set of words that goes to
+    another stream is free by then."""
+    import torch
+    n, m, ptr, nodes = _rows_up_to_128()
+    with H.Graph(n, m, ptr, nodes) as G:
+        z = torch.randn((20, n + m, 16), device="cuda")
+
+        def fresh():
+            return [(z[k, :n].clone(), z[k, n:].clone()) for k in range(20)]
+        want = fresh()
+        for v, e in want:
+            G.refine(0, v, e, 0.3, 60)
+        got = fresh()
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in range(20)]
+        for _ in range(3):
+            for s, (v, e) in zip(streams, got):
+                H.hnv_refine(G.handle, 0, v, e, 0.3, 20, H.SWEEP_TWO_PHASE, s)
+        torch.cuda.synchronize()
+        G.sync_status()
+        for a, b in zip(got, want):
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+def test_more_captures_than_sets_of_barrier_words(H):
+    """Every captured branch has a set of its own; when none is left a capture
+    takes the per-launch path. All replay beside each other."""
+    import torch
+    n, m, ptr, nodes = _rows_up_to_128()
+    with H.Graph(n, m, ptr, nodes) as G:
+        z = torch.randn((60, n + m, 16), device="cuda")
+        want = [(z[k, :n].clone(), z[k, n:].clone()) for k in range(60)]
+        for v, e in want:
+            G.refine(0, v, e, 0.3, 20)
+        got = [(z[k, :n].clone(), z[k, n:].clone()) for k in range(60)]
+        torch.cuda.synchronize()
+        graphs, launches = [], []
+        a, b = torch.cuda.Stream(), torch.cuda.Stream()
+        for k in range(0, 60, 2):
+            graphs.append(torch.cuda.CUDAGraph())
+            before = H.kernel_launch_count()
+            with torch.cuda.graph(graphs[-1], stream=a):
+                b.wait_stream(a)
+                H.hnv_refine(G.handle, 0, *got[k], 0.3, 20, H.SWEEP_TWO_PHASE, a)
+                H.hnv_refine(G.handle, 0, *got[k + 1], 0.3, 20, H.SWEEP_TWO_PHASE, b)
+                a.wait_stream(b)
+            launches.append(H.kernel_launch_count() - before)
+        assert launches[0] == 2 and launches[-1] > 2
+        streams = [torch.cuda.Stream() for _ in graphs]
+        for s, g in zip(streams, graphs):
+            with torch.cuda.stream(s):
+                g.replay()
+        torch.cuda.synchronize()
+        G.sync_status()
+        for x, y in zip(got, want):
+            assert torch.equal(x[0], y[0]) and torch.equal(x[1], y[1])
