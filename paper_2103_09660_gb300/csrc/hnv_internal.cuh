@@ -85,7 +85,9 @@ void dev_free(void* p, cudaStream_t s);
 
 // Temporary device buffers released (stream-ordered) when the pool dies.
 // Small ones are cut from slabs: a level of a 2,000-node graph asks for about
-// 25 of them, and each allocation with its release costs the host 2-3 us.
+// 25 of them, and each allocation with its release costs the host 2-3 us. Where
+// a slab cannot be had (an allocator hook with little memory), each is
+// allocated by itself.
 class TempPool {
  public:
   explicit TempPool(cudaStream_t s) : s_(s) {}
@@ -97,20 +99,25 @@ class TempPool {
   template <typename T>
   int get(T** out, size_t count) {
     const size_t bytes = ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
-    if (bytes <= kSlab / 4) {
-      if (left_ < bytes) {
-        void* p = nullptr;
-        HNV_CHECK(dev_alloc(&p, kSlab, s_));
-        ptrs_.push_back(p);
-        at_ = static_cast<char*>(p);
-        left_ = kSlab;
-      }
-      *out = reinterpret_cast<T*>(at_);
-      at_ += bytes;
-      left_ -= bytes;
-      return HNV_OK;
-    }
     void* p = nullptr;
+    if (bytes <= kSlab / 4 && !no_slabs_) {
+      if (left_ < bytes) {
+        if (dev_alloc(&p, kSlab, s_) == HNV_OK) {
+          ptrs_.push_back(p);
+          at_ = static_cast<char*>(p);
+          left_ = kSlab;
+        } else {
+          clear_error_detail();
+          no_slabs_ = true;
+        }
+      }
+      if (!no_slabs_) {
+        *out = reinterpret_cast<T*>(at_);
+        at_ += bytes;
+        left_ -= bytes;
+        return HNV_OK;
+      }
+    }
     HNV_CHECK(dev_alloc(&p, bytes, s_));
     ptrs_.push_back(p);
     *out = static_cast<T*>(p);
@@ -122,6 +129,7 @@ class TempPool {
   cudaStream_t s_;
   char* at_ = nullptr;
   size_t left_ = 0;
+  bool no_slabs_ = false;
   std::vector<void*> ptrs_;
 };
 

@@ -88,3 +88,38 @@ def test_means_and_cosines(H, k):
         assert_hierarchy_equal(G, h)
         for ell, F in enumerate(h.features):
             np.testing.assert_array_equal(G.level_features(ell), F)
+
+
+def test_build_with_an_allocator_of_small_blocks(H):
+    """An allocator hook that grants no request above 64 KB: the temporaries of
+    a small graph, which share slabs where those can be had, need no more."""
+    import ctypes
+    import torch
+    held, refused = [], []
+
+    def alloc(nbytes, s, ctx):
+        if nbytes > 65536:
+            refused.append(nbytes)
+            return None
+        held.append(torch.empty(nbytes, dtype=torch.uint8, device="cuda"))
+        return held[-1].data_ptr()
+    AF = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p)
+    FF = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+    fns = AF(alloc), FF(lambda p, s, ctx: None)
+    hg = hypergen.random_small_hypergraph(np.random.default_rng(3), 200, 150, 6)
+    X = np.random.default_rng(4).standard_normal((200, 5)).astype(np.float32)
+    assert H.lib().hnv_set_allocator(*[ctypes.cast(f, ctypes.c_void_p) for f in fns], None) == 0
+    try:
+        for policy in (O.ASSIGN_HASH, O.ASSIGN_COSINE):
+            h = O.coarsen(oracle_level0(hg), O.CoarsenParams(
+                policy=policy, features=X if policy == O.ASSIGN_COSINE else None, min_nodes=5,
+                max_levels=4, seed=1))
+            with H.Graph.from_hypergraph(hg) as G:
+                if policy == O.ASSIGN_COSINE:
+                    G.set_node_features(X)
+                G.coarsen(policy=policy, min_nodes=5, max_levels=4, seed=1)
+                assert_hierarchy_equal(G, h)
+        torch.cuda.synchronize()
+    finally:
+        assert H.lib().hnv_set_allocator(None, None, None) == 0
+    assert set(refused) == {512 * 1024}          # slabs only
