@@ -132,7 +132,7 @@ int vcycle_impl(hnv_graph* g, const void* z_coarsest, void* z_v_out, void* z_e_o
   // the levels from the coarsest down that are small enough take one launch
   int first_big = L;
   if (on_device && team_enabled(d) && sweeps <= kTeamMaxSweeps && team_fits(top, dtype, d) &&
-      team_ready(g, s))
+      team_ready(g))
     while (first_big >= 0 && team_fits(g->levels[first_big], dtype, d)) --first_big;
   if (first_big < L) {
     const int b = first_big + 1;
@@ -281,6 +281,8 @@ int hnv_build_incidence(int32_t n_nodes, int32_t n_edges, const int64_t* edge_pt
     rc = build_level0(g, n_nodes, n_edges, d_ptr, d_nodes, d_w, &g->levels[0]);
   } while (0);
   if (rc == HNV_OK) {
+    std::vector<TeamLevel> host;
+    team_upload(g, &host);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) rc = cuda_status(e, "cudaStreamSynchronize (build)");
   }
@@ -351,6 +353,8 @@ int hnv_coarsen(hnv_graph* g, const hnv_coarsen_params* p, int32_t* n_levels) {
       g->levels.push_back(nxt);
     }
   }
+  std::vector<TeamLevel> host;
+  team_upload(g, &host);
   HNV_CUDA(cudaStreamSynchronize(s));
   if (n_levels) *n_levels = (int32_t)g->levels.size();
   return HNV_OK;

@@ -438,14 +438,14 @@ void drop_deal(const hnv_batch* b, BatchDeal& D, cudaStream_t s) {
 // The coarsest level of each graph, -1 for those the teams run: the graphs all
 // of whose levels are small, with the per-class setting and at most
 // kTeamMaxSweeps sweeps.
-std::vector<int> deal_teams(const hnv_batch* b, int dt, int d, int sweeps, cudaStream_t s) {
+std::vector<int> deal_teams(const hnv_batch* b, int dt, int d, int sweeps) {
   std::vector<int> top = b->top;
   if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && !b->no_teams && team_enabled(d) &&
       sweeps <= kTeamMaxSweeps)
     for (size_t i = 0; i < b->graphs.size(); ++i) {
       bool fits = true;
       for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
-      if (fits && team_ready(b->graphs[i], s)) top[i] = -1;
+      if (fits && team_ready(b->graphs[i])) top[i] = -1;
     }
   return top;
 }
@@ -1058,7 +1058,7 @@ int vcycle_once(hnv_batch* b, const void* z_coarsest, void* z_v_out, void* z_e_o
                 float omega, int sweeps, int use_cuda_graph, cudaStream_t s) {
   cudaStream_t cs = b->cap_stream;
   const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
-  BatchDeal& D = use_deal(b, deal_teams(b, dt, d, sweeps, cs), cs);
+  BatchDeal& D = use_deal(b, deal_teams(b, dt, d, sweeps), cs);
   if (!D.plans_ready || D.plans_row_bytes != rb) {
     free_steps(b, D, cs);   // built from the plans
     HNV_CHECK(build_plans(b, D, rb, cs));
@@ -1201,7 +1201,7 @@ int hnv_batch_autotune(hnv_batch* b, hnv_dtype dt, int d, float omega, hnv_batch
   const int old_kernel = b->kernel;
   const std::vector<int> old_lanes(b->lanes, b->lanes + 3);
   b->kernel = HNV_BATCH_KERNEL_PER_CLASS;
-  const std::vector<int> teams_top = deal_teams(b, dt, d, 1, s);
+  const std::vector<int> teams_top = deal_teams(b, dt, d, 1);
   const int64_t teamed = std::count(teams_top.begin(), teams_top.end(), -1);
   const std::vector<int64_t> key = tune_key(b, dt, d, teamed);
   PlanShape best_shape = b->shape;

@@ -53,7 +53,7 @@ int refine_level_until(hnv_graph* g, int level, void* z_v, void* z_e, int dtype,
   const Level& lv = g->levels[level];
   int32_t done = 0;
   float delta = 0.f;
-  if (max_sweeps > 0 && team_enabled(d) && team_fits(lv, dtype, d) && team_ready(g, s)) {
+  if (max_sweeps > 0 && team_enabled(d) && team_fits(lv, dtype, d) && team_ready(g)) {
     // sweeps, changes and the test in one launch (at most kTeamMaxSweeps each)
     const int32_t* result = nullptr;
     int32_t res[3] = {0, 0, 0};

@@ -644,10 +644,12 @@ bool team_enabled(int d);
 // wait gave up are left at *result (device; until the next launch on s).
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
              cudaStream_t s, const float* eps = nullptr, const int32_t** result = nullptr);
-// Uploads the hierarchy's TeamLevels on first use (dropped with the
-// hierarchy). False where it cannot: under capture, or out of memory; the
-// caller then takes the per-launch path.
-bool team_ready(hnv_graph* g, cudaStream_t s);
+// Uploads the TeamLevels of g's levels (from *host, which has to last until the
+// graph's stream is next synchronised; the calls that build levels end with
+// that, so later calls on any stream find them). Without memory for them
+// g->team_levels stays null, and the per-launch path is taken.
+void team_upload(hnv_graph* g, std::vector<TeamLevel>* host);
+inline bool team_ready(const hnv_graph* g) { return g->team_levels != nullptr; }
 int forced_panels();   // HNV_PANELS, or -1
 
 // Two-phase sweeps whose split-row partial sums go to caller-provided

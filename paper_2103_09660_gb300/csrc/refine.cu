@@ -471,31 +471,26 @@ int ensure_scratch(float** p, size_t* have, size_t need, cudaStream_t s) {
 
 bool team_enabled(int d) { return !timing_on() && !use_tma(d) && forced_panels() < 1; }
 
-bool team_ready(hnv_graph* g, cudaStream_t s) {
-  if (g->team_levels) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-    return false;
-  std::vector<TeamLevel> h(g->levels.size());
+void team_upload(hnv_graph* g, std::vector<TeamLevel>* host) {
+  cudaStream_t s = g->stream;
+  host->resize(g->levels.size());
   int64_t row0 = 0;
-  for (size_t l = 0; l < h.size(); ++l) {
-    team_level(g->levels[l], row0, &h[l]);
+  for (size_t l = 0; l < host->size(); ++l) {
+    team_level(g->levels[l], row0, &(*host)[l]);
     row0 += (int64_t)g->levels[l].n + g->levels[l].m;
   }
+  const size_t bytes = sizeof(TeamLevel) * host->size();
   TeamLevel* t = nullptr;
-  if (dev_alloc((void**)&t, sizeof(TeamLevel) * h.size(), s) != HNV_OK) {
+  if (dev_alloc((void**)&t, bytes, s) != HNV_OK) {
     clear_error_detail();
-    return false;
+    return;
   }
-  // done before any stream reads it (later calls may come on other streams)
-  if (cudaMemcpyAsync(t, h.data(), sizeof(TeamLevel) * h.size(), cudaMemcpyHostToDevice, s) !=
-          cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess) {
+  if (cudaMemcpyAsync(t, host->data(), bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) {
+    cudaGetLastError();
     dev_free(t, s);
-    return false;
+    return;
   }
   g->team_levels = t;
-  return true;
 }
 
 namespace {
@@ -647,7 +642,7 @@ int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d
   NvtxRange nvtx("hnv refine level %d (%d sweeps)", level, sweeps);
   Level& lv = g->levels[level];
   if (sweeps > 0 && sweeps <= kTeamMaxSweeps && team_enabled(d) && team_fits(lv, dtype, d) &&
-      team_ready(g, s)) {
+      team_ready(g)) {
     TeamGraph t;
     t.top = t.bottom = level;
     t.zv0 = static_cast<uint4*>(z_v);

@@ -1,8 +1,8 @@
 """Small graphs run whole V-cycles in one cooperative launch (team.cu). Every
 row is summed in the order of the per-launch kernels, so both paths give the
 same bits. Phase timing needs a launch per half-sweep and so selects the
-per-launch path; a graph that is too large for the one-launch path, or a
-capture before its first use, takes it as well."""
+per-launch path; a graph that is too large for the one-launch path takes it as
+well."""
 
 import numpy as np
 import pytest
@@ -399,3 +399,35 @@ def test_more_captures_than_sets_of_barrier_words(H):
         G.sync_status()
         for x, y in zip(got, want):
             assert torch.equal(x[0], y[0]) and torch.equal(x[1], y[1])
+
+
+def test_first_call_on_a_hierarchy_does_not_wait(H):
+    """The first call on a new hierarchy is asynchronous like the others: it
+    returns while the stream is still busy with earlier work."""
+    import torch
+    hg = _hub_graph(300, [])
+    d = 32
+    s = torch.cuda.Stream()
+
+    def once(busy):
+        with H.Graph.from_hypergraph(hg) as G:
+            L = G.coarsen(min_nodes=30, max_levels=3)
+            top = G.level_info(L - 1)
+            g = torch.Generator(device="cuda")
+            g.manual_seed(1)
+            zc = torch.randn((top[0] + top[1], d), generator=g, device="cuda")
+            zv, ze = torch.empty((hg.n, d), device="cuda"), torch.empty((hg.m, d), device="cuda")
+            torch.cuda.synchronize()
+            done = torch.cuda.Event()
+            with torch.cuda.stream(s):
+                if busy:
+                    torch.cuda._sleep(600_000_000)       # about 0.3 s
+                done.record()
+            H.hnv_vcycle(G.handle, zc, zv, ze, 0.5, 3, H.SWEEP_TWO_PHASE, s)
+            early = not done.query()
+            torch.cuda.synchronize()
+            return early, zv, ze
+    want = once(False)                                   # (loads the kernels)
+    got = once(True)
+    assert got[0]
+    assert torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
