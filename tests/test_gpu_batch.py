@@ -4,6 +4,8 @@ order as the single-graph kernels (the order does not depend on lanes per
 row, row-class boundaries or the graph's position in the batch), so the
 batched results equal the per-graph ones bit for bit."""
 
+import os
+
 import numpy as np
 import pytest
 
@@ -218,6 +220,12 @@ def _launches(H, f):
     return H.kernel_launch_count() - before
 
 
+# another gather asked for in the environment turns the teams off
+needs_teams = pytest.mark.skipif(
+    bool(os.environ.get("HNV_PANELS")) or os.environ.get("HNV_GATHER") == "tma",
+    reason="no teams with this environment")
+
+
 class _StepLists:
     """Phase timing selects a launch per half-sweep: every graph in the step
     lists of the batch, and the per-launch path for a single graph."""
@@ -233,6 +241,7 @@ class _StepLists:
         self.H.timing_reset()
 
 
+@needs_teams
 @pytest.mark.parametrize("dtname,d", [("f32", 8), ("f32", 64), ("bf16", 64), ("bf16", 512)])
 def test_teams_and_step_lists_give_the_same_bits(H, dtname, d):
     """Small graphs run by teams in one launch, and lined up in the step lists
@@ -270,6 +279,7 @@ def test_teams_and_step_lists_give_the_same_bits(H, dtname, d):
         G.close()
 
 
+@needs_teams
 @pytest.mark.parametrize("dtname,d", [("f32", 256), ("bf16", 512)])
 def test_batch_of_teams_and_stepped_graphs(H, dtname, d):
     """One graph too large for a team among small ones; calls of more sweeps
@@ -348,6 +358,7 @@ class _Allocator:
         assert self.H.lib().hnv_set_allocator(None, None, None) == 0
 
 
+@needs_teams
 @pytest.mark.parametrize("graph", [False, True])
 def test_batch_survives_a_build_that_fails(H, graph):
     """Work lists for another dealing of the graphs (more sweeps than a team's
@@ -387,6 +398,7 @@ def test_batch_survives_a_build_that_fails(H, graph):
             G.close()
 
 
+@needs_teams
 def test_autotune_times_the_step_lists(H):
     """The row classes and lanes only matter to graphs in the step lists: they
     are timed there, also for a batch whose graphs the teams run, and what is
