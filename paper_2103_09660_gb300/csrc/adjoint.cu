@@ -372,22 +372,14 @@ int prepare_level_adjoint(hnv_graph* g, int level, cudaStream_t s) {
   return HNV_OK;
 }
 
-int ensure_partials(hnv_graph* g, int d, cudaStream_t s) {
+int adjoint_partials(hnv_graph* g, int d, TempPool& pool, float** out, cudaStream_t s) {
   int64_t chunks = 1;
   for (const Level& lv : g->levels)
     chunks = std::max<int64_t>(chunks, std::max({(int64_t)lv.planE.n_chunks,
                                                  (int64_t)lv.planV.n_chunks,
                                                  (int64_t)lv.planC.n_chunks}));
   const size_t need = sizeof(float) * (size_t)chunks * d;
-  if (g->partials && g->partials_bytes >= need) return HNV_OK;
-  if (g->partials) dev_free(g->partials, s);
-  g->partials = nullptr;
-  g->partials_bytes = 0;
-  void* p = nullptr;
-  HNV_CHECK(dev_alloc(&p, need, s));
-  g->partials = static_cast<float*>(p);
-  g->partials_bytes = need;
-  return HNV_OK;
+  return graph_scratch(g, &g->partials, &g->partials_bytes, need, pool, out, s);
 }
 
 }  // namespace
@@ -415,7 +407,9 @@ int vcycle_backward_impl(hnv_graph* g, const float* ckpt, const float* g_v0, con
   const int d4 = d / 4;
   const size_t row = sizeof(float) * (size_t)d;
   for (int l = 0; l <= L; ++l) HNV_CHECK(prepare_level_adjoint(g, l, s));
-  HNV_CHECK(ensure_partials(g, d, s));
+  TempPool pool(s);
+  float* partials = nullptr;
+  HNV_CHECK(adjoint_partials(g, d, pool, &partials, s));
   // omega == 0: every sweep is the identity, and so is its reverse
   const int rsweeps = omega == 0.f ? 0 : sweeps;
   // checkpoint offsets (floats)
@@ -423,7 +417,6 @@ int vcycle_backward_impl(hnv_graph* g, const float* ckpt, const float* g_v0, con
   for (int l = 0; l <= L; ++l)
     off[l + 1] = off[l] + ((size_t)g->levels[l].n + g->levels[l].m) * d;
 
-  TempPool pool(s);
   size_t maxrows = 0, maxm = 1, maxn = 1;
   for (const Level& lv : g->levels) {
     maxrows = std::max(maxrows, (size_t)lv.n + lv.m);
@@ -473,10 +466,10 @@ int vcycle_backward_impl(hnv_graph* g, const float* ckpt, const float* g_v0, con
       if (m > 0)  // z_e^i = (1-w) z_e^{i-1} + w (1/|e|) sum_{v in e} z_v^{i-1}
         HNV_CHECK(gather_rows_f32(lv.planE, lv.e_nodes, nullptr, lv.inv_size_e, zv,
                                   i == 1 ? ck_e : ze_i - rows * d, ze_i, d, 1.f - omega, omega,
-                                  g->partials, s, g));
+                                  partials, s, g));
       if (n > 0 && m > 0) {  // z~^i = s_v / D_v, then z_v^i = (1-w) z_v^{i-1} + w z~^i
         HNV_CHECK(gather_rows_f32(lv.planV, lv.v_edges, lv.v_w, lv.inv_deg_v, ze_i, zt_i, zt_i, d,
-                                  0.f, 1.f, g->partials, s, g));
+                                  0.f, 1.f, partials, s, g));
         if (i < rsweeps)
           HNV_CHECK(launch("row_blend", row_blend_kernel, grid_for((int64_t)n * d4, 256), 256, 0,
                            s, n, d4, (float4*)zv, (const float4*)zt_i, omega,
@@ -512,7 +505,7 @@ int vcycle_backward_impl(hnv_graph* g, const float* ckpt, const float* g_v0, con
         // A_e = sum_{v in e} a_v: an unweighted gather, like the forward
         // hyperedge half-sweep (short rows take the packed kernels)
         HNV_CHECK(gather_rows_f32(lv.planE, lv.e_nodes, nullptr, nullptr, av, A, A, d, 0.f, 1.f,
-                                  g->partials, s, g));
+                                  partials, s, g));
         if (side) {
           HNV_CUDA(cudaEventRecord(g->join_ev[0], g->aux[0]));
           HNV_CUDA(cudaStreamWaitEvent(s, g->join_ev[0], 0));
@@ -526,7 +519,7 @@ int vcycle_backward_impl(hnv_graph* g, const float* ckpt, const float* g_v0, con
       // exactly the rows with incidences, the rows the gather writes.
       if (n > 0 && m > 0)
         HNV_CHECK(gather_rows_f32(lv.planV, lv.v_edges, lv.v_invsize_w, nullptr, ge, gv, gv, d,
-                                  1.f - omega, omega, g->partials, s, g));
+                                  1.f - omega, omega, partials, s, g));
     }
     ps.reset();
     ps.reset(new PhaseScope(HNV_PHASE_ADJOINT_PROJECT, s, by.project));
@@ -543,7 +536,7 @@ int vcycle_backward_impl(hnv_graph* g, const float* ckpt, const float* g_v0, con
     HNV_CUDA(cudaMemsetAsync(GC, 0, row * crow, s));
     if (cv.n > 0)
       HNV_CHECK(gather_rows_f32(lv.planC, lv.ch_idx, nullptr, nullptr, G, GC, GC, d, 0.f, 1.f,
-                                g->partials, s, g));
+                                partials, s, g));
     if (m > 0)
       HNV_CHECK(launch("scatter_kept", scatter_kept_kernel, grid_for((int64_t)m * d4, 256), 256, 0,
                        s, m, d4, (const int32_t*)lv.rep_e, (const float4*)ge,

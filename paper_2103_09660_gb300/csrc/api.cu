@@ -35,6 +35,7 @@ void destroy_graph(hnv_graph* g) {
   dev_free(g->team_levels, s);
   dev_free(g->partials, s);
   dev_free(g->jacobi_tmp, s);
+  for (void* p : g->outgrown) dev_free(p, s);
   dev_free(g->d_words, s);
   cudaStreamSynchronize(s);
   for (TeamSlot& t : g->team_slots)

@@ -470,6 +470,9 @@ struct hnv_graph {
   size_t partials_bytes = 0;
   float* jacobi_tmp = nullptr;   // Jacobi: next hyperedge rows
   size_t jacobi_bytes = 0;
+  // a capture uses the scratch above: what is outgrown is kept for its replays
+  bool captured = false;
+  std::vector<void*> outgrown;
   uint64_t generation = 0;       // bumped whenever the hierarchy is rebuilt
   // side streams on which a half-sweep's row classes run concurrently
   // (forked from and joined back into the caller's stream)
@@ -522,6 +525,11 @@ int coarsen_step(hnv_graph* g, int level, const hnv_coarsen_params* p, const uin
                  Level* fine, Level* coarse);
 
 // refine.cu
+// Scratch of `need` bytes for a call on s: *keep (*have bytes, the graph's),
+// grown if it must be. In a capture, where memory allocated now is valid in the
+// replays only, a larger one comes from the call's pool instead.
+int graph_scratch(hnv_graph* g, float** keep, size_t* have, size_t need, TempPool& pool,
+                  float** out, cudaStream_t s);
 // dtype: HNV_F32 or HNV_BF16 row storage (sums in float32 either way).
 int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d, float omega,
                  int sweeps, int mode, cudaStream_t s);

@@ -453,21 +453,26 @@ int gather_rows_f32(const SplitPlan& plan, const int32_t* idx, const float* wgt,
   return run_half<float>(h, src, self_in, out, d, keep, scale, partials, s);
 }
 
-namespace {
-
-int ensure_scratch(float** p, size_t* have, size_t need, cudaStream_t s) {
-  if (need <= *have && *p) return HNV_OK;
-  if (*p) dev_free(*p, s);
-  *p = nullptr;
-  *have = 0;
-  void* q = nullptr;
-  HNV_CHECK(dev_alloc(&q, need, s));
-  *p = static_cast<float*>(q);
-  *have = need;
+int graph_scratch(hnv_graph* g, float** keep, size_t* have, size_t need, TempPool& pool,
+                  float** out, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  HNV_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (need > *have || !*keep) {
+    if (cap != cudaStreamCaptureStatusNone) return pool.get(out, (need + 3) / 4);
+    if (*keep && g->captured) g->outgrown.push_back(*keep);
+    else if (*keep) dev_free(*keep, s);
+    *keep = nullptr;
+    *have = 0;
+    void* q = nullptr;
+    HNV_CHECK(dev_alloc(&q, need, s));
+    *keep = static_cast<float*>(q);
+    *have = need;
+  } else if (cap != cudaStreamCaptureStatusNone) {
+    g->captured = true;
+  }
+  *out = *keep;
   return HNV_OK;
 }
-
-}  // namespace
 
 bool team_enabled(int d) { return !timing_on() && !use_tma(d) && forced_panels() < 1; }
 
@@ -548,6 +553,7 @@ int team_slot(hnv_graph* g, cudaStream_t s, int* slot) {
 int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweeps, int mode,
              cudaStream_t s, const float* eps, const int32_t** result) {
   if (g->team_refuse) return kTeamRefused;
+  TempPool pool(s);
   int64_t chunks = 1, m = 1;
   int blocks = 1;
   for (int l = t.bottom; l <= t.top; ++l) {
@@ -556,9 +562,12 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
     m = std::max<int64_t>(m, lv.m);
     blocks = std::max(blocks, team_blocks_for(lv, dtype, d));
   }
-  HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes, sizeof(float) * (size_t)chunks * d, s));
+  float* jtmp = nullptr;
+  HNV_CHECK(graph_scratch(g, &g->partials, &g->partials_bytes, sizeof(float) * (size_t)chunks * d,
+                          pool, &t.partials, s));
   if (mode == HNV_SWEEP_JACOBI)
-    HNV_CHECK(ensure_scratch(&g->jacobi_tmp, &g->jacobi_bytes, elem_size(dtype) * (size_t)m * d, s));
+    HNV_CHECK(graph_scratch(g, &g->jacobi_tmp, &g->jacobi_bytes,
+                            elem_size(dtype) * (size_t)m * d, pool, &jtmp, s));
   int k = 0;
   HNV_CHECK(team_slot(g, s, &k));
   TeamSlot& slot = g->team_slots[k];
@@ -568,8 +577,7 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
   t.err = g->d_err;
   t.wait_ns = g->team_wait_ns;
   t.stop_at = g->team_stop_at;
-  t.partials = g->partials;
-  t.jtmp = reinterpret_cast<uint4*>(g->jacobi_tmp);
+  t.jtmp = reinterpret_cast<uint4*>(jtmp);
   TeamArgs a;
   a.one = t;
   a.blocks = blocks;
@@ -604,7 +612,7 @@ double half_bytes(const Level& lv, int side, int dtype, int d) {
 // Both half-sweeps of a level on its plans for d, with scratch for their
 // split rows.
 int level_halves(hnv_graph* g, int level, int dtype, int d, HalfSweep* E, HalfSweep* V,
-                 cudaStream_t s) {
+                 float** partials, TempPool& pool, cudaStream_t s) {
   Level& lv = g->levels[level];
   const size_t es = elem_size(dtype);
   const SplitPlan* planE = &lv.planE;
@@ -614,8 +622,9 @@ int level_halves(hnv_graph* g, int level, int dtype, int d, HalfSweep* E, HalfSw
     HNV_CHECK(side_plan(g, &lv, 1, es * (size_t)d, &planV, s));
   }
   const int64_t chunks = planE->n_chunks > planV->n_chunks ? planE->n_chunks : planV->n_chunks;
-  HNV_CHECK(ensure_scratch(&g->partials, &g->partials_bytes,
-                           sizeof(float) * (size_t)(chunks > 0 ? chunks : 1) * d, s));
+  HNV_CHECK(graph_scratch(g, &g->partials, &g->partials_bytes,
+                          sizeof(float) * (size_t)(chunks > 0 ? chunks : 1) * d, pool, partials,
+                          s));
   *E = HalfSweep{lv.e_nodes, nullptr, lv.inv_size_e, planE, lv.n, lv.m, g->d_err};
   *V = HalfSweep{lv.v_edges, lv.v_w, lv.inv_deg_v, planV, lv.m, lv.n, g->d_err};
   if (g->aux[0] && g->aux[1]) E->conc = V->conc = g;
@@ -627,14 +636,16 @@ int level_halves(hnv_graph* g, int level, int dtype, int d, HalfSweep* E, HalfSw
 int refine_sweep_into(hnv_graph* g, int level, const void* v_in, const void* e_in, void* v_out,
                       void* e_out, int dtype, int d, float omega, int mode, cudaStream_t s) {
   HalfSweep E, V;
-  HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, s));
+  TempPool pool(s);
+  float* partials = nullptr;
+  HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, &partials, pool, s));
   {
     PhaseScope ps(HNV_PHASE_REFINE_E, s, half_bytes(g->levels[level], 0, dtype, d));
-    HNV_CHECK(run_half_dispatch(E, v_in, e_in, e_out, dtype, d, omega, g->partials, s));
+    HNV_CHECK(run_half_dispatch(E, v_in, e_in, e_out, dtype, d, omega, partials, s));
   }
   PhaseScope ps(HNV_PHASE_REFINE_V, s, half_bytes(g->levels[level], 1, dtype, d));
   return run_half_dispatch(V, mode == HNV_SWEEP_JACOBI ? e_in : e_out, v_in, v_out, dtype, d,
-                           omega, g->partials, s);
+                           omega, partials, s);
 }
 
 int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d, float omega,
@@ -651,34 +662,37 @@ int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d
     if (rc != kTeamRefused) return rc;
   }
   HalfSweep E, V;
-  HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, s));
+  TempPool pool(s);
+  float* partials = nullptr;
+  HNV_CHECK(level_halves(g, level, dtype, d, &E, &V, &partials, pool, s));
   const size_t es = elem_size(dtype);
+  float* jtmp = nullptr;
   if (mode == HNV_SWEEP_JACOBI)
-    HNV_CHECK(ensure_scratch(&g->jacobi_tmp, &g->jacobi_bytes,
-                             es * ((size_t)lv.m > 0 ? lv.m : 1) * d, s));
+    HNV_CHECK(graph_scratch(g, &g->jacobi_tmp, &g->jacobi_bytes,
+                            es * ((size_t)lv.m > 0 ? lv.m : 1) * d, pool, &jtmp, s));
   const double bytesE = half_bytes(lv, 0, dtype, d), bytesV = half_bytes(lv, 1, dtype, d);
   // Jacobi: the new hyperedge rows go to a second buffer, the nodes read the
   // old ones, and the buffers change places (one copy back at most, not one a
   // sweep)
-  void *e_cur = z_e, *e_nxt = g->jacobi_tmp;
+  void *e_cur = z_e, *e_nxt = jtmp;
   for (int it = 0; it < sweeps; ++it) {
     if (mode == HNV_SWEEP_TWO_PHASE) {
       {
         PhaseScope ps(HNV_PHASE_REFINE_E, s, bytesE);
-        HNV_CHECK(run_half_dispatch(E, z_v, z_e, z_e, dtype, d, omega, g->partials, s));
+        HNV_CHECK(run_half_dispatch(E, z_v, z_e, z_e, dtype, d, omega, partials, s));
       }
       {
         PhaseScope ps(HNV_PHASE_REFINE_V, s, bytesV);
-        HNV_CHECK(run_half_dispatch(V, z_e, z_v, z_v, dtype, d, omega, g->partials, s));
+        HNV_CHECK(run_half_dispatch(V, z_e, z_v, z_v, dtype, d, omega, partials, s));
       }
     } else {
       {
         PhaseScope ps(HNV_PHASE_REFINE_E, s, bytesE);
-        HNV_CHECK(run_half_dispatch(E, z_v, e_cur, e_nxt, dtype, d, omega, g->partials, s));
+        HNV_CHECK(run_half_dispatch(E, z_v, e_cur, e_nxt, dtype, d, omega, partials, s));
       }
       {
         PhaseScope ps(HNV_PHASE_REFINE_V, s, bytesV);
-        HNV_CHECK(run_half_dispatch(V, e_cur, z_v, z_v, dtype, d, omega, g->partials, s));
+        HNV_CHECK(run_half_dispatch(V, e_cur, z_v, z_v, dtype, d, omega, partials, s));
       }
       std::swap(e_cur, e_nxt);
     }

@@ -431,3 +431,45 @@ def test_first_call_on_a_hierarchy_does_not_wait(H):
     got = once(True)
     assert got[0]
     assert torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("mode", ["two_phase", "jacobi"])
+@pytest.mark.parametrize("warm", [False, True])
+def test_captured_calls_keep_their_scratch(H, mode, warm):
+    """A graph's scratch grows with the row size. A capture that has to grow it
+    takes memory of its own (what it allocates is valid in its replays only),
+    and scratch that a capture uses outlives later growth."""
+    import torch
+    mode = H.SWEEP_JACOBI if mode == "jacobi" else H.SWEEP_TWO_PHASE
+    hg = _hub_graph(4200, [129, 300])
+
+    def rows(d):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(d)
+        return torch.randn((hg.n + hg.m, d), generator=g, device="cuda")
+
+    def plain(G, d):
+        z = rows(d)
+        G.refine(0, z[:hg.n], z[hg.n:], 0.3, 3, mode)
+        return z
+    with H.Graph.from_hypergraph(hg) as G:
+        want = {d: plain(G, d) for d in (32, 64)}
+    with H.Graph.from_hypergraph(hg) as G:
+        if warm:
+            assert torch.equal(plain(G, 32), want[32])
+        z = rows(32)
+        torch.cuda.synchronize()
+        graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=s):
+            H.hnv_refine(G.handle, 0, z[:hg.n], z[hg.n:], 0.3, 3, mode, s)
+        for d in (32, 64):
+            assert torch.equal(plain(G, d), want[d])
+            z.copy_(rows(32))
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(z, want[32])
+        G.sync_status()
+        del graph
+    # nothing of the capture was released outside it
+    with H.Graph.from_hypergraph(hg) as G:
+        assert torch.equal(plain(G, 32), want[32])
