@@ -68,12 +68,16 @@ __device__ __forceinline__ uint64_t global_ns() {
 // A barrier among the `blocks` blocks that share `counter` (0 at launch).
 // False once a wait gave up (the whole block sees the same answer). A wait is
 // limited to g->wait_ns; the barrier at target *stop waits for one arrival
-// more than comes (TeamGraph::stop_at).
+// more than comes (TeamGraph::stop_at). (A timeout is recorded here rather than
+// where the kernel's body returns: with that body in a function of its own the
+// batch of 64 graphs took 76 ms instead of 70, with no more spills.)
 struct TeamBarrier {
   uint32_t* counter;
   uint32_t blocks;
   uint32_t target;
-  int32_t* err;
+  const TeamGraph* graphs;   // a batch's, of which [q, q1) are still to be run
+  int32_t q, q1;
+  int32_t* result;           // the stopping rule's word for a timeout, or null
   int* dead;             // shared memory, as g and stop
   const TeamGraph* g;
   const uint32_t* stop;
@@ -96,7 +100,13 @@ struct TeamBarrier {
             t0 = now;
           } else if (now - t0 > g->wait_ns) {
             *dead = 1;
-            atomicOr(err, (int32_t)ERRBIT_TIMEOUT);
+            if (result) {
+              atomicOr(result, (int32_t)ERRBIT_TIMEOUT);
+            } else if (!graphs) {
+              atomicOr(g->err, (int32_t)ERRBIT_TIMEOUT);
+            } else {   // the team's later graphs are not run
+              for (int32_t r = q; r < q1; ++r) atomicOr(graphs[r].err, (int32_t)ERRBIT_TIMEOUT);
+            }
             break;
           }
         }
@@ -469,68 +479,6 @@ __device__ __forceinline__ void team_project(const TeamLevel& f, const uint4* zc
   }
 }
 
-// Levels top .. bottom of the graph in g by one team. False: a wait gave up.
-template <typename T, int G, int VPL, bool DIFF>
-__device__ __forceinline__ bool team_graph(const TeamArgs& a, const TeamGraph& g, int block,
-                                           float* sm, TeamBarrier& bar) {
-  const int warp = (threadIdx.x >> 5) * a.blocks + block, warps = kTeamWarps * a.blocks;
-  const int64_t thread = (int64_t)warp * 32 + (threadIdx.x & 31), threads = (int64_t)warps * 32;
-  const int dv = a.dv;
-  for (int l = g.top; l >= g.bottom; --l) {
-    const TeamLevel& lv = g.levels[l];
-    uint4* zv = l == g.bottom ? g.zv0 : g.buf[l & 1];
-    uint4* ze = l == g.bottom ? g.ze0 : zv + (size_t)lv.n * dv;
-    uint4* ck = g.ckpt ? g.ckpt + (size_t)lv.row0 * dv : nullptr;
-    if (l == g.top) {
-      if (g.zc) {
-        team_copy(zv, g.zc, (int64_t)lv.n * dv, thread, threads);
-        team_copy(ze, g.zc + (size_t)lv.n * dv, (int64_t)lv.m * dv, thread, threads);
-        if (ck) team_copy(ck, g.zc, ((int64_t)lv.n + lv.m) * dv, thread, threads);
-      }
-    } else {
-      const uint4* cv = g.buf[(l + 1) & 1];
-      team_project<G, VPL>(lv, cv, cv + (size_t)g.levels[l + 1].n * dv, zv, ze, ck, dv, warp,
-                          warps);
-    }
-    uint4* e_in = ze;
-    StepHeads he = load_heads<T, G, false>(lv.side[0], dv, block, a.blocks);
-    if (!bar.wait()) return false;
-    for (int it = 0; it < a.sweeps; ++it) {
-      // Jacobi: the new hyperedge rows go to a second buffer, the nodes
-      // read the old ones, and the buffers change places
-      uint4* e_out = a.jacobi ? (e_in == ze ? g.jtmp : ze) : ze;
-      unsigned* slot = DIFF ? a.delta + it % 3 : nullptr;
-      // the slot of the next sweep was last read two barriers ago
-      if (DIFF && blockIdx.x == 0 && threadIdx.x == 0) a.delta[(it + 1) % 3] = 0u;
-      if (!team_half<T, G, VPL, false, DIFF>(lv.side[0], he, zv, e_in, e_out, g.partials, dv,
-                                             a.keep, a.omega, block, a.blocks, sm, slot, bar))
-        return false;
-      const StepHeads hv = load_heads<T, G, true>(lv.side[1], dv, block, a.blocks);
-      if (!bar.wait()) return false;
-      if (!team_half<T, G, VPL, true, DIFF>(lv.side[1], hv, a.jacobi ? e_in : e_out, zv, zv,
-                                            g.partials, dv, a.keep, a.omega, block, a.blocks,
-                                            sm, slot, bar))
-        return false;
-      he = load_heads<T, G, false>(lv.side[0], dv, block, a.blocks);
-      if (!bar.wait()) return false;
-      e_in = e_out;
-      if (DIFF) {
-        const float delta = __uint_as_float(load_word(slot));
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-          a.result[0] = it + 1;
-          a.result[1] = __float_as_int(delta);
-        }
-        if (delta <= a.eps) break;
-      }
-    }
-    if (e_in != ze) {
-      team_copy(ze, e_in, (int64_t)lv.m * dv, thread, threads);
-      if (!bar.wait()) return false;
-    }
-  }
-  return true;
-}
-
 template <typename T, int G, int VPL, bool DIFF>
 __global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(const TeamArgs a) {
   __shared__ __align__(16) float sm[kFinSlots * VecT<T>::N];
@@ -539,8 +487,12 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(const TeamArgs a)
   __shared__ TeamGraph g;
   if (threadIdx.x == 0) dead = 0;
   const int team = blockIdx.x / a.blocks, block = blockIdx.x - team * a.blocks;
-  TeamBarrier bar{a.barriers + 32 * team, (uint32_t)a.blocks, 0u, nullptr, &dead, &g, &stop};
+  const int warp = (threadIdx.x >> 5) * a.blocks + block, warps = kTeamWarps * a.blocks;
+  const int64_t thread = (int64_t)warp * 32 + (threadIdx.x & 31), threads = (int64_t)warps * 32;
+  TeamBarrier bar{a.barriers + 32 * team, (uint32_t)a.blocks, 0u,    a.graphs, 0, 0,
+                  DIFF ? a.result + 2 : nullptr,          &dead, &g,       &stop};
   const int32_t q0 = a.graphs ? a.team_first[team] : 0, q1 = a.graphs ? a.team_first[team + 1] : 1;
+  const int dv = a.dv;
   for (int32_t q = q0; q < q1; ++q) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -548,12 +500,59 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(const TeamArgs a)
       stop = g.stop_at > 0 ? bar.target + (uint32_t)g.stop_at * bar.blocks : 0u;
     }
     __syncthreads();
-    bar.err = DIFF ? a.result + 2 : g.err;
-    if (!team_graph<T, G, VPL, DIFF>(a, g, block, sm, bar)) {
-      // the team's later graphs are not run: their rows are not valid either
-      if (threadIdx.x == 0)
-        for (int32_t r = q + 1; r < q1; ++r) atomicOr(a.graphs[r].err, (int32_t)ERRBIT_TIMEOUT);
-      return;
+    bar.q = q;
+    bar.q1 = q1;
+    for (int l = g.top; l >= g.bottom; --l) {
+      const TeamLevel& lv = g.levels[l];
+      uint4* zv = l == g.bottom ? g.zv0 : g.buf[l & 1];
+      uint4* ze = l == g.bottom ? g.ze0 : zv + (size_t)lv.n * dv;
+      uint4* ck = g.ckpt ? g.ckpt + (size_t)lv.row0 * dv : nullptr;
+      if (l == g.top) {
+        if (g.zc) {
+          team_copy(zv, g.zc, (int64_t)lv.n * dv, thread, threads);
+          team_copy(ze, g.zc + (size_t)lv.n * dv, (int64_t)lv.m * dv, thread, threads);
+          if (ck) team_copy(ck, g.zc, ((int64_t)lv.n + lv.m) * dv, thread, threads);
+        }
+      } else {
+        const uint4* cv = g.buf[(l + 1) & 1];
+        team_project<G, VPL>(lv, cv, cv + (size_t)g.levels[l + 1].n * dv, zv, ze, ck, dv, warp,
+                            warps);
+      }
+      uint4* e_in = ze;
+      StepHeads he = load_heads<T, G, false>(lv.side[0], dv, block, a.blocks);
+      if (!bar.wait()) return;
+      for (int it = 0; it < a.sweeps; ++it) {
+        // Jacobi: the new hyperedge rows go to a second buffer, the nodes
+        // read the old ones, and the buffers change places
+        uint4* e_out = a.jacobi ? (e_in == ze ? g.jtmp : ze) : ze;
+        unsigned* slot = DIFF ? a.delta + it % 3 : nullptr;
+        // the slot of the next sweep was last read two barriers ago
+        if (DIFF && blockIdx.x == 0 && threadIdx.x == 0) a.delta[(it + 1) % 3] = 0u;
+        if (!team_half<T, G, VPL, false, DIFF>(lv.side[0], he, zv, e_in, e_out, g.partials, dv,
+                                               a.keep, a.omega, block, a.blocks, sm, slot, bar))
+          return;
+        const StepHeads hv = load_heads<T, G, true>(lv.side[1], dv, block, a.blocks);
+        if (!bar.wait()) return;
+        if (!team_half<T, G, VPL, true, DIFF>(lv.side[1], hv, a.jacobi ? e_in : e_out, zv, zv,
+                                              g.partials, dv, a.keep, a.omega, block, a.blocks,
+                                              sm, slot, bar))
+          return;
+        he = load_heads<T, G, false>(lv.side[0], dv, block, a.blocks);
+        if (!bar.wait()) return;
+        e_in = e_out;
+        if (DIFF) {
+          const float delta = __uint_as_float(load_word(slot));
+          if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.result[0] = it + 1;
+            a.result[1] = __float_as_int(delta);
+          }
+          if (delta <= a.eps) break;
+        }
+      }
+      if (e_in != ze) {
+        team_copy(ze, e_in, (int64_t)lv.m * dv, thread, threads);
+        if (!bar.wait()) return;
+      }
     }
   }
 }
