@@ -132,9 +132,9 @@ int vcycle_impl(hnv_graph* g, const void* z_coarsest, void* z_v_out, void* z_e_o
   const uint8_t* zc = static_cast<const uint8_t*>(z_coarsest);
   // the levels from the coarsest down that are small enough take one launch
   int first_big = L;
-  if (on_device && team_enabled(d) && sweeps <= kTeamMaxSweeps && team_fits(top, dtype, d) &&
+  if (on_device && team_enabled(d) && sweeps <= kTeamMaxSweeps && team_pays(top, dtype, d) &&
       team_ready(g))
-    while (first_big >= 0 && team_fits(g->levels[first_big], dtype, d)) --first_big;
+    while (first_big >= 0 && team_pays(g->levels[first_big], dtype, d)) --first_big;
   if (first_big < L) {
     const int b = first_big + 1;
     TeamGraph t;

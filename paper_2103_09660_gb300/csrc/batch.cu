@@ -18,10 +18,10 @@
 // every item of the half-sweep (warps take tasks from a counter; see
 // batched_persistent_kernel). Both are followed by the split-row reduction.
 //
-// Graphs whose levels are all small (team_fits) take neither: with the
+// Graphs whose levels are all small (team_fits) may take neither: with the
 // per-class setting they are dealt over teams of blocks that run a graph's
-// whole V-cycle each, in one launch (team.cu), and only the other graphs are
-// lined up by level.
+// whole V-cycle each, in one launch (team.cu), where that is estimated to be
+// faster (plan_teams), and only the other graphs are lined up by level.
 //
 // Autotuner: the row-class boundaries (PlanShape) and the lanes per row of
 // the short classes of the per-class kernel, and the persistent kernel, are
@@ -371,6 +371,14 @@ struct BatchDeal {
   int exec_kernel = -1;            // the half-sweep kernel it was captured with
 };
 
+// The graphs that may go to teams for one (dtype, d), and their deal.
+struct TeamPlan {
+  int dt = -1, d = -1;
+  std::vector<int> top;                  // coarsest level of each graph, -1: to a team
+  std::vector<std::vector<int>> lists;   // graphs of each team
+  int blocks = 1;                        // blocks per team
+};
+
 struct hnv_batch {
   std::vector<hnv_graph*> graphs;
   std::vector<uint64_t> generation;   // each graph's hierarchy generation at creation
@@ -389,6 +397,7 @@ struct hnv_batch {
   // [0] small graphs run by teams, [1] every graph in the step lists
   BatchDeal deal[2];
   bool no_teams = false;           // the device refused the teams' launch
+  TeamPlan team_plan;
   // half-sweep kernel: 0 one launch per row class, 1 one persistent launch
   int kernel = HNV_BATCH_KERNEL_PER_CLASS;
   // task counters of the persistent launches, one per half-sweep of a V-cycle
@@ -435,19 +444,82 @@ void drop_deal(const hnv_batch* b, BatchDeal& D, cudaStream_t s) {
   D.plans_ready = false;
 }
 
-// The coarsest level of each graph, -1 for those the teams run: the graphs all
-// of whose levels are small, with the per-class setting and at most
-// kTeamMaxSweeps sweeps.
-std::vector<int> deal_teams(const hnv_batch* b, int dt, int d, int sweeps) {
-  std::vector<int> top = b->top;
-  if (b->kernel == HNV_BATCH_KERNEL_PER_CLASS && !b->no_teams && team_enabled(d) &&
-      sweeps <= kTeamMaxSweeps)
-    for (size_t i = 0; i < b->graphs.size(); ++i) {
-      bool fits = true;
-      for (const Level& lv : b->graphs[i]->levels) fits = fits && team_fits(lv, dt, d);
-      if (fits && team_ready(b->graphs[i])) top[i] = -1;
+// Deals the graphs all of whose levels are small over teams (longest first, each
+// to the team with the least work so far), over the number of teams with the
+// shortest longest team, and decides whether that pays: the longest team against
+// what the graphs would add to the step lists, both estimated. (On batches of 2
+// to 300 graphs at 12 row sizes the choice was at most 1.15 times slower than the
+// better path, 1.007 on average; teams throughout were up to 1.64 times slower,
+// with rows of 16-32 bytes, or float32 rows of 512 and more, and the whole device
+// at work.)
+void plan_teams(hnv_batch* b, int dt, int d) {
+  TeamPlan& p = b->team_plan;
+  if (p.dt == dt && p.d == d) return;
+  p = TeamPlan();
+  p.dt = dt;
+  p.d = d;
+  p.top = b->top;
+  std::vector<int> own;
+  size_t rest_steps = 0, own_steps = 0;   // levels of the deepest graph
+  int64_t own_nnz = 0;
+  for (size_t i = 0; i < b->graphs.size(); ++i) {
+    const std::vector<Level>& levels = b->graphs[i]->levels;
+    bool fits = team_ready(b->graphs[i]);
+    for (const Level& lv : levels) fits = fits && team_fits(lv, dt, d);
+    size_t& steps = fits ? own_steps : rest_steps;
+    steps = std::max(steps, levels.size());
+    if (!fits) continue;
+    own.push_back((int)i);
+    for (const Level& lv : levels) own_nnz += lv.nnz;
+  }
+  if (own.empty()) return;
+  const int sms = num_sms();
+  double best_us = -1.0;
+  for (int teams = 1; teams <= std::min<int>(sms, (int)own.size()); ++teams) {
+    const int blocks = sms / teams;
+    std::vector<std::pair<double, int>> cost;
+    for (int i : own) {
+      double us = 0.0;
+      for (const Level& lv : b->graphs[i]->levels) us += team_sweep_us(lv, dt, d, blocks);
+      cost.push_back({us, i});
     }
-  return top;
+    std::sort(cost.begin(), cost.end(), [](const std::pair<double, int>& x, const std::pair<double, int>& y) {
+      return x.first != y.first ? x.first > y.first : x.second < y.second;
+    });
+    std::vector<std::vector<int>> deal(teams);
+    std::vector<double> load(teams, 0.0);
+    for (const auto& c : cost) {
+      const int t = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      deal[t].push_back(c.second);
+      load[t] += c.first;
+    }
+    const double us = *std::max_element(load.begin(), load.end());
+    if (best_us < 0.0 || us < best_us) {
+      best_us = us;
+      p.lists = deal;
+      p.blocks = blocks;
+    }
+  }
+  double teams_us = 0.0;
+  for (const std::vector<int>& list : p.lists) {
+    double us = 0.0;
+    for (int i : list)
+      for (const Level& lv : b->graphs[i]->levels) us += team_batch_us(lv, dt, d, p.blocks);
+    teams_us = std::max(teams_us, us);
+  }
+  const int more = own_steps > rest_steps ? (int)(own_steps - rest_steps) : 0;
+  if (teams_us > 1.15 * step_batch_us(more, own_nnz, dt, d)) return;
+  for (int i : own) p.top[i] = -1;
+}
+
+// The coarsest level of each graph, -1 for those the teams run (with the
+// per-class setting and at most kTeamMaxSweeps sweeps).
+const std::vector<int>& deal_teams(hnv_batch* b, int dt, int d, int sweeps) {
+  if (b->kernel != HNV_BATCH_KERNEL_PER_CLASS || b->no_teams || !team_enabled(d) ||
+      sweeps > kTeamMaxSweeps)
+    return b->top;
+  plan_teams(b, dt, d);
+  return b->team_plan.top;
 }
 
 // The deal that belongs to `top` (the second if no graph is with the teams).
@@ -501,51 +573,18 @@ int build_plans(hnv_batch* b, BatchDeal& D, size_t row_bytes, cudaStream_t s,
   return HNV_OK;
 }
 
-// Deals the teams' graphs (longest first, each to the team with the least
-// work so far) over the number of teams with the shortest longest team, and
-// uploads their descriptors. Row buffers and partials belong to a team, so
-// that its next graph finds them in L2.
-int build_teams(const hnv_batch* b, BatchDeal& D, int dt, int d, const uint8_t* zc, uint8_t* zv0, uint8_t* ze0,
-                cudaStream_t s) {
+// Uploads the descriptors of the teams' graphs, dealt by plan_teams. Row buffers
+// and partials belong to a team, so that its next graph finds them in L2.
+int build_teams(const hnv_batch* b, BatchDeal& D, int dt, int d, const uint8_t* zc, uint8_t* zv0,
+                uint8_t* ze0, cudaStream_t s) {
   const size_t rb = (dt == HNV_BF16 ? 2 : 4) * (size_t)d;
-  std::vector<int> own;
-  for (size_t i = 0; i < b->graphs.size(); ++i)
-    if (D.step_top[i] < 0) own.push_back((int)i);
   D.teams = 0;
-  if (own.empty()) return HNV_OK;
-  const int sms = num_sms();
-  std::vector<std::vector<int>> best;
-  double best_us = -1.0;
-  int best_blocks = 1;
-  for (int teams = 1; teams <= std::min<int>(sms, (int)own.size()); ++teams) {
-    const int blocks = sms / teams;
-    std::vector<std::pair<double, int>> cost;
-    for (int i : own) {
-      double us = 0.0;
-      for (const Level& lv : b->graphs[i]->levels) us += team_sweep_us(lv, dt, d, blocks);
-      cost.push_back({us, i});
-    }
-    std::sort(cost.begin(), cost.end(), [](const std::pair<double, int>& x, const std::pair<double, int>& y) {
-      return x.first != y.first ? x.first > y.first : x.second < y.second;
-    });
-    std::vector<std::vector<int>> deal(teams);
-    std::vector<double> load(teams, 0.0);
-    for (const auto& c : cost) {
-      const int t = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-      deal[t].push_back(c.second);
-      load[t] += c.first;
-    }
-    const double us = *std::max_element(load.begin(), load.end());
-    if (best_us < 0.0 || us < best_us) {
-      best_us = us;
-      best = deal;
-      best_blocks = blocks;
-    }
-  }
-  const int teams = (int)best.size();
+  if (std::count(D.step_top.begin(), D.step_top.end(), -1) == 0) return HNV_OK;
+  const TeamPlan& plan = b->team_plan;
+  const int teams = (int)plan.lists.size();
   std::vector<TeamGraph> hg;
   std::vector<int32_t> first{0};
-  for (const std::vector<int>& list : best) {
+  for (const std::vector<int>& list : plan.lists) {
     size_t rows = 0;
     int64_t chunks = 1;
     for (int i : list)
@@ -583,7 +622,7 @@ int build_teams(const hnv_batch* b, BatchDeal& D, int dt, int d, const uint8_t* 
   HNV_CUDA(cudaStreamSynchronize(s));   // the host vectors die here
   D.team.graphs = dg;
   D.team.team_first = df;
-  D.team.blocks = best_blocks;
+  D.team.blocks = plan.blocks;
   D.teams = teams;
   return HNV_OK;
 }

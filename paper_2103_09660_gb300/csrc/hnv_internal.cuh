@@ -625,18 +625,30 @@ struct TeamArgs {
   float eps = 0.f;
 };
 
-// Levels the team kernel takes: rows of at most 64 vectors, and so little
-// work per half-sweep that launches, not bandwidth, would set its time.
+// Levels the team kernel can take: rows of at most 64 vectors, and so little
+// work per half-sweep that launches, not bandwidth, may set its time. The
+// stopping rule takes it for all of these: a launch per half-sweep also reads
+// both tables again and the host waits every sweep (1.05-3 times slower on
+// every level measured, 35 levels of 4 to 1,000K rows, 8 to 1,024 bytes a row).
 constexpr int64_t kTeamMaxRowBytes = 1024;
 constexpr int64_t kTeamMaxGather = 192000000;   // bytes gathered per half-sweep
 constexpr int64_t kTeamMaxRows = 96000000;      // bytes of both row tables
 constexpr int kTeamMaxSweeps = 512;             // of one launch
 bool team_fits(const Level& lv, int dtype, int d);
+// Levels of a fixed number of sweeps that it also runs faster than a launch per
+// row class does (team.cu).
+bool team_pays(const Level& lv, int dtype, int d);
 void team_level(const Level& lv, int64_t row0, TeamLevel* out);
 // Blocks that the items of one level's larger side fill.
 int team_blocks_for(const Level& lv, int dtype, int d);
-// Estimated microseconds of one sweep of a level by a team of `blocks`.
+// Estimated microseconds of one sweep of a level by a team of `blocks` (to deal
+// a batch's graphs over teams).
 double team_sweep_us(const Level& lv, int dtype, int d, int blocks);
+// Estimates to choose a batch's path by, fitted to the same batches (team.cu): a
+// sweep of a level by a team of `blocks` of the device's SMs; a sweep each of
+// `steps` steps of the step lists with `nnz` incidences in all.
+double team_batch_us(const Level& lv, int dtype, int d, int blocks);
+double step_batch_us(int steps, int64_t nnz, int dtype, int d);
 // kTeamRefused: the device would not run the blocks at once (it has fewer SMs
 // for this process than it says, or no cooperative launches), and nothing was
 // launched; the caller takes the per-launch path.

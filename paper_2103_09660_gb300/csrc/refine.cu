@@ -652,7 +652,7 @@ int refine_level(hnv_graph* g, int level, void* z_v, void* z_e, int dtype, int d
                  int sweeps, int mode, cudaStream_t s) {
   NvtxRange nvtx("hnv refine level %d (%d sweeps)", level, sweeps);
   Level& lv = g->levels[level];
-  if (sweeps > 0 && sweeps <= kTeamMaxSweeps && team_enabled(d) && team_fits(lv, dtype, d) &&
+  if (sweeps > 0 && sweeps <= kTeamMaxSweeps && team_enabled(d) && team_pays(lv, dtype, d) &&
       team_ready(g)) {
     TeamGraph t;
     t.top = t.bottom = level;

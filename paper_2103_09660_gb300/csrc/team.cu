@@ -26,16 +26,17 @@
 //
 // The items and split rows are the level's plans (SplitPlan) and every row is
 // summed in the order of the per-launch kernels (refine.cu, batch.cu): the
-// results are the same bits.
+// results are the same bits. Which levels take it: team_pays, team_fits, and for a
+// batch the estimates below.
 //
 // Measured (GB300, same bits): the V-cycle of a 2,000-node graph (d = 32, 7
 // levels x 10 sweeps) 2.25 -> 0.74 ms, of a 41K-node graph (d = 100, 33 levels
 // x 20 sweeps) 31.2 -> 13.2 ms, of a batch of 64 graphs of 1K-100K nodes
 // (d = 64) 91 -> 76 ms. What is left of a sweep of the 41K-node graph (20 us)
 // is 3-6 us of dependent loads a half-sweep, 1.4 us a barrier (2 or 3 a
-// sweep) and 4 us for a hub row's reduction. Above kTeamMaxGather the
-// per-launch kernels, with twice the warps per SM, are faster (a level of
-// 150K nodes, 2.1M incidences, d = 100: 2.0 against 3.9 ms for 10 sweeps).
+// sweep) and 4 us for a hub row's reduction. On larger levels the per-launch
+// kernels, with twice the warps per SM, are faster (a level of 150K nodes, 2.1M
+// incidences, d = 100: 2.0 against 3.9 ms for 10 sweeps).
 //
 // Rows written in one step are read in the next by other blocks, so row and
 // partial loads are plain (never the read-only path); the barrier's
@@ -44,6 +45,7 @@
 // goes to the graph's error word (read by hnv_sync_status), or, with the
 // stopping rule, to the launch's own result, which that call reads anyway.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "refine_device.cuh"
@@ -619,6 +621,32 @@ bool team_fits(const Level& lv, int dtype, int d) {
          ((int64_t)lv.n + lv.m) * rb <= kTeamMaxRows;
 }
 
+// The line between the two paths, measured on 36 levels of graphs of 5K-600K
+// nodes (members of 2-3,000, coarse levels with hub nodes of up to thousands of
+// incidences) at 17 row sizes, us a sweep, this path against a launch per row
+// class (whose time differs by up to 20% between runs):
+//   - it costs about 35 us per million incidences however narrow the rows are,
+//     where the launches' floor is 50 us: of 32 bytes 1.36M 59 against 81-85,
+//     1.74M 65 against 69-75, 1.87M 68 against 50, 2.14M 82 against 52 (the
+//     launches are slower for bfloat16 rows of one vector: 1.87M 70 against 87,
+//     2.14M 84 against 59);
+//   - beyond 100 MB of gathered rows its 16 warps per SM keep too few loads in
+//     flight: 256-byte float32 rows 115 MB 51 against 56, 400-byte ones 131 MB 66
+//     against 52, 162 MB 79 against 56-60. The launches need more time for rows of
+//     at most 128 bytes (174 MB: float32 74 against 88-105, bfloat16 77 against
+//     75-94), for bfloat16, whose conversions they spend issue slots on (256 bytes:
+//     167 MB 69 against 83, 215 MB 80 against 73), and for rows of two vectors per
+//     lane (151 MB 50 against 60).
+bool team_pays(const Level& lv, int dtype, int d) {
+  const int64_t rb = (int64_t)(dtype == HNV_BF16 ? 2 : 4) * d;
+  int64_t gather = 125000000;
+  if (rb > 512) gather = 160000000;
+  else if (rb <= 128) gather = kTeamMaxGather;
+  else if (dtype == HNV_BF16 && rb <= 256) gather = 170000000;
+  const int64_t most = dtype == HNV_BF16 && rb == 16 ? 2000000 : 1800000;
+  return team_fits(lv, dtype, d) && lv.nnz <= most && lv.nnz * rb <= gather;
+}
+
 int team_blocks_for(const Level& lv, int dtype, int d) {
   // warps of one pass over the larger side: a short row takes a lane per
   // vector, a long row or chunk a lane per word
@@ -641,6 +669,35 @@ double team_sweep_us(const Level& lv, int dtype, int d, int blocks) {
   const double bytes = (double)(dtype == HNV_BF16 ? 2 : 4) * d *
                        (2.0 * lv.nnz + 3.0 * ((double)lv.n + lv.m));
   return 12.0 + bytes / (52e3 * blocks);
+}
+
+namespace {
+
+// Nanoseconds per incidence of a sweep (both sides) on the whole device, at rows
+// of 16 << i bytes; between them by the logarithm. From batches of 2-300 graphs
+// of 2K-600K nodes with the whole device at work (float32, bfloat16).
+constexpr double kTeamNs[2][7] = {{.034, .034, .037, .055, .112, .23, .42},
+                                  {.039, .040, .045, .062, .112, .21, .415}};
+constexpr double kStepNs[2][7] = {{.020, .020, .034, .054, .118, .182, .34},
+                                  {.026, .023, .040, .070, .137, .27, .53}};
+
+double per_incidence_us(const double* ns, double row_bytes) {
+  const double x = std::max(0.0, std::log2(row_bytes / 16.0));
+  const int i = std::min((int)x, 5);
+  return 1e-3 * (ns[i] + (x - i) * (ns[i + 1] - ns[i]));
+}
+
+}  // namespace
+
+double team_batch_us(const Level& lv, int dtype, int d, int blocks) {
+  const int k = dtype == HNV_BF16 ? 1 : 0;
+  return 8.0 + (double)lv.nnz * per_incidence_us(kTeamNs[k], (k ? 2.0 : 4.0) * d) * num_sms() /
+                   blocks;
+}
+
+double step_batch_us(int steps, int64_t nnz, int dtype, int d) {
+  const int k = dtype == HNV_BF16 ? 1 : 0;
+  return 50.0 * steps + (double)nnz * per_incidence_us(kStepNs[k], (k ? 2.0 : 4.0) * d);
 }
 
 int team_launch(TeamArgs a, int teams, int dtype, int d, cudaStream_t s) {

@@ -473,3 +473,69 @@ def test_captured_calls_keep_their_scratch(H, mode, warm):
     # nothing of the capture was released outside it
     with H.Graph.from_hypergraph(hg) as G:
         assert torch.equal(plain(G, 32), want[32])
+
+
+def _ring(n, m):
+    """m hyperedges of three consecutive nodes: 3 m incidences."""
+    nodes = (np.arange(m, dtype=np.int64)[:, None] + np.arange(3)[None, :]) % n
+    return n, m, 3 * np.arange(m + 1, dtype=np.int64), nodes.astype(np.int32).ravel()
+
+
+# incidences at which the launch per row class takes over, by row size
+@pytest.mark.parametrize("dtname,d,most", [
+    ("f32", 4, 1_800_000), ("bf16", 8, 2_000_000), ("f32", 8, 1_800_000), ("bf16", 16, 1_800_000),
+    ("f32", 32, 192_000_000 // 128), ("bf16", 64, 192_000_000 // 128),
+    ("f32", 36, 125_000_000 // 144), ("bf16", 128, 170_000_000 // 256),
+    ("bf16", 136, 125_000_000 // 272), ("f32", 128, 125_000_000 // 512),
+    ("f32", 132, 160_000_000 // 528), ("bf16", 512, 160_000_000 // 1024)])
+def test_levels_at_the_limit(H, dtname, d, most):
+    """Both sides of the line between the one-launch path and the launch per
+    row class; the stopping rule's is at 192 MB of gathered rows throughout."""
+    import torch
+    dt = torch.float32 if dtname == "f32" else torch.bfloat16
+    for m in (most // 3, most // 3 + 1):
+        n = 30_000 if d > 500 else 60_000 if d > 100 else 100_000
+        with H.Graph(*_ring(n, m)) as G:
+            z = torch.randn((n + m, d), device="cuda").to(dt)
+
+            def refine():
+                v, e = z[:n].clone(), z[n:].clone()
+                G.refine(0, v, e, 0.3, 2)
+                return v, e
+            a, b, one, many = _both(H, refine)
+            assert (one == 1) == (3 * m <= most) and many > 1
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+            def until():
+                v, e = z[:n].clone(), z[n:].clone()
+                return v, e, G.refine_until(0, v, e, 0.3, 2, -1.0)
+            a, b, one, many = _both(H, until)
+            assert (one == 1) == (3 * m * d * z.element_size() <= 192_000_000) and a[2] == b[2]
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("d,teams", [(8, False), (32, True)])
+def test_batch_takes_the_path_estimated_faster(H, d, teams):
+    """Eight graphs that fill the device: narrow rows go to the step lists."""
+    import torch
+    Gs = [H.Graph(*_ring(200_000, 400_000 + i)) for i in range(8)]
+    with H.Batch(Gs) as B:
+        co, vo, eo = (int(a[-1]) for a in B.offsets())
+        zc = torch.randn((co, d), device="cuda")
+        zv, ze = torch.empty((vo, d), device="cuda"), torch.empty((eo, d), device="cuda")
+
+        def vcycle():
+            zv.fill_(float("nan"))
+            ze.fill_(float("nan"))
+            B.vcycle(zc, zv, ze, 0.3, 2)
+            return zv.clone(), ze.clone()
+        vcycle()                                         # (builds the lists)
+        H.timing_enable(True)
+        vcycle()
+        H.timing_enable(False)
+        H.timing_reset()
+        a, b, one, many = _both(H, vcycle)
+        assert (one == 1) == teams and many > 1
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+    for G in Gs:
+        G.close()
