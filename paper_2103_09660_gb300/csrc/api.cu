@@ -32,7 +32,7 @@ void destroy_graph(hnv_graph* g) {
   cudaStream_t s = g->stream;
   for (auto& lv : g->levels) free_level(&lv, s);
   g->levels.clear();
-  dev_free(g->team_levels, s);
+  team_drop(g);
   dev_free(g->partials, s);
   dev_free(g->jacobi_tmp, s);
   for (void* p : g->outgrown) dev_free(p, s);
@@ -228,10 +228,12 @@ int hnv_build_incidence(int32_t n_nodes, int32_t n_edges, const int64_t* edge_pt
       break;
     }
     // the error word, the scratch words and the sets of team words, each on
-    // lines of its own
-    if ((rc = dev_alloc((void**)&g->d_words, (96 + kTeamSlots * kTeamWords) * sizeof(int32_t),
-                        s)) != HNV_OK)
+    // lines of its own, and the level descriptors
+    constexpr size_t kWords = 96 + kTeamSlots * kTeamWords;
+    if ((rc = dev_alloc((void**)&g->d_words,
+                        kWords * sizeof(int32_t) + kTeamLevels * sizeof(TeamLevel), s)) != HNV_OK)
       break;
+    g->team_buf = reinterpret_cast<TeamLevel*>(g->d_words + kWords);
     g->d_err = g->d_words;
     g->d_buf = g->d_words + 32;
     g->team_words = g->d_words + 96;
@@ -318,8 +320,7 @@ int hnv_coarsen(hnv_graph* g, const hnv_coarsen_params* p, int32_t* n_levels) {
     g->levels.pop_back();
   }
   drop_maps(&g->levels[0], s);
-  dev_free(g->team_levels, s);   // describes the old hierarchy
-  g->team_levels = nullptr;
+  team_drop(g);   // describes the old hierarchy
   const int32_t m0 = g->levels[0].m;
   {
     PhaseScope ps(HNV_PHASE_COARSEN, s, 0.0);

@@ -446,6 +446,7 @@ struct TeamSlot {
   cudaEvent_t done = nullptr;       // after it: another stream may take the set
 };
 constexpr int kTeamSlots = 32, kTeamStreamSlots = 8;   // sets; of them kept for streams
+constexpr int kTeamLevels = 40;   // levels a graph has room to describe from the start
 
 }  // namespace hnv
 
@@ -456,12 +457,15 @@ struct hnv_graph {
   int32_t* d_err = nullptr;      // device error word
   int32_t* h_buf = nullptr;      // pinned host scratch (64 ints)
   int32_t* d_buf = nullptr;      // device scratch (64 ints)
-  // one allocation: d_err, d_buf and kTeamSlots x kTeamWords team_words
+  // one allocation: d_err, d_buf, kTeamSlots x kTeamWords team_words and
+  // kTeamLevels of the team_levels
   int32_t* d_words = nullptr;
   int32_t* team_words = nullptr;
   hnv::TeamSlot team_slots[hnv::kTeamSlots];
   uint64_t team_turn = 0;
-  hnv::TeamLevel* team_levels = nullptr;   // device, one per level (team.cu)
+  hnv::TeamLevel* team_buf = nullptr;
+  // device, one per level (team.cu): team_buf, or an allocation of its own
+  hnv::TeamLevel* team_levels = nullptr;
   // hnv_selftest_team_timeout: of the one-launch calls' barriers
   uint64_t team_wait_ns = hnv::kTeamWaitNs;
   int32_t team_stop_at = 0;
@@ -669,6 +673,7 @@ int team_run(hnv_graph* g, TeamGraph t, int dtype, int d, float omega, int sweep
 // that, so later calls on any stream find them). Without memory for them
 // g->team_levels stays null, and the per-launch path is taken.
 void team_upload(hnv_graph* g, std::vector<TeamLevel>* host);
+void team_drop(hnv_graph* g);   // the descriptors of a hierarchy that goes
 inline bool team_ready(const hnv_graph* g) { return g->team_levels != nullptr; }
 int forced_panels();   // HNV_PANELS, or -1
 

@@ -485,17 +485,22 @@ void team_upload(hnv_graph* g, std::vector<TeamLevel>* host) {
     row0 += (int64_t)g->levels[l].n + g->levels[l].m;
   }
   const size_t bytes = sizeof(TeamLevel) * host->size();
-  TeamLevel* t = nullptr;
-  if (dev_alloc((void**)&t, bytes, s) != HNV_OK) {
+  team_drop(g);
+  TeamLevel* t = g->team_buf;
+  if (host->size() > (size_t)kTeamLevels && dev_alloc((void**)&t, bytes, s) != HNV_OK) {
     clear_error_detail();
     return;
   }
+  g->team_levels = t;
   if (cudaMemcpyAsync(t, host->data(), bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) {
     cudaGetLastError();
-    dev_free(t, s);
-    return;
+    team_drop(g);
   }
-  g->team_levels = t;
+}
+
+void team_drop(hnv_graph* g) {
+  if (g->team_levels != g->team_buf) dev_free(g->team_levels, g->stream);
+  g->team_levels = nullptr;
 }
 
 namespace {

@@ -539,3 +539,32 @@ def test_batch_takes_the_path_estimated_faster(H, d, teams):
         assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
     for G in Gs:
         G.close()
+
+
+def test_hierarchies_of_many_levels(H):
+    """Coarsening one graph again and again, to fewer and to more levels than
+    a graph has room to describe from the start (40)."""
+    import torch
+    # hyperedges along a path, taken in order of their weight: a step merges
+    # three nodes of 300
+    n = 300
+    nodes = (np.arange(n - 2)[:, None] + np.arange(3)[None, :]).astype(np.int32).ravel()
+    prio = np.tile(np.arange(n - 2, dtype=np.uint64), (70, 1))
+    with H.Graph(n, n - 2, 3 * np.arange(n - 1, dtype=np.int64), nodes) as G:
+        seen = set()
+        for most in (3, 64, 64, 5, 70):
+            L = G.coarsen(policy=H.ASSIGN_EXPLICIT, explicit_prio=prio, min_nodes=2,
+                          max_levels=most)
+            seen.add(L > 40)
+            top = G.level_info(L - 1)
+            zc = torch.randn((top[0] + top[1], 16), device="cuda")
+            zv = torch.empty((n, 16), device="cuda")
+            ze = torch.empty((n - 2, 16), device="cuda")
+
+            def vcycle():
+                G.vcycle(zc, zv, ze, 0.5, 2)
+                return zv.clone(), ze.clone()
+            a, b, one, many = _both(H, vcycle)
+            assert one == 1 and many > one
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+        assert seen == {False, True}
