@@ -33,7 +33,16 @@
  *    half-sweep's row classes run, forked from and joined back into the
  *    caller's stream). Calls on the same graph or batch must therefore not
  *    run concurrently from several host threads, or on streams whose work
- *    overlaps; different graphs are independent.
+ *    overlaps; different graphs are independent. One exception: two-phase
+ *    hnv_refine calls on a small level (below) whose rows all have at most 128
+ *    incidences use no shared scratch, and may be queued (by one host thread,
+ *    outside captures or within one) on streams whose work overlaps.
+ *  - Small levels (at most 1.8M incidences and 192 MB of gathered rows, less for
+ *    some row sizes) run all their sweeps, and small hierarchies whole V-cycles,
+ *    in one cooperative launch with bounded waits between its blocks; the
+ *    results are the same bits as those of a launch per row class. A wait that
+ *    gives up ends the launch and is reported as HNV_ERR_TIMEOUT, by
+ *    hnv_refine_until itself and by hnv_sync_status after the others.
  */
 #ifndef HNV_H_
 #define HNV_H_
@@ -222,7 +231,10 @@ int hnv_project(const hnv_graph* g, int fine_level, const void* zc_v, const void
  * that side's long rows are summed in pieces, one per range of neighbour
  * IDs (panels), and the pieces added in order: the first call for a new
  * row size builds that plan (allocating; HNV_PANELS=<k> in the environment
- * forces k panels).
+ * forces k panels). The graph's split-row scratch (and a hyperedge table for
+ * JACOBI) grows with the largest row size used; a call that needs no more
+ * allocates nothing. In a stream capture, a call that needs more allocates it
+ * inside the capture, for its replays.
  *   z_v [n_l x d], z_e [m_l x d] : device, read and written
  *   omega in [0, 1]; sweeps >= 0
  * ------------------------------------------------------------------------- */
@@ -236,8 +248,11 @@ int hnv_refine(hnv_graph* g, int level, void* z_v, void* z_e, hnv_dtype dt, int 
  * is the largest |change| of any coordinate of any node or hyperedge row
  * (as stored). Runs at most max_sweeps sweeps; eps < 0 never stops early.
  *   sweeps_done [out] : sweeps run; last_delta [out] : the last difference
- * Synchronises the stream after every sweep (to read the difference) and
- * allocates two row buffers of the level for the previous iterate.
+ * A small level runs up to 512 sweeps a launch, the test within it, and
+ * synchronises the stream after each launch; a larger one synchronises after
+ * every sweep (to read the difference) and allocates two row buffers of the
+ * level for the previous iterate. HNV_ERR_TIMEOUT if a bounded wait gave up in
+ * any sweep (the rows are then not valid, and the outputs not written).
  * ------------------------------------------------------------------------- */
 int hnv_refine_until(hnv_graph* g, int level, void* z_v, void* z_e, hnv_dtype dt, int d,
                      float omega, int max_sweeps, float eps, hnv_sweep mode,
@@ -338,13 +353,16 @@ int hnv_vcycle_backward(hnv_graph* g, const float* checkpoints, const float* g_v
  * Batched V-cycle: many independent hypergraphs refined together
  *
  * Each graph is built and coarsened as usual (its hierarchy does not change).
- * The batch lines the graphs up by level index: at step s (deepest level
- * first) every graph whose coarsest level is >= s projects onto its level s
- * (or starts from its input rows at its coarsest level) and runs the
- * two-phase sweeps of Algorithm 2 there. Per half-sweep, one launch per row
- * class (or one persistent launch) covers the rows of all graphs (a work
- * list with a graph index per item); the whole V-cycle can be captured once
- * into a CUDA graph and replayed. Results equal hnv_vcycle on each graph
+ * Graphs all of whose levels are small may be dealt over teams of thread
+ * blocks (with HNV_BATCH_KERNEL_PER_CLASS and at most 512 sweeps, where that is
+ * estimated to be faster): one launch, each team its graphs' whole V-cycles one
+ * after the other. The batch lines the other graphs up by level index: at step
+ * s (deepest level first) every such graph whose coarsest level is >= s
+ * projects onto its level s (or starts from its input rows at its coarsest
+ * level) and runs the two-phase sweeps of Algorithm 2 there. Per half-sweep,
+ * one launch per row class (or one persistent launch) covers the rows of all of
+ * them (a work list with a graph index per item); the whole V-cycle can be
+ * captured once into a CUDA graph and replayed. Results equal hnv_vcycle on each graph
  * (same per-row sums). The persistent launches use a small array of task
  * counters owned by the batch (one per half-sweep), cleared at the start of
  * every V-cycle; V-cycles of one batch must not overlap on the GPU.
@@ -353,10 +371,11 @@ typedef struct hnv_batch hnv_batch;
 
 /* Half-sweep kernels of the batched V-cycle. PER_CLASS: one launch per row
  * class (rows of 1..a_max, a_max+1..b_max and longer rows with chunks), the
- * classes on concurrent streams. PERSISTENT: one launch per half-sweep over
- * every item of every class and graph; resident warps take fixed-size tasks
- * from a counter in device memory, the longest items first. Both are followed
- * by the split-row reduction and give the same bits. */
+ * classes on concurrent streams (but for graphs that go to teams, above).
+ * PERSISTENT: one launch per half-sweep over every item of every class and
+ * graph; resident warps take fixed-size tasks from a counter in device memory,
+ * the longest items first. Both are followed by the split-row reduction and
+ * give the same bits. */
 enum { HNV_BATCH_KERNEL_PER_CLASS = 0, HNV_BATCH_KERNEL_PERSISTENT = 1 };
 
 /* Row-length classes, lanes per row and half-sweep kernel chosen by
@@ -475,8 +494,9 @@ const char* hnv_last_error_detail(void);
 
 /* Replaces the device allocator (NULL, NULL restores the library's pool:
  * cudaMallocFromPoolAsync / cudaFreeAsync). alloc returns NULL on failure,
- * which the library reports as HNV_ERR_OOM. Not thread-safe with respect to
- * calls in flight. */
+ * which the library reports as HNV_ERR_OOM. Small temporaries of a call are cut
+ * from blocks of 512 KB; a call whose block is refused asks for them one by one.
+ * Not thread-safe with respect to calls in flight. */
 typedef void* (*hnv_alloc_fn)(size_t bytes, hnv_stream_t stream, void* ctx);
 typedef void (*hnv_free_fn)(void* ptr, hnv_stream_t stream, void* ctx);
 int hnv_set_allocator(hnv_alloc_fn alloc_fn, hnv_free_fn free_fn, void* ctx);
