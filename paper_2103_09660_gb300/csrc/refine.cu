@@ -259,9 +259,11 @@ int launch_items(const HalfSweep& h, const int4* items, int32_t n_items, bool ln
   const int64_t warps = ((int64_t)n_items + R - 1) / R;
   const int64_t blocks64 = (warps + WPB - 1) / WPB;
   const unsigned blocks = (unsigned)(blocks64 > 0x7fffffff ? 0x7fffffff : blocks64);
+  // (unweighted float32 rows of fewer than 32 lanes: both are the same code)
+  constexpr bool DIFFERS = G == 32 || sizeof(T) == 2;
   auto kern = h.inc_w ? (lng ? gather_kernel<T, G, VPL, true, true>
                              : gather_kernel<T, G, VPL, true, false>)
-                      : (lng ? gather_kernel<T, G, VPL, false, true>
+                      : (lng ? gather_kernel<T, G, VPL, false, DIFFERS>
                              : gather_kernel<T, G, VPL, false, false>);
   return launch(h.inc_w ? "gather_w" : "gather", kern, blocks, kGatherThreads, 0, s, items,
                 n_items, h.idx, h.inc_w, h.inv_norm, (const uint4*)src, (const uint4*)self_in,
