@@ -30,9 +30,9 @@
 // batch the estimates below.
 //
 // Measured (GB300, same bits): the V-cycle of a 2,000-node graph (d = 32, 7
-// levels x 10 sweeps) 2.25 -> 0.74 ms, of a 41K-node graph (d = 100, 33 levels
-// x 20 sweeps) 31.2 -> 13.2 ms, of a batch of 64 graphs of 1K-100K nodes
-// (d = 64) 91 -> 76 ms. What is left of a sweep of the 41K-node graph (20 us)
+// levels x 10 sweeps) 2.25 -> 0.70 ms, of a 41K-node graph (d = 100, 33 levels
+// x 20 sweeps) 31.2 -> 13.0 ms, of a batch of 64 graphs of 1K-100K nodes
+// (d = 64) 91 -> 71 ms. What is left of a sweep of the 41K-node graph (20 us)
 // is 3-6 us of dependent loads a half-sweep, 1.4 us a barrier (2 or 3 a
 // sweep) and 4 us for a hub row's reduction. On larger levels the per-launch
 // kernels, with twice the warps per SM, are faster (a level of 150K nodes, 2.1M
@@ -72,7 +72,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 // limited to g->wait_ns; the barrier at target *stop waits for one arrival
 // more than comes (TeamGraph::stop_at). (A timeout is recorded here rather than
 // where the kernel's body returns: with that body in a function of its own the
-// batch of 64 graphs took 76 ms instead of 70, with no more spills.)
+// batch of 64 graphs took 76.2 ms instead of 72.2, with no more spills.)
 struct TeamBarrier {
   uint32_t* counter;
   uint32_t blocks;
