@@ -479,7 +479,8 @@ int hnv_selftest_team_timeout(hnv_graph* g, int32_t barrier, uint32_t limit_us);
  * (its blocks would not all be resident): with refuse != 0 the library acts as
  * if every such launch of the graph, or of a batch that holds it, were refused,
  * and takes a launch per half-sweep; the results are the same bits. 0 restores
- * the normal launches. Errors: HNV_ERR_INVALID_ARG. */
+ * the normal launches (a batch that met a refusal keeps to its step lists).
+ * Errors: HNV_ERR_INVALID_ARG. */
 int hnv_selftest_team_refuse(hnv_graph* g, int refuse);
 
 /* Releases the hierarchy (stream-ordered on the graph's stream). NULL is a no-op. */
